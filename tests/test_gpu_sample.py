@@ -65,3 +65,23 @@ def test_shots_from_simulated_distribution_follow_it(slos):
         f = counts[b].double().cpu().numpy() / shots
         sd = np.sqrt(p * (1 - p) / shots)
         assert np.all(np.abs(f - p) <= 5 * sd + 2e-6)
+
+
+@pytest.mark.parametrize("m,s,offset,B,shots", [(12, [1, 0] * 6, 0, 3, 33), (12, [1, 0] * 6, 1, 3, 1), (8, [1, 0] * 4, 2, 40, 31),
+                                                (16, [1, 0] * 7 + [0, 0], 3, 1, 500), (2, [8, 0], 0, 2, 7)])
+def test_samples_off_a_16_byte_boundary_and_ragged_shots(slos, m, s, offset, B, shots):
+    """Rows that allow 16-byte reads and rows that do not (offset base, row
+    lengths not a multiple of 4), shot counts around the 32 of a block."""
+    plan = slos.Plan(m, s)
+    K = plan.n_outputs
+    p = workloads.random_distributions(B, K, seed=70 + m, zero_fraction=0.5)
+    u = workloads.uniforms(B, shots, seed=71 + m)
+    buf = torch.zeros(B * K + offset, dtype=torch.float32, device="cuda")
+    pt = buf[offset:].view(B, K)
+    pt.copy_(torch.tensor(p))
+    samples, counts = plan.sample(pt, torch.tensor(u, device="cuda"), counts=True)
+    assert torch.equal(samples, plan.sample(pt, torch.tensor(u, device="cuda")))
+    for b in range(B):
+        ref = oracle.sample_outcomes(p[b], u[b])
+        assert np.array_equal(samples[b].cpu().numpy(), ref)
+        assert np.array_equal(counts[b].cpu().numpy(), np.bincount(ref, minlength=K))
