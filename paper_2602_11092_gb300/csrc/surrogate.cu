@@ -183,8 +183,99 @@ __global__ void transpose_kernel(const __nv_bfloat16 *in, int R, int C, __nv_bfl
     }
 }
 
-// One block per row: q = softmax(z); loss_row = sum p (log p - log q);
-// dz = (q - p) * scale (bf16); optionally q out (float).
+// Block-wide maximum / sum of one float per thread, in a fixed order; every
+// thread gets it.  red: one float per warp.
+template <bool MAX>
+__device__ __forceinline__ float block_reduce(float v, float *red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float w = __shfl_xor_sync(0xffffffffu, v, o);
+        v = MAX ? fmaxf(v, w) : v + w;
+    }
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    v = lane < warps ? red[lane] : (MAX ? -INFINITY : 0.f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float w = __shfl_xor_sync(0xffffffffu, v, o);
+        v = MAX ? fmaxf(v, w) : v + w;
+    }
+    __syncthreads();
+    return v;
+}
+
+// Rows of up to 4 * kSoftmaxVecs * 1024 logits whose length and buffers allow
+// 16-byte accesses: one block per row, the whole row in registers, so each
+// logit is read from memory once.  Memory-bound: 8 bytes per output (12 with a
+// target).  q = e^{z - max} / sum for the forward pass; a training step keeps
+// the log-probability z - lse for its loss.  Measured on 16384 rows of 12,376
+// (1.62 GB): 672 us while the row was read from L2 in three passes of 4-byte
+// loads, 270 us now.  Two blocks of up to 1024 threads per SM keep both
+// rows' loads in flight; a row per warp would leave too few.
+constexpr int kSoftmaxVecs = 4;
+template <bool TRAIN>
+__global__ void __launch_bounds__(1024, 2) softmax_row_kernel(const float *z, const float *p, int K, float scale,
+                                                              __nv_bfloat16 *dz, float *loss_rows, float *q_out) {
+    __shared__ float red[32];
+    const int64_t r = blockIdx.x;
+    const int K4 = K / 4;
+    const float4 *zr = reinterpret_cast<const float4 *>(z + r * K);
+    float4 v[kSoftmaxVecs];
+    float mx = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < kSoftmaxVecs; ++q) {
+        const int i = threadIdx.x + q * blockDim.x;
+        v[q] = i < K4 ? __ldcs(zr + i) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    }
+#pragma unroll
+    for (int q = 0; q < kSoftmaxVecs; ++q) mx = fmaxf(mx, fmaxf(fmaxf(v[q].x, v[q].y), fmaxf(v[q].z, v[q].w)));
+    mx = block_reduce<true>(mx, red);
+    float se = 0.f;
+#pragma unroll
+    for (int q = 0; q < kSoftmaxVecs; ++q) {
+        if (threadIdx.x + q * blockDim.x < K4) {
+            const float4 e = make_float4(expf(v[q].x - mx), expf(v[q].y - mx), expf(v[q].z - mx), expf(v[q].w - mx));
+            se += (e.x + e.y) + (e.z + e.w);
+            if (!TRAIN) v[q] = e;
+        }
+    }
+    se = block_reduce<false>(se, red);
+    if (!TRAIN) {
+        const float inv = 1.f / se;
+        float4 *qr = reinterpret_cast<float4 *>(q_out + r * K);
+#pragma unroll
+        for (int q = 0; q < kSoftmaxVecs; ++q) {
+            const int i = threadIdx.x + q * blockDim.x;
+            if (i < K4) __stcs(qr + i, make_float4(v[q].x * inv, v[q].y * inv, v[q].z * inv, v[q].w * inv));
+        }
+        return;
+    }
+    const float lse = mx + logf(se);
+    const float4 *pr = reinterpret_cast<const float4 *>(p + r * K);
+    float kl = 0.f;
+#pragma unroll
+    for (int q = 0; q < kSoftmaxVecs; ++q) {
+        const int i = threadIdx.x + q * blockDim.x;
+        if (i >= K4) continue;
+        const float4 pv = __ldcs(pr + i);
+        const float zz[4] = {v[q].x, v[q].y, v[q].z, v[q].w}, pp[4] = {pv.x, pv.y, pv.z, pv.w};
+        __align__(8) __nv_bfloat16 d[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float lq = zz[c] - lse;
+            if (pp[c] > 0.f) kl += pp[c] * (logf(pp[c]) - lq);
+            d[c] = __float2bfloat16((expf(lq) - pp[c]) * scale);
+        }
+        *reinterpret_cast<uint2 *>(dz + r * K + 4 * i) = *reinterpret_cast<const uint2 *>(d);
+    }
+    kl = block_reduce<false>(kl, red);
+    if (threadIdx.x == 0) loss_rows[r] = kl;
+}
+
+// Any row length and alignment, one block per row: q = softmax(z);
+// loss_row = sum p (log p - log q); dz = (q - p) * scale (bf16); optionally
+// q out (float).
 __global__ void softmax_kl_kernel(const float *z, const float *p, int K, float scale, __nv_bfloat16 *dz,
                                   float *loss_rows, float *q_out) {
     const int64_t r = blockIdx.x;
@@ -232,6 +323,22 @@ __global__ void softmax_kl_kernel(const float *z, const float *p, int K, float s
         float v = 0.f;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w];
         if (loss_rows) loss_rows[r] = v;
+    }
+}
+
+// Softmax of B rows of K logits: with a target p, dz and the row losses (a
+// training step), otherwise q_out.
+void launch_softmax(const float *z, const float *p, int B, int K, float scale, __nv_bfloat16 *dz, float *loss_rows,
+                    float *q_out, cudaStream_t s) {
+    const int K4 = K / 4;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(z) | reinterpret_cast<uintptr_t>(p) |
+                         reinterpret_cast<uintptr_t>(q_out) | reinterpret_cast<uintptr_t>(dz);
+    if (K % 4 == 0 && at % 16 == 0 && K4 <= kSoftmaxVecs * 1024) {
+        const int threads = std::max(32, ((K4 + kSoftmaxVecs - 1) / kSoftmaxVecs + 31) / 32 * 32);
+        if (p) softmax_row_kernel<true><<<B, threads, 0, s>>>(z, p, K, scale, dz, loss_rows, q_out);
+        else softmax_row_kernel<false><<<B, threads, 0, s>>>(z, p, K, scale, dz, loss_rows, q_out);
+    } else {
+        softmax_kl_kernel<<<B, 256, 0, s>>>(z, p, K, scale, dz, loss_rows, q_out);
     }
 }
 
@@ -571,7 +678,7 @@ slos_status_t surr_forward(surr_model_t M, const float *phases, int B, float *pr
     slos_status_t st = forward_impl(M, phases, B, s);
     if (st) return st;
     ProfScope ps("surr_softmax", 8.0 * B * M->K, s);
-    softmax_kl_kernel<<<B, 256, 0, s>>>(M->logits, nullptr, M->K, 0.f, nullptr, nullptr, probs);
+    launch_softmax(M->logits, nullptr, B, M->K, 0.f, nullptr, nullptr, probs, s);
     return launch_check("softmax");
 }
 
@@ -583,8 +690,7 @@ slos_status_t surr_train_step(surr_model_t M, const float *phases, const float *
     if (st) return st;
     {
         ProfScope ps("surr_softmax", 12.0 * B * M->K, s);
-        softmax_kl_kernel<<<B, 256, 0, s>>>(M->logits, target, M->K, 1.0f / B, M->dlog, loss_rows ? loss_rows : M->loss_rows,
-                                            nullptr);
+        launch_softmax(M->logits, target, B, M->K, 1.0f / B, M->dlog, loss_rows ? loss_rows : M->loss_rows, nullptr, s);
     }
     if ((st = launch_check("softmax_kl"))) return st;
     // backward through the layers: g = dL/d(pre-activation of layer l), [B][fan_out]

@@ -184,3 +184,32 @@ def test_training_checkpoint_resume_is_bitwise(tmp_path):
     c = Surrogate(n_phases=n_ph, hidden=128, n_hidden_layers=2, n_outputs=K, max_batch=Bn, seed=1)
     with pytest.raises(Exception):
         c.load(path)
+
+
+@pytest.mark.parametrize("K,offset", [(8, 0), (4104, 0), (12376, 0), (16384, 0), (16392, 0), (12376, 1)])
+def test_softmax_row_lengths_and_alignment(K, offset):
+    """Rows kept whole in registers (up to 16384 logits, the last partly
+    filled vectors) and the general kernel (longer rows, an output off a
+    16-byte boundary): with zero output weights the logits are the bias, so
+    q and KL(p || q) are known."""
+    from paper_2602_11092_gb300 import surrogate as S
+    rng = np.random.default_rng(K + offset)
+    Bn = 8
+    model = S.Surrogate(n_phases=4, hidden=8, n_hidden_layers=1, n_outputs=K, max_batch=Bn, seed=2)
+    bias = rng.uniform(-8.0, 8.0, K).astype(np.float32)
+    model.set_param(1, np.zeros((K, 8), dtype=np.float32), bias)
+    ref = np.exp(bias.astype(np.float64) - bias.max())
+    ref /= ref.sum()
+    buf = torch.empty(Bn * K + offset, device="cuda")
+    q = model.forward(torch.rand(Bn, 4, device="cuda"), out=buf[offset:].view(Bn, K)).double().cpu().numpy()
+    # |z - max| <= 16: half an ulp of it (1e-6) plus the exponential's and the sum's rounding
+    assert np.abs(q / ref[None, :] - 1).max() <= 4e-6
+    p = rng.dirichlet(np.ones(K), size=Bn).astype(np.float32)
+    p[0] = 0.0
+    p[0, K // 3] = 1.0
+    losses = torch.zeros(Bn, device="cuda")
+    model.train_step(torch.rand(Bn, 4, device="cuda"), torch.tensor(p, device="cuda"), 0.0, losses)
+    S.sync_status()
+    pd = p.astype(np.float64)
+    kl = (pd * (np.log(np.where(pd > 0, pd, 1.0)) - np.log(ref)[None, :])).sum(axis=1)
+    assert np.abs(losses.cpu().numpy() - kl).max() <= 2e-5
