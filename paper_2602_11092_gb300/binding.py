@@ -124,15 +124,23 @@ def _check(status: int):
 
 
 def _ptr(t: torch.Tensor | None):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_cuda_ready = False
 
 
 def _stream(stream=None):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    """The stream's handle; by default the current device's current stream
+    (read as a handle: building a torch.cuda.Stream object takes 3 us, more
+    than a launch)."""
+    if stream is not None:
+        return stream.cuda_stream
+    global _cuda_ready
+    if not _cuda_ready:
+        torch.cuda.init()
+        _cuda_ready = True
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _need(t: torch.Tensor, dtype, name: str):
@@ -187,9 +195,10 @@ def mesh_unitary_backward(m: int, theta, data, batch: int, dU: torch.Tensor, dat
     dtheta = torch.empty((P,) if shared else (batch, P), dtype=torch.float32, device=dU.device)
     ddata = torch.empty((batch, n_data), dtype=torch.float32, device=dU.device) if n_data else None
     dw = torch.empty((batch, n_data), dtype=torch.float32, device=dU.device) if (n_data and need_dw) else None
-    nbytes = ctypes.c_size_t()
+    ws, nbytes = None, ctypes.c_size_t()
     _check(lib.mesh_unitary_backward_workspace(ctypes.byref(desc), batch, ts, ctypes.byref(nbytes)))
-    ws = torch.empty(max(1, nbytes.value), dtype=torch.uint8, device=dU.device)
+    if nbytes.value:
+        ws = torch.empty(nbytes.value, dtype=torch.uint8, device=dU.device)
     ds = 0 if data is None else data.shape[-1]
     if w is None:
         _check(lib.mesh_unitary_backward(ctypes.byref(desc), _ptr(theta), ts, _ptr(data), ds, batch, _ptr(dU),
@@ -248,15 +257,23 @@ class Plan:
         K, F, st = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int()
         _check(lib.slos_plan_query(h, ctypes.byref(K), ctypes.byref(F), ctypes.byref(st)))
         self.n_outputs, self.fock_dim, self.checkpoint_stride = K.value, F.value, st.value
+        self._ws_bytes = {}  # (batch, training) -> workspace bytes, a few sizes
 
     @property
     def handle(self):
         return self._h
 
     def workspace_bytes(self, batch: int, training: bool) -> int:
-        b = ctypes.c_size_t()
-        _check(load().slos_workspace_bytes(self._h, batch, 1 if training else 0, ctypes.byref(b)))
-        return b.value
+        key = (batch, bool(training))
+        size = self._ws_bytes.get(key)
+        if size is None:
+            b = ctypes.c_size_t()
+            _check(load().slos_workspace_bytes(self._h, batch, 1 if training else 0, ctypes.byref(b)))
+            size = b.value
+            if len(self._ws_bytes) >= 16:
+                self._ws_bytes.clear()
+            self._ws_bytes[key] = size
+        return size
 
     def workspace(self, batch: int, training: bool, device="cuda") -> torch.Tensor:
         return torch.empty(max(1, self.workspace_bytes(batch, training)), dtype=torch.uint8, device=device)

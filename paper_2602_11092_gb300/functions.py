@@ -3,6 +3,8 @@ simulation; Sec. II-B: the quantum layer as a composable module).
 
 MeshFn  : (theta, data) -> U           via mesh_unitary / mesh_unitary_backward
 SlosFn  : U -> probabilities or amps   via slos_forward / slos_backward
+LayerFn : (theta, x, w) -> layer output: the calls of the above, the
+          renormalisation and the expectations as one autograd node
 QuantumLayer: theta (trainable) and data phases x*w (formed in the mesh kernel)
 -> output distribution.
 
@@ -22,17 +24,13 @@ class MeshFn(torch.autograd.Function):
         data = data.contiguous() if data is not None else None
         w = w.contiguous() if w is not None else None
         U = B.mesh_unitary(m, theta, data, batch, data_col, w=w)
-        empty = torch.empty(0, device=theta.device)
-        ctx.save_for_backward(theta, data if data is not None else empty, w if w is not None else empty)
+        ctx.save_for_backward(theta, data, w)
         ctx.m, ctx.batch, ctx.data_col = m, batch, data_col
-        ctx.has_data, ctx.has_w = data is not None, w is not None
         return U
 
     @staticmethod
     def backward(ctx, dU):
         theta, data, w = ctx.saved_tensors
-        data = data if ctx.has_data else None
-        w = w if ctx.has_w else None
         need_dw = w is not None and ctx.needs_input_grad[5]
         res = B.mesh_unitary_backward(ctx.m, theta, data, ctx.batch, dU.contiguous(), ctx.data_col, w=w,
                                       need_dw=need_dw)
@@ -40,12 +38,28 @@ class MeshFn(torch.autograd.Function):
         return res[0], res[1], None, None, None, dw
 
 
+def _gradient_row(dout):
+    """dout as the library takes it: [K] when every instance has the same row (stride 0), else [B, K]."""
+    if dout.dim() == 2 and dout.stride(0) == 0 and dout.stride(1) == 1:
+        return dout[0]
+    return dout.contiguous()
+
+
+_RELEASED = ("{}: a second backward through the same forward is not supported (its activations were released by the "
+             "first backward); run the forward again")
+
+
 class SlosFn(torch.autograd.Function):
+    """save: keep the activations for backward (without them the plan's
+    inference kernels run, and the node has no backward)."""
+
     @staticmethod
-    def forward(ctx, U, plan: B.Plan, output: int):
+    def forward(ctx, U, plan: B.Plan, output: int, save: bool = True):
         U = U.contiguous()
-        ws = plan.workspace(U.shape[0], training=True, device=U.device)
-        out = plan.forward(U, output, save_for_backward=True, workspace=ws)
+        ws = plan.workspace(U.shape[0], training=save, device=U.device)
+        out = plan.forward(U, output, save_for_backward=save, workspace=ws)
+        if not save:
+            return out
         ctx.save_for_backward(U)
         ctx.plan, ctx.ws, ctx.output = plan, ws, output
         return out
@@ -53,16 +67,11 @@ class SlosFn(torch.autograd.Function):
     @staticmethod
     def backward(ctx, dout):
         (U,) = ctx.saved_tensors
-        if dout.dim() == 2 and dout.stride(0) == 0 and dout.stride(1) == 1:
-            d = dout[0]  # the same gradient row for every instance (stride 0)
-        else:
-            d = dout.contiguous()
         if ctx.ws is None:
-            raise RuntimeError("SlosFn: a second backward through the same forward is not supported (its activations "
-                               "were released by the first backward); run the forward again")
-        dU = ctx.plan.backward(U, d, ctx.ws, ctx.output)
+            raise RuntimeError(_RELEASED.format("SlosFn"))
+        dU = ctx.plan.backward(U, _gradient_row(dout), ctx.ws, ctx.output)
         ctx.ws = None
-        return dU, None, None
+        return dU, None, None, None
 
 
 class ExpectationFn(torch.autograd.Function):
@@ -94,13 +103,56 @@ class RenormaliseFn(torch.autograd.Function):
         return ctx.plan.renormalise_backward(q, Z, dq.contiguous()), None
 
 
+class LayerFn(torch.autograd.Function):
+    """The whole of QuantumLayer's forward as one autograd node: mesh, SLOS
+    recursion, renormalisation and expectations (whichever the layer has), and
+    their backwards in reverse.  One node instead of up to four: each costs a
+    Python call from the autograd engine's thread, about 40 us of a step.
+    save: as in SlosFn."""
+
+    @staticmethod
+    def forward(ctx, theta, x, w, plan: B.Plan, output: int, renormalise: bool, expectations: bool, save: bool):
+        theta, x, w = theta.contiguous(), x.contiguous(), w.contiguous()
+        batch = x.shape[0]
+        U = B.mesh_unitary(plan.m, theta, x, batch, w=w)
+        ws = plan.workspace(batch, training=save, device=U.device)
+        y = plan.forward(U, output, save_for_backward=save, workspace=ws)
+        q = Z = None
+        if renormalise:
+            y, Z = plan.renormalise(y)
+            q = y
+        if expectations:
+            y = plan.expectations(y)
+        if save:
+            ctx.save_for_backward(theta, x, w, U, q, Z)
+            ctx.plan, ctx.ws, ctx.output, ctx.expectations = plan, ws, output, expectations
+        return y
+
+    @staticmethod
+    def backward(ctx, dout):
+        theta, x, w, U, q, Z = ctx.saved_tensors
+        plan = ctx.plan
+        if ctx.ws is None:
+            raise RuntimeError(_RELEASED.format("LayerFn"))
+        if ctx.expectations:
+            dout = plan.expectations_backward(dout.contiguous())
+        if q is not None:
+            dout = plan.renormalise_backward(q, Z, dout.contiguous())
+        dU = plan.backward(U, _gradient_row(dout), ctx.ws, ctx.output)
+        ctx.ws = None
+        need_dw = ctx.needs_input_grad[2]
+        res = B.mesh_unitary_backward(plan.m, theta, x, x.shape[0], dU, w=w, need_dw=need_dw)
+        dw = B.mesh_sum_rows(res[2]) if need_dw else None
+        return res[0], res[1], dw, None, None, None, None, None
+
+
 def mesh_unitary(theta, data, m: int, batch: int, data_col: int | None = None, w=None):
     """U(theta, data) with data phases data (or data * w, formed in the kernel)."""
     return MeshFn.apply(theta, data, m, batch, m // 2 if data_col is None else data_col, w)
 
 
 def slos(U, plan: B.Plan, output: int = B.PROBS):
-    return SlosFn.apply(U, plan, output)
+    return SlosFn.apply(U, plan, output, torch.is_grad_enabled() and U.requires_grad)
 
 
 class QuantumLayer(torch.nn.Module):
@@ -136,13 +188,12 @@ class QuantumLayer(torch.nn.Module):
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         x = x.to(torch.float32).contiguous()
-        U = mesh_unitary(self.theta, x, self.m, x.shape[0], w=self.w[: x.shape[-1]].contiguous())
-        y = slos(U, self.plan, self.output)
-        if self.renormalise:
-            y = RenormaliseFn.apply(y, self.plan)
-        if self.measurement == "expectations":
-            y = ExpectationFn.apply(y, self.plan)
-        return y
+        theta, w = self.theta, self.w
+        if w.shape[0] != x.shape[-1]:
+            w = w[: x.shape[-1]]
+        save = torch.is_grad_enabled() and (theta.requires_grad or x.requires_grad or w.requires_grad)
+        return LayerFn.apply(theta, x, w, self.plan, self.output, self.renormalise,
+                             self.measurement == "expectations", save)
 
 
 class FidelityKernel(torch.nn.Module):

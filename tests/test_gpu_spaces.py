@@ -239,3 +239,47 @@ def test_layer_unbunched_renormalised_expectations_gradient(slos):
         assert np.linalg.norm(gx - g_d) / np.linalg.norm(g_d) <= G_TOL
     g = layer.theta.grad.cpu().double().numpy()
     assert np.linalg.norm(g - g_th) / np.linalg.norm(g_th) <= G_TOL
+
+
+@pytest.mark.parametrize("det,space,renorm,measure,features", [
+    (0, 0, False, "probs", 8), (1, 0, False, "expectations", 5), (0, 1, True, "expectations", 8), (0, 1, True, "probs", 3),
+    (0, 0, False, "amps", 8)])
+def test_layer_node_equals_its_parts(slos, det, space, renorm, measure, features):
+    """QuantumLayer's single autograd node against the same calls as separate
+    nodes: outputs and gradients (trainable phases, features, encoding
+    weights) bit for bit; without gradients the same outputs within rounding."""
+    from paper_2602_11092_gb300 import functions as F
+    m, s, B = 8, [1, 0, 1, 0, 1, 0, 0, 0], 37
+    gen = torch.Generator().manual_seed(7)
+    layer = F.QuantumLayer(m, s, det, space=space, renormalise=renorm, measurement=measure,
+                           theta=torch.rand(m * (m - 1), generator=gen), w=torch.rand(m, generator=gen))
+    layer.w.requires_grad_(True)
+    x = torch.randn(B, features, generator=gen).cuda().requires_grad_(True)
+    y = layer(x)
+    U = F.mesh_unitary(layer.theta, x, m, B, w=layer.w[:features].contiguous())
+    z = F.slos(U, layer.plan, layer.output)
+    if renorm:
+        z = F.RenormaliseFn.apply(z, layer.plan)
+    if measure == "expectations":
+        z = F.ExpectationFn.apply(z, layer.plan)
+    assert torch.equal(y, z)
+    g = torch.randn(y.shape, generator=gen).to(y.dtype).cuda()
+    for grads in (g, g[:1].expand(B, -1)):
+        inputs = (layer.theta, x, layer.w)
+        a = torch.autograd.grad(layer(x), inputs, grads)
+        U = F.mesh_unitary(layer.theta, x, m, B, w=layer.w[:features].contiguous())
+        z = F.slos(U, layer.plan, layer.output)
+        z = F.RenormaliseFn.apply(z, layer.plan) if renorm else z
+        z = F.ExpectationFn.apply(z, layer.plan) if measure == "expectations" else z
+        b = torch.autograd.grad(z, inputs, grads)
+        assert all(torch.equal(p, q) for p, q in zip(a, b))
+    with torch.no_grad():
+        v = layer(x)
+    assert not v.requires_grad and (v - y.detach()).abs().max() <= 1e-6
+    assert not F.slos(U.detach(), layer.plan, layer.output).requires_grad
+    again = layer(x)
+    torch.autograd.grad(again, x, g, retain_graph=True)
+    with pytest.raises(RuntimeError, match="second backward"):
+        torch.autograd.grad(again, x, g)
+    with torch.no_grad(), torch.autograd.forward_ad.dual_level(), pytest.raises(Exception):
+        layer(torch.autograd.forward_ad.make_dual(x.detach(), torch.ones_like(x)))  # no forward-mode rule: refused
