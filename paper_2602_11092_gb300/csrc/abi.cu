@@ -486,13 +486,14 @@ static slos_status_t build_tables_unbunched(slos_plan_s *p) {
     }
     // final layer: prod t! = 1, so every weight is 1 / prod s!
     std::vector<float> w(p->F[n], p->inv_sfact);
-    std::vector<uint8_t> occ((size_t)p->K * m, 0);
+    const int mp = occ_row(m);
+    std::vector<uint8_t> occ((size_t)p->K * mp, 0);
     {
         std::vector<int> S(n);
         for (int q = 0; q < n; ++q) S[q] = q;
         int64_t c = 0;
         do {
-            for (int q : S) occ[(size_t)c * m + q] = 1;
+            for (int q : S) occ[(size_t)c * mp + q] = 1;
             ++c;
         } while (next_subset(S, m));
     }
@@ -575,12 +576,13 @@ static slos_status_t build_tables(slos_plan_s *p) {
         const int L = n + m - 1;
         std::vector<float> w(p->F[n]);
         std::vector<int32_t> pat(p->F[n]);
-        std::vector<uint8_t> occ((size_t)p->K * m, 0);
+        const int mp = occ_row(m);
+        std::vector<uint8_t> occ((size_t)p->K * mp, 0);
         uint64_t z = init_mask(n);
         for (int64_t c = 0; c < p->F[n]; ++c) {
             bars_of(z, m, L, bar.data(), t.data());
             if (p->det == SLOS_DETECT_PNR)
-                for (int j = 0; j < m; ++j) occ[(size_t)c * m + j] = (uint8_t)t[j];
+                for (int j = 0; j < m; ++j) occ[(size_t)c * mp + j] = (uint8_t)t[j];
             double f = 1.0;
             uint32_t supp = 0;
             for (int j = 0; j < m; ++j) {
@@ -594,7 +596,7 @@ static slos_status_t build_tables(slos_plan_s *p) {
                 if ((supp >> q) & 1u) r += binom_host(q, i++);
             pat[c] = p->pat_off[__builtin_popcount(supp)] + (int32_t)r;
             if (p->det == SLOS_DETECT_THRESHOLD)
-                for (int j = 0; j < m; ++j) occ[(size_t)pat[c] * m + j] = (uint8_t)((supp >> j) & 1u);
+                for (int j = 0; j < m; ++j) occ[(size_t)pat[c] * mp + j] = (uint8_t)((supp >> j) & 1u);
             z = next_comb_host(z);
         }
         if (plan_malloc(&p->tab.occ, occ.size()) != cudaSuccess) {

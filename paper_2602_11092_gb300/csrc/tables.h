@@ -56,10 +56,13 @@ struct PlanTables {
     int32_t *lseg = nullptr;         // [nseg + 1] forward work items: runs of whole patterns
     int nseg = 0;
     float *gfact = nullptr;          // [F_n]: sqrt(prod t_j!) of the final states (amplitude encoding)
-    uint8_t *occ = nullptr;          // [K][m]: occupation of mode j in output k (photon counts for PNR
-                                     // outputs, 0/1 for threshold outcomes)
+    uint8_t *occ = nullptr;          // [K][occ_row(m)]: occupation of mode j in output k (photon counts for
+                                     // PNR outputs, 0/1 for threshold outcomes), 0 past the last mode
     size_t bytes = 0;
 };
+
+// Bytes of a row of the occupation table: whole 32-bit words.
+constexpr int occ_row(int m) { return (m + 3) & ~3; }
 
 constexpr size_t kTableBudgetBytes = size_t(1) << 30;  // per plan
 constexpr int64_t kMaxTableParent = int64_t(1) << 26;

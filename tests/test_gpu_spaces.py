@@ -283,3 +283,41 @@ def test_layer_node_equals_its_parts(slos, det, space, renorm, measure, features
         torch.autograd.grad(again, x, g)
     with torch.no_grad(), torch.autograd.forward_ad.dual_level(), pytest.raises(Exception):
         layer(torch.autograd.forward_ad.make_dual(x.detach(), torch.ones_like(x)))  # no forward-mode rule: refused
+
+
+@pytest.mark.parametrize("m,n,det,B", [(3, 2, 0, 1), (3, 2, 0, 305), (8, 4, 0, 306), (16, 5, 0, 3), (16, 5, 0, 310),
+                                       (9, 4, 1, 307), (20, 3, 0, 5), (24, 3, 0, 308), (16, 6, 0, 2), (6, 12, 0, 4)])
+def test_reductions_over_split_rows(slos, m, n, det, B):
+    """Expectations and renormalisation of arbitrary rows against FP64 sums,
+    over the ways a row is cut: one CTA or a cluster per row, one or four
+    instances per CTA, a row within or beyond a CTA's registers, occupation
+    rows of 1 to 6 words."""
+    s = [1 if i < n else 0 for i in range(m)] if n <= m else [n - m + 1] + [1] * (m - 1)
+    plan = slos.Plan(m, s, det)
+    K = plan.n_outputs
+    rng = np.random.default_rng(m * 100 + n + B)
+    p = rng.exponential(size=(B, K)).astype(np.float32)
+    p64 = p.astype(np.float64)
+    if det:
+        occ = np.zeros((K, m))
+        for i, b_ in enumerate(oracle.threshold_patterns(m, n)):
+            occ[i, list(b_)] = 1.0
+    else:
+        occ = oracle.enumerate_fock(m, n).astype(np.float64)
+    pt = torch.tensor(p, device="cuda")
+    # a thread adds at most K / 256 / (CTAs) + a tree of positive terms, each addition half an ulp
+    E = plan.expectations(pt).double().cpu().numpy()
+    ref = p64 @ occ
+    assert np.abs(E / ref - 1).max() <= (K / 256 / 4 + 32) * 6e-8
+    dE = rng.standard_normal((B, m)).astype(np.float32)
+    dp = plan.expectations_backward(torch.tensor(dE, device="cuda")).double().cpu().numpy()
+    assert np.abs(dp - dE.astype(np.float64) @ occ.T).max() <= m * 6e-8 * n * np.abs(dE).max()
+    q, Z = plan.renormalise(pt)
+    # the sum to float, its reciprocal, the product: half an ulp each
+    assert np.abs(Z.double().cpu().numpy() / p64.sum(axis=1) - 1).max() <= 1e-7
+    assert np.abs(q.double().cpu().numpy() / (p64 / p64.sum(axis=1, keepdims=True)) - 1).max() <= 3e-7
+    dq = rng.standard_normal((B, K)).astype(np.float32)
+    got = plan.renormalise_backward(q, Z, torch.tensor(dq, device="cuda")).double().cpu().numpy()
+    q64, Z64 = q.double().cpu().numpy(), Z.double().cpu().numpy()[:, None]
+    dot = (dq * q64).sum(axis=1, keepdims=True)
+    assert np.abs(got - (dq - dot) / Z64).max() <= 4e-7 * ((np.abs(dq).max() + np.abs(dot).max()) / Z64.min())
