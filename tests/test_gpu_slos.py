@@ -414,6 +414,33 @@ def test_backward_threshold(slos, m, n, B):
         assert np.linalg.norm(dU[b] - ref) / np.linalg.norm(ref) <= G_TOL
 
 
+@pytest.mark.parametrize("m,n,kind,B", [(4, 2, "probs", 1), (8, 4, "probs", 65), (8, 4, "amps", 33), (16, 4, "threshold", 33),
+                                        (9, 6, "threshold", 31), (3, 8, "threshold", 2), (17, 3, "amps", 5)])
+def test_output_gradient_rows_shared_or_per_instance(slos, m, n, kind, B):
+    """A gradient row shared by the batch and the same row handed over per
+    instance give the same dU: the per-instance transposition (tiles of 64
+    states, ragged last tile, patterns spanning tiles) against the shared
+    seed; a dense gradient is linear in its rows."""
+    s = [1] * min(n, m) + [0] * max(0, m - n)
+    s[0] += max(0, n - m)
+    rng = np.random.default_rng(m * 31 + n)
+    U = c64(workloads.haar_unitaries(m, B, rng))
+    plan = slos.Plan(m, s, slos.THRESHOLD if kind == "threshold" else slos.PNR)
+    out = slos.AMPS if kind == "amps" else slos.PROBS
+    ws = plan.workspace(B, training=True)
+    plan.forward(U, out, save_for_backward=True, workspace=ws)
+    g = torch.tensor(rng.standard_normal((B, plan.n_outputs)), device=dev(),
+                     dtype=torch.complex64 if kind == "amps" else torch.float32)
+    shared = plan.backward(U, g[0].contiguous(), ws, out)
+    dense = plan.backward(U, g[:1].expand(B, -1).contiguous(), ws, out)
+    # the two seeds differ by at most the order of one product: a few ulps of dU
+    assert (shared - dense).abs().max() <= 2e-6 * shared.abs().max()
+    whole = plan.backward(U, g, ws, out)
+    for b in (0, B - 1):
+        alone = plan.backward(U, g[b].contiguous(), ws, out)
+        assert (alone[b] - whole[b]).abs().max() <= 2e-6 * whole[b].abs().max()
+
+
 @pytest.mark.parametrize("m,n,det,B", [(8, 4, "pnr", 33), (13, 4, "threshold", 40), (20, 3, "threshold", 5),
                                        (24, 3, "pnr", 3), (6, 6, "threshold", 7)])
 def test_arithmetic_index_path_matches_oracle(slos, m, n, det, B):
