@@ -54,3 +54,23 @@ def test_fidelity_kernel_rejects(slos):
         slos.fidelity_kernel([3, 3, 3, 0], U)   # 9 photons
     with pytest.raises(slos.SlosError):
         slos.fidelity_kernel([0, 0, 0, 0], U)   # no photon
+
+
+@pytest.mark.parametrize("m,s,N", [(3, [1, 0, 0], 1), (4, [1, 1, 0, 0], 16), (5, [2, 1, 0, 0, 0], 17), (7, [1, 1, 0, 2, 0, 0, 0], 33),
+                                   (5, [1] * 5, 50), (6, [1] * 6, 31), (24, [1] * 6 + [0] * 18, 18), (8, [1] * 7 + [0], 20),
+                                   (8, [1] * 8, 17)])
+def test_set_against_itself_computes_half_and_mirrors(slos, m, s, N):
+    """1 to 8 photons (the subset expansion's halves of 0 to 3 rows, Glynn's
+    formula beyond), ragged 16 x 16 tiles: a set against itself, where only
+    half of the tiles is computed, against the oracle, exactly symmetric, and
+    against a copy of the set, where every tile is."""
+    rng = np.random.default_rng(m * 7 + N)
+    U = workloads.haar_unitaries(m, N, rng).astype(np.complex64)
+    Ut = torch.tensor(U, device="cuda")
+    G = slos.fidelity_kernel(s, Ut)
+    full = slos.fidelity_kernel(s, Ut, Ut.clone())
+    assert torch.equal(G, G.T)
+    # the mirrored entry conjugates W: FP32 inner products rounded in the same order, up to a few ulps of 1
+    assert (G - full).abs().max() <= 1e-6
+    ref = oracle.fidelity_kernel(U.astype(np.complex128), U.astype(np.complex128), s)
+    assert np.abs(full.cpu().numpy() - ref).max() <= 2e-6
