@@ -16,18 +16,20 @@
 //     [Yr | Yi](b, t) = sum_s  xr_s [Ar | Ai](s, t) + xi_s [-Ai | Ar](s, t),
 // x_s = X[b][s] / g_s, A = A_n, its output columns interleaved (2t = re,
 // 2t + 1 = im of output t) so the epilogue forms g_t (Yr + i Yi) and its
-// |.|^2 from adjacent columns of one row.  For FP32-accurate products in TF32
-// (the tensor core reads 10 mantissa bits) every operand value v is split
-// into hi = v rounded to TF32 and lo = v - hi, and the GEMM sums
-// A_hi B_hi + A_hi B_lo + A_lo B_hi (the three-product split-precision
-// scheme; the dropped lo lo term is ~2^-22 of the product), accumulating in
-// FP32, in chunks of 32 MMAs in tensor memory whose sums the epilogue adds
-// in FP32 registers with round-to-nearest (tc_gemm_chunked_kernel: the
-// tensor core's own accumulation over the whole K biased |psi|^2 low by
-// 4e-5).  The batch runs in chunks of kEncodeChunk rows, so the split copy of
-// X needs a fixed workspace.
+// |.|^2 from adjacent columns of one row.  For FP32-accurate products on the
+// FP16 tensor path (tc_gemm_split_kernel) every operand value is scaled by a
+// power of two, one per row of X and one per output t, that brings the row's
+// largest magnitude to [2^14, 2^15), and split into hi = v rounded to FP16 and
+// lo = (v - hi) rounded to FP16: 22 significant bits down to 2^-18 of the
+// row's largest value, an absolute 2^-40 of it below.  The epilogue undoes
+// both scales.  The batch runs in chunks of kEncodeChunk rows, so the split
+// copy of X needs a fixed workspace.
+//
+// One call, 4096 states of 2002 amplitudes: 818 us with TF32 operands (GEMM
+// 645, splits and their clearing 110, transfer matrix 47), 441 us now (315, 67, 43).
 #include <cuda.h>
 #include <cudaTypedefs.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -47,17 +49,27 @@ namespace slos {
 slos_status_t fail(slos_status_t st, const std::string &msg);
 
 constexpr int kTransferThreads = 256;
+constexpr int kTransferRows = 4;  // input columns per block: they share the slot rows of the outputs
 
+// Layer k of the transfer matrix.  colmax (the last layer): per output t the
+// largest |re|, |im| over the inputs, as the bits of a non-negative float
+// (zeroed before the launch).
 template <int KW>
 __global__ void __launch_bounds__(kTransferThreads)
     transfer_kernel(const float2 *U, int m, const uint32_t *slots, const uint32_t *colinfo, int64_t Fk, int64_t Fp,
-                    const float2 *prev, float2 *cur, int first) {
-    __shared__ float2 uc[32];  // column c of U, zero past m (padding slots name mode kMaxModes)
-    const int64_t s = blockIdx.y;
-    const uint32_t ci = __ldg(colinfo + s);
-    const int c = (int)(ci & 31u);
-    const int64_t sp = ci >> 5;
-    if (threadIdx.x < 32) uc[threadIdx.x] = (int)threadIdx.x < m ? U[threadIdx.x * m + c] : make_float2(0.f, 0.f);
+                    const float2 *prev, float2 *cur, int first, unsigned int *colmax) {
+    __shared__ float2 uc[kTransferRows][32];  // column c of U, zero past m (padding slots name mode kMaxModes)
+    __shared__ int64_t from[kTransferRows];
+    const int64_t s0 = (int64_t)blockIdx.y * kTransferRows;
+    const int rows = (int)min((int64_t)kTransferRows, Fk - s0);
+    if (threadIdx.x < kTransferRows * 32) {
+        const int r = threadIdx.x >> 5, j = threadIdx.x & 31;
+        if (r < rows) {
+            const uint32_t ci = __ldg(colinfo + s0 + r);
+            uc[r][j] = j < m ? U[j * m + (int)(ci & 31u)] : make_float2(0.f, 0.f);
+            if (j == 0) from[r] = (int64_t)(ci >> 5) * Fp;
+        }
+    }
     __syncthreads();
     const int64_t t = (int64_t)blockIdx.x * kTransferThreads + threadIdx.x;
     if (t >= Fk) return;
@@ -71,37 +83,53 @@ __global__ void __launch_bounds__(kTransferThreads)
         e[4 * q4 + 2] = w4.z;
         e[4 * q4 + 3] = w4.w;
     }
-    float2 acc;
-    if (first) {
-        acc = uc[e[0] & 31u];  // one photon: <e_j|U|e_c> = U[j][c]
-    } else {
-        const float2 *pv = prev + sp * Fp;
-        acc = make_float2(0.f, 0.f);
+    unsigned int top = 0u;
 #pragma unroll
-        for (int q = 0; q < KW; ++q) acc = cfma(uc[e[q] & 31u], pv[e[q] >> 5], acc);
+    for (int r = 0; r < kTransferRows; ++r) {
+        if (r >= rows) break;
+        float2 acc;
+        if (first) {
+            acc = uc[r][e[0] & 31u];  // one photon: <e_j|U|e_c> = U[j][c]
+        } else {
+            const float2 *pv = prev + from[r];
+            acc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < KW; ++q) acc = cfma(uc[r][e[q] & 31u], pv[e[q] >> 5], acc);
+        }
+        cur[(s0 + r) * Fk + t] = acc;
+        // as unsigned integers non-negative floats order like their values, NaN above infinity
+        top = max(top, max(__float_as_uint(fabsf(acc.x)), __float_as_uint(fabsf(acc.y))));
     }
-    cur[s * Fk + t] = acc;
+    if (colmax) atomicMax(colmax + t, top);
 }
 
-// TF32 split of an FP32 value: hi = v rounded to nearest TF32 (ties away),
-// lo = v - hi (exact in FP32).
-__device__ __forceinline__ void tf32_split(float v, float &hi, float &lo) {
-    uint32_t h;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(v));
-    hi = __uint_as_float(h);
-    lo = v - hi;
+// Exponent of the power of two that brings a row whose largest magnitude has
+// these bits to [2^14, 2^15); 0 for rows of zeros and of values that are not
+// finite (their products are not either, whatever the scale).
+__device__ __forceinline__ int split_exponent(unsigned int bits) {
+    if (bits == 0u || bits >= 0x7f800000u) return 0;
+    return max(-126, min(126, 14 - ilogbf(__uint_as_float(bits))));
+}
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
+
+// v (scaled) = hi + lo in FP16.
+__device__ __forceinline__ void f16_split(float v, __half &hi, __half &lo) {
+    hi = __float2half_rn(v);
+    lo = __float2half_rn(v - __half2float(hi));
 }
 
 constexpr int kEncodeChunk = 4096;  // batch rows per GEMM launch
-constexpr int kEncodeKAlign = 32;   // K' padded to whole 128-byte TF32 stage rows
+constexpr int kEncodeKAlign = 64;   // K' padded to whole 128-byte FP16 stage rows
 
 // Real-form operand B of the GEMM, [N = 2K rows][K2 cols], K-major:
-//   row 2t:     cols s -> Ar[s][t],  K + s -> -Ai[s][t]
+//   row 2t:     cols s -> Ar[s][t],  K + s -> -Ai[s][t],  2K .. K2-1 -> 0
 //   row 2t + 1: cols s -> Ai[s][t],  K + s ->  Ar[s][t]
-// split into hi and lo copies; 32 x 32 tiles of A through shared memory, so
-// both the read (along t) and the writes (along s) are coalesced.
-__global__ void __launch_bounds__(256) encode_split_b_kernel(const float2 *A, int64_t K, int64_t K2, float *bhi,
-                                                             float *blo) {
+// scaled and split into hi and lo copies; 32 x 32 tiles of A through shared
+// memory, so both the read (along t) and the writes (along s) are coalesced.
+// colscale[t] = g_t over t's scale.
+__global__ void __launch_bounds__(256) encode_split_b_kernel(const float2 *A, int64_t K, int64_t K2,
+                                                             const unsigned int *colmax, const float *g, __half *bhi,
+                                                             __half *blo, float *colscale) {
     __shared__ float2 tile[32][33];
     const int64_t s0 = (int64_t)blockIdx.y * 32, t0 = (int64_t)blockIdx.x * 32;
     for (int i = threadIdx.y; i < 32; i += 8) {
@@ -111,42 +139,89 @@ __global__ void __launch_bounds__(256) encode_split_b_kernel(const float2 *A, in
     __syncthreads();
     for (int i = threadIdx.y; i < 32; i += 8) {
         const int64_t tt = t0 + i, ss = s0 + threadIdx.x;
-        if (tt >= K || ss >= K) continue;
-        const float2 v = tile[threadIdx.x][i];  // A[ss][tt]
-        const float vals[4] = {v.x, -v.y, v.y, v.x};  // (2t, s), (2t, K+s), (2t+1, s), (2t+1, K+s)
-        const int64_t o[4] = {2 * tt * K2 + ss, 2 * tt * K2 + K + ss, (2 * tt + 1) * K2 + ss, (2 * tt + 1) * K2 + K + ss};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float h, l;
-            tf32_split(vals[q], h, l);
-            bhi[o[q]] = h;
-            blo[o[q]] = l;
+        if (tt >= K) continue;
+        const int ex = split_exponent(__ldg(colmax + tt));
+        if (blockIdx.y == 0 && threadIdx.x == 0) colscale[tt] = g[tt] * pow2f(-ex);
+        if (blockIdx.y + 1 == gridDim.y) {
+            for (int64_t c = 2 * K + threadIdx.x; c < K2; c += 32)
+                bhi[2 * tt * K2 + c] = blo[2 * tt * K2 + c] = bhi[(2 * tt + 1) * K2 + c] = blo[(2 * tt + 1) * K2 + c] =
+                    __float2half_rn(0.f);
         }
+        if (ss >= K) continue;
+        const float sc = pow2f(ex);
+        const float2 v = tile[threadIdx.x][i];  // A[ss][tt]
+        __half rh, rl, ih, il;
+        f16_split(v.x * sc, rh, rl);
+        f16_split(v.y * sc, ih, il);
+        const int64_t o = 2 * tt * K2 + ss;
+        bhi[o] = rh;
+        blo[o] = rl;
+        bhi[o + K] = __hneg(ih);
+        blo[o + K] = __hneg(il);
+        bhi[o + K2] = ih;
+        blo[o + K2] = il;
+        bhi[o + K2 + K] = rh;
+        blo[o + K2 + K] = rl;
     }
 }
 
-// Real-form operand A of the GEMM for batch rows [b0, b0 + rows):
-// [rows][K2], cols s -> Re X[b][s] / g_s, K + s -> Im X[b][s] / g_s, the
-// padding columns 2K .. K2-1 zero; split into hi and lo copies.
-__global__ void __launch_bounds__(256) encode_split_a_kernel(const float2 *X, const float *g, int64_t b0, int rows,
-                                                             int64_t K, int64_t K2, float *ahi, float *alo) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)rows * K2) return;
-    const int64_t r = i / K2, c = i % K2;
-    float v = 0.f;
-    if (c < 2 * K) {
-        const int64_t ss = c < K ? c : c - K;
-        const float2 x = X[(b0 + r) * K + ss];
-        v = (c < K ? x.x : x.y) / __ldg(g + ss);
+// Real-form operand A of the GEMM for batch rows [b0, b0 + rows), one block
+// per row: [rows][K2], cols s -> Re X[b][s] / g_s, K + s -> Im X[b][s] / g_s,
+// the padding columns 2K .. K2-1 zero; scaled and split into hi and lo copies.
+// rowscale[r] = 1 over the row's scale.
+constexpr int kSplitThreads = 256;
+constexpr int kSplitKeep = 8;  // values per thread kept in registers between the maximum and the split
+__global__ void __launch_bounds__(kSplitThreads) encode_split_a_kernel(const float2 *X, const float *g, int64_t b0,
+                                                                       int64_t K, int64_t K2, __half *ahi, __half *alo,
+                                                                       float *rowscale) {
+    __shared__ unsigned int red[kSplitThreads / 32];
+    const int64_t r = blockIdx.x;
+    const float2 *x = X + (b0 + r) * K;
+    auto value = [&](int64_t s) {
+        const float2 v = x[s];
+        const float gs = __ldg(g + s);
+        return make_float2(v.x / gs, v.y / gs);
+    };
+    auto bits = [](float2 v) { return max(__float_as_uint(fabsf(v.x)), __float_as_uint(fabsf(v.y))); };
+    float2 keep[kSplitKeep];
+    unsigned int top = 0u;
+#pragma unroll
+    for (int i = 0; i < kSplitKeep; ++i) {
+        const int64_t s = threadIdx.x + (int64_t)i * kSplitThreads;
+        keep[i] = s < K ? value(s) : make_float2(0.f, 0.f);
+        top = max(top, bits(keep[i]));
     }
-    float h, l;
-    tf32_split(v, h, l);
-    ahi[i] = h;
-    alo[i] = l;
+    const int64_t rest = threadIdx.x + (int64_t)kSplitKeep * kSplitThreads;
+    for (int64_t s = rest; s < K; s += kSplitThreads) top = max(top, bits(value(s)));
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kSplitThreads / 32; ++w) top = max(top, red[w]);
+    const int ex = split_exponent(top);
+    const float sc = pow2f(ex);
+    __half *h = ahi + r * K2, *l = alo + r * K2;
+    auto put = [&](int64_t s, float2 v) {
+        __half rh, rl, ih, il;
+        f16_split(v.x * sc, rh, rl);
+        f16_split(v.y * sc, ih, il);
+        h[s] = rh;
+        l[s] = rl;
+        h[K + s] = ih;
+        l[K + s] = il;
+    };
+#pragma unroll
+    for (int i = 0; i < kSplitKeep; ++i) {
+        const int64_t s = threadIdx.x + (int64_t)i * kSplitThreads;
+        if (s < K) put(s, keep[i]);
+    }
+    for (int64_t s = rest; s < K; s += kSplitThreads) put(s, value(s));
+    for (int64_t c = 2 * K + threadIdx.x; c < K2; c += kSplitThreads) h[c] = l[c] = __float2half_rn(0.f);
+    if (threadIdx.x == 0) rowscale[r] = pow2f(-ex);
 }
 
-// FP32 matrix [rows][cols] (row stride ld elements, a multiple of 4), box
-// 32 x box_rows, 128-byte swizzle: the TF32 operand layout of tc_gemm.cuh.
+// FP16 matrix [rows][cols] (row stride ld elements, a multiple of 8), box
+// 64 x box_rows, 128-byte swizzle: the operand layout of tc_gemm.cuh.
 static PFN_cuTensorMapEncodeTiled_v12000 encode_map_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
     static std::once_flag once;
@@ -160,14 +235,14 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_map_fn() {
     });
     return fn;
 }
-static bool make_map_f32(CUtensorMap *map, const float *ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+static bool make_map_f16(CUtensorMap *map, const __half *ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
     auto fn = encode_map_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)(ld * 4)};
-    cuuint32_t box[2] = {(cuuint32_t)tc::TcKind<1>::kElems, (cuuint32_t)box_rows};
+    cuuint64_t strides[1] = {(cuuint64_t)(ld * 2)};
+    cuuint32_t box[2] = {(cuuint32_t)tc::BK, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(ptr), dims, strides, box, estr,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half *>(ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -185,15 +260,33 @@ static int64_t encode_k2(const slos_plan_s *p) {
     return (2 * p->K + kEncodeKAlign - 1) / kEncodeKAlign * kEncodeKAlign;
 }
 
-// workspace: the transfer matrices of layers n and n-1, then the split
-// operands B_hi, B_lo [2K][K2] and A_hi, A_lo [kEncodeChunk][K2]
-static size_t encode_bytes(const slos_plan_s *p) {
+// workspace: the transfer matrices of layers n and n-1, the split operands
+// B_hi, B_lo [2K][K2] and A_hi, A_lo [kEncodeChunk][K2], then the largest
+// magnitude and the scale of each output and the scale of each row of a chunk
+struct EncodeLayout {
+    size_t a, b, bhi, blo, ahi, alo, colmax, colscale, rowscale, total;
+};
+static EncodeLayout encode_layout(const slos_plan_s *p) {
     const int n = p->n;
-    const size_t a = (size_t)p->F[n] * p->F[n] * sizeof(float2);
-    const size_t b = n >= 2 ? (size_t)p->F[n - 1] * p->F[n - 1] * sizeof(float2) : 0;
-    const size_t bs = (size_t)2 * p->K * encode_k2(p) * sizeof(float);
-    const size_t as = (size_t)kEncodeChunk * encode_k2(p) * sizeof(float);
-    return align256(a) + align256(b) + 2 * align256(bs) + 2 * align256(as);
+    const size_t K = (size_t)p->K, K2 = (size_t)encode_k2(p);
+    EncodeLayout L;
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = at;
+        at += align256(bytes);
+        return o;
+    };
+    L.a = take((size_t)p->F[n] * p->F[n] * sizeof(float2));
+    L.b = take(n >= 2 ? (size_t)p->F[n - 1] * p->F[n - 1] * sizeof(float2) : 0);
+    L.bhi = take(2 * K * K2 * sizeof(__half));
+    L.blo = take(2 * K * K2 * sizeof(__half));
+    L.ahi = take(kEncodeChunk * K2 * sizeof(__half));
+    L.alo = take(kEncodeChunk * K2 * sizeof(__half));
+    L.colmax = take(K * sizeof(unsigned int));
+    L.colscale = take(K * sizeof(float));
+    L.rowscale = take(kEncodeChunk * sizeof(float));
+    L.total = at;
+    return L;
 }
 
 }  // namespace slos
@@ -207,7 +300,7 @@ slos_status_t slos_encoded_workspace_bytes(slos_plan_t p, size_t *bytes) {
     if (!encodable(p))
         return fail(SLOS_ERR_UNSUPPORTED, "slos_encoded_workspace_bytes: amplitude encoding needs a PNR plan with at "
                                           "most 32768 outputs");
-    *bytes = encode_bytes(p);
+    *bytes = encode_layout(p).total;
     return SLOS_OK;
 }
 
@@ -221,27 +314,32 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
     if (output != SLOS_OUT_PROBS && output != SLOS_OUT_AMPS)
         return fail(SLOS_ERR_INVALID_ARG, "slos_encoded_forward: bad output");
     if (!U || (batch > 0 && (!X || !out))) return fail(SLOS_ERR_INVALID_ARG, "slos_encoded_forward: NULL pointer");
-    if (!workspace || workspace_bytes < encode_bytes(p))
+    const EncodeLayout L = encode_layout(p);
+    if (!workspace || workspace_bytes < L.total)
         return fail(SLOS_ERR_INVALID_ARG, "slos_encoded_forward: workspace too small (slos_encoded_workspace_bytes)");
     cudaStream_t s = (cudaStream_t)stream;
     const int n = p->n, m = p->m;
     char *ws = reinterpret_cast<char *>(workspace);
-    float2 *buf[2] = {reinterpret_cast<float2 *>(ws),
-                      reinterpret_cast<float2 *>(ws + align256((size_t)p->F[n] * p->F[n] * sizeof(float2)))};
+    float2 *buf[2] = {reinterpret_cast<float2 *>(ws + L.a), reinterpret_cast<float2 *>(ws + L.b)};
+    unsigned int *colmax = reinterpret_cast<unsigned int *>(ws + L.colmax);
     const float2 *Ud = reinterpret_cast<const float2 *>(U);
     cudaError_t e;
+    if ((e = cudaMemsetAsync(colmax, 0, (size_t)p->K * sizeof(unsigned int), s)) != cudaSuccess)
+        return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
     {
         ProfScope ps("slos_transfer", 0.0, s);
         for (int k = 1; k <= n; ++k) {
             const int64_t Fk = p->F[k], Fp = p->F[k - 1];
             float2 *cur = buf[(n - k) & 1];
             const float2 *prev = k >= 2 ? buf[(n - k + 1) & 1] : nullptr;
-            dim3 grid((unsigned)((Fk + kTransferThreads - 1) / kTransferThreads), (unsigned)Fk);
+            dim3 grid((unsigned)((Fk + kTransferThreads - 1) / kTransferThreads),
+                      (unsigned)((Fk + kTransferRows - 1) / kTransferRows));
+            unsigned int *top = k == n ? colmax : nullptr;
             const uint32_t *sl = p->tab.layer[k].slots, *ci = p->tab.layer[k].colinfo;
             switch (p->tab.layer[k].kw) {
-                case 4: transfer_kernel<4><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1); break;
-                case 8: transfer_kernel<8><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1); break;
-                default: transfer_kernel<12><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1); break;
+                case 4: transfer_kernel<4><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top); break;
+                case 8: transfer_kernel<8><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top); break;
+                default: transfer_kernel<12><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top); break;
             }
             if ((e = cudaGetLastError()) != cudaSuccess)
                 return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
@@ -249,19 +347,13 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
     }
     if (batch == 0) return SLOS_OK;
     const int64_t K = p->K, K2 = encode_k2(p);
-    const size_t bs = (size_t)2 * K * K2 * sizeof(float), as = (size_t)kEncodeChunk * K2 * sizeof(float);
-    char *w = ws + align256((size_t)p->F[n] * p->F[n] * sizeof(float2)) +
-              (n >= 2 ? align256((size_t)p->F[n - 1] * p->F[n - 1] * sizeof(float2)) : 0);
-    float *bhi = reinterpret_cast<float *>(w), *blo = reinterpret_cast<float *>(w + align256(bs));
-    float *ahi = reinterpret_cast<float *>(w + 2 * align256(bs));
-    float *alo = reinterpret_cast<float *>(w + 2 * align256(bs) + align256(as));
+    __half *bhi = reinterpret_cast<__half *>(ws + L.bhi), *blo = reinterpret_cast<__half *>(ws + L.blo);
+    __half *ahi = reinterpret_cast<__half *>(ws + L.ahi), *alo = reinterpret_cast<__half *>(ws + L.alo);
+    float *colscale = reinterpret_cast<float *>(ws + L.colscale), *rowscale = reinterpret_cast<float *>(ws + L.rowscale);
     {
         ProfScope ps("slos_encode_split", 0.0, s);
-        // B's padding columns stay zero: clear both copies, then fill
-        if ((e = cudaMemsetAsync(bhi, 0, 2 * align256(bs), s)) != cudaSuccess)
-            return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
         dim3 grid((unsigned)((K + 31) / 32), (unsigned)((K + 31) / 32));
-        encode_split_b_kernel<<<grid, dim3(32, 8), 0, s>>>(buf[0], K, K2, bhi, blo);
+        encode_split_b_kernel<<<grid, dim3(32, 8), 0, s>>>(buf[0], K, K2, colmax, p->tab.gfact, bhi, blo, colscale);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
     }
@@ -269,23 +361,22 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_done[dev]) {
-        if ((e = cudaFuncSetAttribute(tc::tc_gemm_chunked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      tc::kCkSmem)) != cudaSuccess)
+        if ((e = cudaFuncSetAttribute(tc::tc_gemm_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      tc::kSpSmem)) != cudaSuccess)
             return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
         attr_done[dev] = true;
     }
     CUtensorMap mah, mal, mbh, mbl;
-    if (!make_map_f32(&mbh, bhi, 2 * K, K2, K2, tc::kCkBN) || !make_map_f32(&mbl, blo, 2 * K, K2, K2, tc::kCkBN) ||
-        !make_map_f32(&mah, ahi, kEncodeChunk, K2, K2, tc::BM) || !make_map_f32(&mal, alo, kEncodeChunk, K2, K2, tc::BM))
+    if (!make_map_f16(&mbh, bhi, 2 * K, K2, K2, tc::kSpBN) || !make_map_f16(&mbl, blo, 2 * K, K2, K2, tc::kSpBN) ||
+        !make_map_f16(&mah, ahi, kEncodeChunk, K2, K2, tc::BM) || !make_map_f16(&mal, alo, kEncodeChunk, K2, K2, tc::BM))
         return fail(SLOS_ERR_CUDA, "slos_encoded_forward: cuTensorMapEncodeTiled failed");
     const float2 *Xd = reinterpret_cast<const float2 *>(X);
     for (int b0 = 0; b0 < batch; b0 += kEncodeChunk) {
         const int rows = std::min(kEncodeChunk, batch - b0);
         {
             ProfScope ps("slos_encode_split", 0.0, s);
-            const int64_t cnt = (int64_t)rows * K2;
-            encode_split_a_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(Xd, p->tab.gfact, b0, rows, K, K2,
-                                                                                 ahi, alo);
+            encode_split_a_kernel<<<(unsigned)rows, kSplitThreads, 0, s>>>(Xd, p->tab.gfact, b0, K, K2, ahi, alo,
+                                                                           rowscale);
             if ((e = cudaGetLastError()) != cudaSuccess)
                 return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
         }
@@ -297,13 +388,14 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
         g.ldc = (int)K;
         g.C = output == SLOS_OUT_AMPS ? (void *)(reinterpret_cast<float2 *>(out) + (int64_t)b0 * K)
                                       : (void *)(reinterpret_cast<float *>(out) + (int64_t)b0 * K);
-        g.colscale = p->tab.gfact;
+        g.colscale = colscale;
+        g.rowscale = rowscale;
         g.amps = output == SLOS_OUT_AMPS ? 1 : 0;
         g.err = p->d_status + 2;
-        const int64_t tiles = (int64_t)((g.N + tc::kCkBN - 1) / tc::kCkBN) * ((rows + tc::BM - 1) / tc::BM);
+        const int64_t tiles = (int64_t)((g.N + tc::kSpBN - 1) / tc::kSpBN) * ((rows + tc::BM - 1) / tc::BM);
         const unsigned grid = (unsigned)std::min<int64_t>(tiles, p->sm_count);
         ProfScope ps("slos_encode_gemm", 3.0 * 2.0 * rows * (double)g.N * (double)K2, s);  // flops
-        tc::tc_gemm_chunked_kernel<<<grid, tc::kCkThreads, tc::kCkSmem, s>>>(mah, mbh, mal, mbl, g);
+        tc::tc_gemm_split_kernel<<<grid, tc::kSpThreads, tc::kSpSmem, s>>>(mah, mbh, mal, mbl, g);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
     }

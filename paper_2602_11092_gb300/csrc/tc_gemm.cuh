@@ -1,9 +1,8 @@
 // Tensor-core GEMM for sm_103a: C[M][N] = A[M][K] . B[N][K]^T, BF16 inputs
 // (both K-major), FP32 accumulation in tensor memory (TMEM), fused epilogues.
-// tc_gemm_chunked_kernel (end of the file) takes TF32 operands (FP32
-// storage, the tensor core reads 19 bits of each): a stage row is 128 bytes
-// either way (64 BF16 or 32 FP32 elements), four MMAs of 32 bytes of K each
-// (K = 16 or 8), so the ring, the swizzle and the descriptors are the same.
+// tc_gemm_split_kernel (end of the file) multiplies FP32-accurate operands
+// given as pairs of FP16 copies, with the same stage rows of 128 bytes (64
+// 16-bit elements), swizzle and descriptors.
 // Two kernels share the pipeline below: tc_gemm_kernel (one tile per CTA) and
 // tc_gemm_persist_kernel (one CTA per SM over many tiles, two accumulators,
 // the epilogue of one tile overlapping the next tile's MMAs), which the
@@ -46,7 +45,7 @@ enum TcEpi : int {
     TC_GELU = 2,       // Z = acc + bias[n] (bf16, aux), C = gelu(Z) (bf16)
     TC_GELU_BWD = 3,   // C = acc * gelu'(Z), Z = aux (bf16 in), C bf16
     TC_F32_ACCUM = 4,  // C += acc                        (float)
-    TC_ENCODE = 5,     // columns (2t, 2t+1) = (re, im) of output t: psi = colscale[t] (re + i im);
+    TC_ENCODE = 5,     // columns (2t, 2t+1) = (re, im) of output t: psi = rowscale[row] colscale[t] (re + i im);
                        //   C float |psi|^2, or complex64 psi when amps (row stride ldc outputs)
 };
 
@@ -58,6 +57,7 @@ struct TcArgs {
     __nv_bfloat16 *aux;   // [M][ldc] (Z for TC_GELU out, TC_GELU_BWD in)
     int *err;             // error word (device)
     const float *colscale;  // TC_ENCODE: [N / 2]
+    const float *rowscale;  // TC_ENCODE: [M]
     int amps;               // TC_ENCODE: complex64 output
 };
 
@@ -122,12 +122,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
         "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
         : "memory");
 }
-// Operand kinds: 0 = BF16, 1 = TF32; elements per 128-byte stage row.
-template <int KIND>
-struct TcKind {
-    static constexpr int kElems = KIND == 0 ? 64 : 32;
-};
-
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
@@ -167,12 +161,13 @@ template <int EPI>
 __device__ __forceinline__ void tc_store16(const TcArgs &g, int row, int col0, float (&v)[16], bool vec) {
     if (EPI == TC_ENCODE) {
         if (row < g.M) {
+            const float rs = g.rowscale[row];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int t = col0 / 2 + i;
                 if (2 * t >= g.N) break;
                 const float c = g.colscale[t];
-                const float re = v[2 * i] * c, im = v[2 * i + 1] * c;
+                const float re = v[2 * i] * rs * c, im = v[2 * i + 1] * rs * c;  // rs a power of two
                 const int64_t o = (int64_t)row * g.ldc + t;
                 if (g.amps) reinterpret_cast<float2 *>(g.C)[o] = make_float2(re, im);
                 else reinterpret_cast<float *>(g.C)[o] = re * re + im * im;
@@ -512,80 +507,85 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
 namespace slos {
 namespace tc {
 
-// ---------------------------------------------------------------- chunked accumulation
-// tc_gemm_chunked_kernel: the persistent pipeline (128 x 256 tiles) with the
-// K sum taken in chunks of kChunkStages stages.  The tensor core's FP32
-// accumulation does not round to nearest: over the ~1500 MMAs of a long K its
-// errors pile up in one direction (measured: |psi|^2 of the amplitude-encoding
-// GEMM biased low by 4e-5 at K' = 3 x 4032).  Here each chunk accumulates
-// into one of two TMEM buffers while the epilogue warps move the other
-// buffer's finished chunk into FP32 registers (half a row, 128 columns, per
-// thread; round-to-nearest adds), so a truncation bias builds up only within
-// one chunk.  Roles: warp 0 TMA producer, warp 1 MMA issuer, warps 2-9
-// epilogue (TMEM lane quarter = warp % 4, columns 0-127 for warps 2-5 and
-// 128-255 for warps 6-9).  Waits are bounded as above.
-constexpr int kCkBN = 256;
-constexpr int kCkStages = 4;
-constexpr int kChunkStages = 8;  // 32 MMAs per chunk
-constexpr int kCkThreads = 320;
-constexpr int kCkEpiWarps = 8;
-constexpr int kCkATile = BM * 128, kCkBTile = kCkBN * 128;  // bytes: 128-byte rows
-constexpr int kCkStageBytes = kCkATile + kCkBTile;
-constexpr int kCkSmem = kCkStages * kCkStageBytes + 1024 + 256;
-constexpr uint32_t kCkTmemCols = 2 * kCkBN;
-// kind::tf32: A and B TF32 (bits 7-9 = 2, 10-12 = 2), otherwise as kIdesc.
-constexpr uint32_t kIdescTf32 =
-    (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kCkBN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+// ---------------------------------------------------------------- split operands
+// tc_gemm_split_kernel: FP32-accurate products on the FP16 tensor path.  Each
+// operand value is scaled by a power of two of its row and split into two FP16
+// numbers, v = hi + lo (22 significant bits), and the product is
+// A_hi B_hi + A_hi B_lo + A_lo B_hi (the dropped lo lo term is ~2^-22 of it).
+//
+// A stage holds the hi and the lo tile of both operands for 64 values of K and
+// feeds all three products from them (12 MMAs).  The loads bound a GEMM of
+// 128 x 256 tiles here: one product per pair of tiles needs 96 bytes per clock
+// and SM at full tensor rate, against the 56 or so that the L2 delivers, the
+// shared stage 64.  TF32 operands in three passes over hi and lo copies, the
+// form before, need twice the MMAs (K = 8 each at half rate) and one load per
+// product: 645 us for 4096 x 2002 complex (611 TFLOP/s of MMA work),
+// 315 us now (1250 TFLOP/s).
+//
+// The tensor core's FP32 accumulation does not round to nearest: over the
+// ~1500 MMAs of a long K its errors pile up in one direction (measured:
+// |psi|^2 of the amplitude-encoding GEMM biased low by 4e-5 when one
+// accumulator took all of them).  So the K sum is taken in chunks of
+// kSpChunkStages stages: each chunk accumulates into one of two TMEM buffers
+// while the epilogue warps move the other buffer's finished chunk into FP32
+// registers (half a row, 128 columns, per thread; round-to-nearest adds).
+// Roles: warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue (TMEM lane
+// quarter = warp % 4, columns 0-127 for warps 2-5 and 128-255 for warps 6-9).
+// Waits are bounded as above.
+constexpr int kSpBN = 256;
+constexpr int kSpStages = 2;
+constexpr int kSpChunkStages = 2;  // 24 MMAs per chunk
+constexpr int kSpThreads = 320;
+constexpr int kSpEpiWarps = 8;
+constexpr int kSpATile = BM * 128, kSpBTile = kSpBN * 128;  // bytes: 128-byte rows
+constexpr int kSpStageBytes = 2 * (kSpATile + kSpBTile);    // A hi, A lo, B hi, B lo
+constexpr int kSpSmem = kSpStages * kSpStageBytes + 1024 + 256;
+constexpr uint32_t kSpTmemCols = 2 * kSpBN;
+// kind::f16 with A and B FP16 (bits 7-9 = 0, 10-12 = 0), otherwise as kIdesc.
+constexpr uint32_t kIdescF16 = (1u << 4) | ((uint32_t)(kSpBN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(kIdescTf32), "r"(accumulate)
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(kIdescF16), "r"(accumulate)
         : "memory");
 }
 
-// TF32 operands in three K segments, A_hi B_hi + A_hi B_lo + A_lo B_hi, each
-// segment's tiles taken from the hi or lo copy of an operand (the
-// three-TF32-product scheme for FP32-accurate products); TC_ENCODE epilogue.
-static __global__ void __launch_bounds__(kCkThreads, 1)
-    tc_gemm_chunked_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-                           const __grid_constant__ CUtensorMap ta_lo, const __grid_constant__ CUtensorMap tb_lo,
-                           TcArgs g) {
-    constexpr int KE = TcKind<1>::kElems;
+static __global__ void __launch_bounds__(kSpThreads, 1)
+    tc_gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
+                         const __grid_constant__ CUtensorMap ta_lo, const __grid_constant__ CUtensorMap tb_lo,
+                         TcArgs g) {
     extern __shared__ uint8_t smem_tc[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_tc) + 1023) & ~uintptr_t(1023));
-    uint8_t *sA = base;
-    uint8_t *sB = base + kCkStages * kCkATile;
-    uint64_t *full = reinterpret_cast<uint64_t *>(sB + kCkStages * kCkBTile);
-    uint64_t *empty = full + kCkStages;
-    uint64_t *cfull = empty + kCkStages;  // [2] a chunk's MMAs are done
+    uint64_t *full = reinterpret_cast<uint64_t *>(base + kSpStages * kSpStageBytes);
+    uint64_t *empty = full + kSpStages;
+    uint64_t *cfull = empty + kSpStages;  // [2] a chunk's MMAs are done
     uint64_t *cempty = cfull + 2;         // [2] the epilogue has taken the chunk
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(cempty + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nk1 = (g.K + KE - 1) / KE;
-    const int nk = 3 * nk1;
-    const int nchunks = (nk + kChunkStages - 1) / kChunkStages;
-    const int ntn = (g.N + kCkBN - 1) / kCkBN;
+    const int nk = (g.K + BK - 1) / BK;
+    const int nchunks = (nk + kSpChunkStages - 1) / kSpChunkStages;
+    const int ntn = (g.N + kSpBN - 1) / kSpBN;
     const int ntiles = ((g.M + BM - 1) / BM) * ntn;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kCkStages; ++s) {
+        for (int s = 0; s < kSpStages; ++s) {
             mbar_init(full + s, 1);
             mbar_init(empty + s, 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(cfull + a, 1);
-            mbar_init(cempty + a, kCkEpiWarps);
+            mbar_init(cempty + a, kSpEpiWarps);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(kCkTmemCols)
+                     "r"(kSpTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -599,25 +599,26 @@ static __global__ void __launch_bounds__(kCkThreads, 1)
             // producer: every stage of every tile, in order
             uint32_t it = 0;
             for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
-                const int m0 = (t / ntn) * BM, n0 = (t % ntn) * kCkBN;
+                const int m0 = (t / ntn) * BM, n0 = (t % ntn) * kSpBN;
                 for (int kt = 0; kt < nk; ++kt, ++it) {
-                    const int s = it % kCkStages;
-                    const uint32_t ph = (it / kCkStages) & 1;
-                    if (it >= (uint32_t)kCkStages && !mbar_wait(empty + s, ph ^ 1)) {
+                    const int s = it % kSpStages;
+                    const uint32_t ph = (it / kSpStages) & 1;
+                    if (it >= (uint32_t)kSpStages && !mbar_wait(empty + s, ph ^ 1)) {
                         atomicExch(g.err, 1);
                         *abort_flag = 1;
                         break;
                     }
                     if (*abort_flag) break;
-                    mbar_expect_tx(full + s, kCkStageBytes);
-                    const int seg = kt / nk1;  // 0: A_hi B_hi, 1: A_hi B_lo, 2: A_lo B_hi
-                    const int kx = (kt - seg * nk1) * KE;
-                    tma_load_2d(sA + s * kCkATile, seg == 2 ? &ta_lo : &ta, kx, m0, full + s);
-                    tma_load_2d(sB + s * kCkBTile, seg == 1 ? &tb_lo : &tb, kx, n0, full + s);
+                    uint8_t *st = base + s * kSpStageBytes;
+                    mbar_expect_tx(full + s, kSpStageBytes);
+                    tma_load_2d(st, &ta, kt * BK, m0, full + s);
+                    tma_load_2d(st + 2 * kSpATile, &tb, kt * BK, n0, full + s);
+                    tma_load_2d(st + 2 * kSpATile + kSpBTile, &tb_lo, kt * BK, n0, full + s);
+                    tma_load_2d(st + kSpATile, &ta_lo, kt * BK, m0, full + s);
                 }
             }
-            for (uint32_t q = (it > (uint32_t)kCkStages ? it - kCkStages : 0); q < it; ++q)
-                mbar_wait(full + (q % kCkStages), (q / kCkStages) & 1);
+            for (uint32_t q = (it > (uint32_t)kSpStages ? it - kSpStages : 0); q < it; ++q)
+                mbar_wait(full + (q % kSpStages), (q / kSpStages) & 1);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -633,22 +634,27 @@ static __global__ void __launch_bounds__(kCkThreads, 1)
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(b * kCkBN);
-                    const int k1 = min(nk, (ch + 1) * kChunkStages);
-                    for (int kt = ch * kChunkStages; kt < k1; ++kt, ++it) {
-                        const int s = it % kCkStages;
-                        const uint32_t ph = (it / kCkStages) & 1;
+                    const uint32_t d = tmem + (uint32_t)(b * kSpBN);
+                    const int k1 = min(nk, (ch + 1) * kSpChunkStages);
+                    for (int kt = ch * kSpChunkStages; kt < k1; ++kt, ++it) {
+                        const int s = it % kSpStages;
+                        const uint32_t ph = (it / kSpStages) & 1;
                         if (*abort_flag || !mbar_wait(full + s, ph)) {
                             atomicExch(g.err, 2);
                             *abort_flag = 1;
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t a0 = smem_u32(sA + s * kCkATile), b0 = smem_u32(sB + s * kCkBTile);
+                        const uint32_t ah = smem_u32(base + s * kSpStageBytes), al = ah + kSpATile;
+                        const uint32_t bh = ah + 2 * kSpATile, bl = bh + kSpBTile;
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            mma_tf32(d, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32),
-                                     (kt > ch * kChunkStages || kk > 0) ? 1u : 0u);
+                        for (int kk = 0; kk < 4; ++kk) {
+                            const uint64_t dah = sw128_desc(ah + kk * 32), dal = sw128_desc(al + kk * 32);
+                            const uint64_t dbh = sw128_desc(bh + kk * 32), dbl = sw128_desc(bl + kk * 32);
+                            mma_f16(d, dal, dbh, (kt > ch * kSpChunkStages || kk > 0) ? 1u : 0u);
+                            mma_f16(d, dah, dbl, 1u);
+                            mma_f16(d, dah, dbh, 1u);
+                        }
                         mma_commit(empty + s);
                     }
                     if (*abort_flag) break;
@@ -658,7 +664,7 @@ static __global__ void __launch_bounds__(kCkThreads, 1)
         }
     } else {
         // epilogue warps: each thread sums 128 columns of its row over the chunks
-        constexpr int HC = kCkBN / 2;
+        constexpr int HC = kSpBN / 2;
         const int q = warp & 3;
         const int hc = (warp - 2) >> 2;  // column half
         uint32_t c = 0;
@@ -678,7 +684,7 @@ static __global__ void __launch_bounds__(kCkThreads, 1)
                     break;
                 }
                 tc_fence_after();
-                const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * kCkBN + hc * HC);
+                const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * kSpBN + hc * HC);
 #pragma unroll
                 for (int c16 = 0; c16 < HC; c16 += 16) {
                     float v[16];
@@ -691,7 +697,7 @@ static __global__ void __launch_bounds__(kCkThreads, 1)
                 if (lane == 0) mbar_arrive(cempty + b);
             }
             if (!ok) break;
-            const int m0 = (t / ntn) * BM, n0 = (t % ntn) * kCkBN + hc * HC;
+            const int m0 = (t / ntn) * BM, n0 = (t % ntn) * kSpBN + hc * HC;
             const int row = m0 + q * 32 + lane;
 #pragma unroll
             for (int c16 = 0; c16 < HC; c16 += 16) {
@@ -706,7 +712,7 @@ static __global__ void __launch_bounds__(kCkThreads, 1)
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCkTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSpTmemCols) : "memory");
     }
 }
 

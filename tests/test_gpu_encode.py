@@ -90,3 +90,32 @@ def test_encoded_rejects_large_or_threshold_plans(slos):
         slos.Plan(4, [1, 1, 0, 0], slos.THRESHOLD).encoded_forward(
             torch.eye(4, dtype=torch.complex64, device="cuda"), torch.zeros((1, 10), dtype=torch.complex64,
                                                                             device="cuda"))
+
+
+@pytest.mark.parametrize("m,n,B", [(5, 2, 6), (6, 3, 131), (11, 5, 5), (2, 7, 1)])
+def test_encoded_rows_and_outputs_of_any_scale(slos, m, n, B):
+    """The operands are split into FP16 pairs at a scale of their own per
+    state vector and per output: vectors of norms 1e-20 to 1e15 and a zero
+    vector, and a lossy map (one mode damped by 1e-5, so outputs with many
+    photons there are 1e-25 of the others), odd output counts and ones beyond
+    a row's registers.  Every vector and every output keeps the relative
+    accuracy of its own size: the split's 2^-22 and the FP32 recursion's few
+    ulps, accumulated over the sum, against an FP64 restatement."""
+    rng = np.random.default_rng(17 * m + n)
+    plan = slos.Plan(m, [n] + [0] * (m - 1))
+    basis = oracle.enumerate_fock(m, n)
+    K = plan.n_outputs
+    U = workloads.haar_unitaries(m, 1, rng)[0]
+    U[1, :] *= 1e-5
+    U = U.astype(np.complex64)
+    X = rand_states(rng, B, K).astype(np.complex128)
+    X *= (10.0 ** rng.uniform(-20, 15, size=B))[:, None]
+    X[B // 2] = 0.0
+    X = X.astype(np.complex64)
+    amps = plan.encoded_forward(torch.tensor(U, device="cuda"), torch.tensor(X, device="cuda"), slos.AMPS).cpu().numpy()
+    ref = oracle.encoded_amplitudes(U.astype(np.complex128), X.astype(np.complex128), basis)
+    norm = np.linalg.norm(X.astype(np.complex128), axis=1)
+    size = np.abs(oracle.transfer_matrix(U.astype(np.complex128), basis)).max(axis=1)  # largest entry of each output
+    bound = 4e-6 * np.sqrt(K) * norm[:, None] * size[None, :]
+    assert np.all(np.abs(amps - ref) <= bound + 1e-44)
+    assert np.all(amps[B // 2] == 0)
