@@ -1438,7 +1438,8 @@ slos_status_t slos_workspace_bytes(slos_plan_t p, int batch, int training, size_
 }
 
 static slos_status_t launch_layer_fwd(slos_plan_s *p, const Layout &Ly, char *ws, const float2 *U, int batch, int k,
-                                      int epi, bool save, void *out, cudaStream_t s, bool recompute = false) {
+                                      int epi, bool save, void *out, cudaStream_t s, bool recompute = false,
+                                      int width = kLanes) {
     int *counter = reinterpret_cast<int *>(ws + Ly.counters) + (recompute ? kCtrRecompute + k : k);
     const int NG = groups_for(batch);
     FwdArgs a;
@@ -1486,6 +1487,10 @@ static slos_status_t launch_layer_fwd(slos_plan_s *p, const Layout &Ly, char *ws
         }
         // warp items: one chunk of consecutive states (threshold: one run of
         // whole patterns) of a group pair
+        if (width < kLanes) {
+            SLOS_CUDA(slos_launch_fwd_narrow(a, t, epi, width, s));
+            return SLOS_OK;
+        }
         const int64_t chunks = epi == EPI_THRESH ? t.nseg : (a.Fk + slos_pair_chunk() - 1) / slos_pair_chunk();
         const int64_t items = chunks * ((NG + 1) / 2);
         const int64_t blocks = (items + slos_pair_warps() - 1) / slos_pair_warps();
@@ -1520,6 +1525,7 @@ static PrefixArgs prefix_args(const slos_plan_s *p, const float2 *U, int batch) 
     pa.m = p->m;
     pa.L = L;
     pa.B = batch;
+    pa.lanes = kLanes;
     pa.NI = slos_prefix_ni(p->m, L, p->F.data(), batch, p->sm_count);
     if (p->tune_prefix_ni > 0 && slos_prefix_bwd_smem(p->tune_prefix_ni, L, p->F.data()) <= kPrefixSmemLimit)
         pa.NI = p->tune_prefix_ni;
@@ -1529,8 +1535,10 @@ static PrefixArgs prefix_args(const slos_plan_s *p, const float2 *U, int batch) 
 // Layers 1..prefix_L in one on-chip launch; writes layer k to the workspace
 // when bit k of `want` is set.
 static slos_status_t launch_prefix_fwd(const slos_plan_s *p, const Layout &Ly, char *ws, const float2 *U, int batch,
-                                       uint32_t want, const char *name, cudaStream_t s) {
+                                       uint32_t want, const char *name, cudaStream_t s, int lanes = kLanes) {
     PrefixArgs pa = prefix_args(p, U, batch);
+    pa.lanes = lanes;
+    pa.NI = std::min(pa.NI, lanes);
     double bytes = 8.0 * p->m * p->m;
     for (int k = 1; k <= pa.L; ++k)
         if ((want >> k) & 1u) {
@@ -1540,6 +1548,33 @@ static slos_status_t launch_prefix_fwd(const slos_plan_s *p, const Layout &Ly, c
     ProfScope ps(name, bytes * batch, s);
     SLOS_CUDA(slos_launch_prefix_fwd(pa, s));
     return SLOS_OK;
+}
+
+// Width of the lane = state kernels (slos_narrow.cu) for an inference forward,
+// or kLanes for the others.  They cost in proportion to the batch, the two-group
+// walk at least the latency of 64 instances per layer, the on-chip forward that
+// of one CTA per few instances however few there are.  Measured (us, this
+// kernel / the other, whole forwards replayed from a graph):
+//   layered, PNR:  m=16 n=8 batch 1 25 / 184, 16 77 / 190, 64 236 / 236;
+//                  m=14 n=7 64 47 / 66, 512 259 / 290; m=20 n=5 256 62 / 67, 2048 457 / 435
+//   layered, threshold (parents of a pattern's states lie apart, so a warp's
+//   gathers share less): m=16 n=6 64 55 / 70, 256 151 / 125; m=20 n=6 48 104 / 111,
+//                  64 131 / 117; m=14 n=6 192 66 / 72, 256 83 / 80; m=16 n=4 2048 66 / 74
+//   on chip, 1024-thread CTAs: m=12 n=6 1 17 / 32, 192 30 / 37, 384 46 / 37;
+//                  m=13 n=6 192 37 / 37; m=16 n=5 256 30 / 37, 384 45 / 37
+//   on chip, small: m=10 n=5 1 10.4 / 8.4, 4..256 10.5 / 12.5, 384 17 / 13; m=9 n=4 8.5 / 6.4
+// hence the lines: final states of the whole batch for the layered plans, a
+// little over one instance per SM for the on-chip ones.
+static int narrow_width(const slos_plan_s *p, int batch) {
+    if (!p->tab.enabled) return kLanes;
+    const int width = slos_narrow_width(batch);
+    if (p->fused_ni > 0) {
+        if (4 * (int64_t)batch > 5 * (int64_t)p->sm_count) return kLanes;
+        if (p->fused_threads == 1024) return width;
+        return p->F[p->n] >= 2000 && batch >= 4 ? width : kLanes;
+    }
+    const int64_t most = p->det == SLOS_DETECT_PNR ? (int64_t)1 << 25 : 6500000;
+    return (int64_t)batch * p->F[p->n] <= most ? width : kLanes;
 }
 
 slos_status_t slos_forward(slos_plan_t p, const void *U, int batch, slos_output_t output, void *out,
@@ -1566,7 +1601,8 @@ slos_status_t slos_forward(slos_plan_t p, const void *U, int batch, slos_output_
     char *ws = reinterpret_cast<char *>(workspace);
     const float2 *Ud = reinterpret_cast<const float2 *>(U);
     const int n = p->n;
-    if (!save && p->fused_ni > 0) {
+    const int width = save ? kLanes : narrow_width(p, batch);
+    if (!save && p->fused_ni > 0 && width == kLanes) {
         // whole plan on chip: only U in and the outputs out
         FusedArgs fa;
         memset(&fa, 0, sizeof(fa));
@@ -1601,7 +1637,7 @@ slos_status_t slos_forward(slos_plan_t p, const void *U, int batch, slos_output_
         SLOS_CUDA(slos_launch_fused(fa, output == SLOS_OUT_AMPS ? EPI_AMPS : EPI_PROBS, s));
         return SLOS_OK;
     }
-    SLOS_CUDA(cudaMemsetAsync(ws + Ly.counters, 0, kCounters * sizeof(int), s));
+    if (width == kLanes) SLOS_CUDA(cudaMemsetAsync(ws + Ly.counters, 0, kCounters * sizeof(int), s));
     int k0 = 1;
     if (prefix_layers(p) >= 2) {
         // kept layers of the prefix and its last layer (which layer L + 1 reads)
@@ -1609,19 +1645,20 @@ slos_status_t slos_forward(slos_plan_t p, const void *U, int batch, slos_output_
         uint32_t want = 1u << L;
         for (int k = 1; k < L; ++k)
             if (save && p->stored[k]) want |= 1u << k;
-        slos_status_t st = launch_prefix_fwd(p, Ly, ws, Ud, batch, want, "slos_fwd_prefix", s);
+        slos_status_t st = launch_prefix_fwd(p, Ly, ws, Ud, batch, want, "slos_fwd_prefix", s, width);
         if (st != SLOS_OK) return st;
         k0 = L + 1;
     }
     for (int k = k0; k < n; ++k) {
-        slos_status_t st = launch_layer_fwd(p, Ly, ws, Ud, batch, k, EPI_STORE, true, nullptr, s);
+        slos_status_t st = launch_layer_fwd(p, Ly, ws, Ud, batch, k, EPI_STORE, true, nullptr, s, false, width);
         if (st != SLOS_OK) return st;
     }
     if (p->det != SLOS_DETECT_THRESHOLD)
-        return launch_layer_fwd(p, Ly, ws, Ud, batch, n, output == SLOS_OUT_AMPS ? EPI_AMPS : EPI_PROBS, save, out, s);
+        return launch_layer_fwd(p, Ly, ws, Ud, batch, n, output == SLOS_OUT_AMPS ? EPI_AMPS : EPI_PROBS, save, out, s,
+                                false, width);
     // threshold: each pattern summed in a fixed order by one warp, during the
     // final layer's walk (tables) or from the stored a_n (no tables)
-    if (p->tab.enabled) return launch_layer_fwd(p, Ly, ws, Ud, batch, n, EPI_THRESH, save, out, s);
+    if (p->tab.enabled) return launch_layer_fwd(p, Ly, ws, Ud, batch, n, EPI_THRESH, save, out, s, false, width);
     slos_status_t st = launch_layer_fwd(p, Ly, ws, Ud, batch, n, EPI_STORE, true, nullptr, s);
     if (st != SLOS_OK) return st;
     ThreshArgs ta;

@@ -22,8 +22,9 @@ struct PrefixArgs {
     const int32_t *ctab[kMaxPhotons + 1];     // child table of layer k: [F_{k-1}][m], rank of t' + e_j
     int F[kMaxPhotons + 1];
     int cols[kMaxPhotons];                    // input mode of photon k (ascending)
-    // forward: layer k <= L is written to out[k] (group layout [NG][F_k][32]) when non-null
+    // forward: layer k <= L is written to out[k] (group layout [groups][F_k][lanes]) when non-null
     float2 *out[kMaxPhotons + 1];
+    int lanes;                                // instances per group of out (NI divides it, or is it)
     // backward: G_L (group layout) in, the dU partial row of each layer k <= L out
     const float2 *GL;
     float2 *dUpart[kMaxPhotons + 1];          // [NG][1][32][m] of layer k

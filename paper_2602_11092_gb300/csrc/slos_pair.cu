@@ -307,8 +307,8 @@ __global__ void __launch_bounds__(kPairThreads, kPairMinBlocks) slos_fwd_pair_ke
                     const float w = __shfl_sync(0xffffffffu, wl, ci);
                     const int r0 = (32 * h + 2 * sl) * (TS + 1) + h;  // tile word of instance 2 sl, state 0
                     if (EPI == EPI_PROBS) {
-                        tile[r0 + (ci & (TS - 1))] = w * (acc0.x * acc0.x + acc0.y * acc0.y);
-                        tile[r0 + (TS + 1) + (ci & (TS - 1))] = w * (acc1.x * acc1.x + acc1.y * acc1.y);
+                        tile[r0 + (ci & (TS - 1))] = w * cabs2(acc0);
+                        tile[r0 + (TS + 1) + (ci & (TS - 1))] = w * cabs2(acc1);
                     } else if (EPI == EPI_AMPS) {
                         const float sw = sqrtf(w);
                         reinterpret_cast<float2 *>(tile)[r0 + (ci & (TS - 1))] = cscale(acc0, sw);
@@ -321,8 +321,8 @@ __global__ void __launch_bounds__(kPairThreads, kPairMinBlocks) slos_fwd_pair_ke
                             run_pat = pat;
                             run0 = run1 = 0.f;
                         }
-                        run0 += w * (acc0.x * acc0.x + acc0.y * acc0.y);
-                        run1 += w * (acc1.x * acc1.x + acc1.y * acc1.y);
+                        run0 = __fmaf_rn(w, cabs2(acc0), run0);
+                        run1 = __fmaf_rn(w, cabs2(acc1), run1);
                     }
                 }
                 // a full tile (or the chunk's last states) goes out: TS consecutive

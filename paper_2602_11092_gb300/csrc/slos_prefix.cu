@@ -114,7 +114,7 @@ __device__ __forceinline__ void prefix_layer(const PrefixArgs &a, int k, const f
                 for (int q = 0; q < KW; ++q) acc = cfma(u[e[q] & 31u], pv[e[q] >> 5], acc);
             }
             cur[(size_t)i * capc + c] = acc;
-            if (gout) gout[(size_t)c * kLanes + i] = acc;
+            if (gout) gout[(size_t)c * a.lanes + i] = acc;
         }
     }
 }
@@ -137,11 +137,11 @@ __global__ void __launch_bounds__(kPrefixThreads, 2) slos_fwd_prefix_kernel(Pref
     buf[1] = buf[0] + (size_t)NI * a.cap[0];
     const int inst0 = blockIdx.x * NI;
     const int ni = min(NI, a.B - inst0);
-    const int grp = inst0 / kLanes, l0 = inst0 % kLanes;
+    const int grp = inst0 / a.lanes, l0 = inst0 % a.lanes;
     prefix_stage_u(a, us, inst0, ni);
     __syncthreads();
     for (int k = 1; k <= a.L; ++k) {
-        float2 *gout = a.out[k] ? a.out[k] + ((size_t)grp * a.F[k]) * kLanes + l0 : nullptr;
+        float2 *gout = a.out[k] ? a.out[k] + ((size_t)grp * a.F[k]) * a.lanes + l0 : nullptr;
         prefix_layer_kw(a, k, us, buf[(k - 1) & 1], a.cap[(k - 1) & 1], buf[k & 1], a.cap[k & 1], ni, gout);
         __syncthreads();
     }
@@ -279,7 +279,7 @@ static size_t prefix_smem_args(const PrefixArgs &a, bool bwd) {
 
 cudaError_t slos_launch_prefix_fwd(const PrefixArgs &a, cudaStream_t s) {
     const size_t sm = prefix_smem_args(a, false);
-    if (sm > kPrefixSmemLimit || a.NI < 1 || kLanes % a.NI != 0) return cudaErrorInvalidValue;
+    if (sm > kPrefixSmemLimit || a.NI < 1 || a.lanes % a.NI != 0) return cudaErrorInvalidValue;
     slos_fwd_prefix_kernel<<<(a.B + a.NI - 1) / a.NI, kPrefixThreads, sm, s>>>(a);
     return cudaGetLastError();
 }

@@ -32,4 +32,9 @@ int slos_pair_warps();
 int slos_pair_chunk();
 cudaError_t slos_launch_fwd_pair(const FwdArgs &a, const TabArgs &t, int epi, bool save, int blocks, cudaStream_t s);
 
+// Inference, lane = state: layer k of a group of `width` (1, 2 or 4) instances
+// as complex64 [F_k][width] (slos_narrow.cu; abi.cu's narrow_width says when).
+int slos_narrow_width(int batch);
+cudaError_t slos_launch_fwd_narrow(const FwdArgs &a, const TabArgs &t, int epi, int width, cudaStream_t s);
+
 }  // namespace slos

@@ -327,6 +327,28 @@ def test_on_chip_forward_matches_layered_forward(slos, m, s, B):
         assert np.abs(p[b] - oracle.probabilities(Uh[b], s, outs)).max() <= P_TOL
 
 
+@pytest.mark.parametrize("m,s,det,space,B", [
+    (16, [1, 0] * 7 + [0, 0], 0, 0, 1), (13, [1] * 7 + [0] * 6, 0, 0, 2), (14, [1, 0] * 7, 0, 0, 3),
+    (20, [1, 0] * 5 + [0] * 10, 0, 0, 18), (24, [3, 1] + [0] * 22, 1, 0, 1), (9, [5, 5, 2] + [0] * 6, 1, 0, 2),
+    (16, [1, 0] * 6 + [0] * 4, 1, 0, 100), (7, [1, 1, 0, 1, 0, 0, 0], 1, 0, 333), (12, [1, 0] * 6, 0, 0, 1),
+    (12, [1, 0] * 6, 0, 0, 190), (12, [1, 0] * 6, 0, 0, 191), (10, [1, 0] * 5, 0, 0, 4), (16, [1, 0] * 6 + [0] * 4, 0, 1, 5),
+    (2, [7, 5], 1, 0, 5), (3, [1, 0, 0], 1, 0, 1)])
+def test_lane_per_state_forward_matches_layered_forward(slos, m, s, det, space, B):
+    """Inference of small and middling batches (groups of 1, 2 and 4
+    instances, ragged last groups; 4-, 8- and 12-slot rows; patterns of one
+    state and of hundreds; either side of the lines to the other kernels)
+    against the layered forward that keeps its activations."""
+    rng = np.random.default_rng(m * 13 + B)
+    U = c64(workloads.haar_unitaries(m, B, rng))
+    plan = slos.Plan(m, s, det, space=space)
+    for out_kind in (slos.PROBS, slos.AMPS) if det == 0 else (slos.PROBS,):
+        got = plan.forward(U, out_kind)
+        ref = plan.forward(U, out_kind, save_for_backward=True, workspace=plan.workspace(B, training=True))
+        # the same sums in the same order, up to the order of a pattern's states
+        assert torch.allclose(got, ref, atol=1e-7, rtol=0)
+        assert torch.equal(got, plan.forward(U, out_kind))
+
+
 def test_empty_batch_is_noop(slos):
     plan = slos.Plan(4, [1, 1, 0, 0])
     U = torch.empty((0, 4, 4), dtype=torch.complex64, device=dev())
