@@ -2,29 +2,33 @@
 // persistent kernel launch (graph-capturable), with launch shapes picked by
 // an autotuner.
 //
-// Instances with the same shape are packed 16 per "lane group", a shape's
-// remaining instances in groups of 8 and 4 (9..12 left: 8 + 4); a warp serves one lane group
-// and walks 32 / width Fock states at a time (part p of the warp takes every
-// (32 / width)-th state, lane % width is the instance), so the ~14 instances
-// a shape typically has in a 1024-instance batch fill most lanes and a shape
-// with a few instances does not walk idle lanes' rows.  Layer k of a lane
-// group lives in workspace as complex64 [F_k][width].  Each shape's
+// Instances with the same shape are packed 4 per "lane group"; layer k of a lane
+// group lives in workspace as complex64 [F_k][4], a 32-byte sector per state.
+// A warp serves one lane group with lane = state: a lane sums its state for the
+// group's four instances, so a warp has 32 states' parent rows in flight, the
+// slot decode is paid once for four instances and outputs leave coalesced.
+// (With lane = instance, 16-, 8- and 4-wide groups and 2 to 8 states per warp
+// step, the 1024-instance batch took 6.9 ms at the default launch shape and
+// 5.1 ms tuned: a step had too few bytes in flight for the gathers of the
+// largest shapes, which miss L2.  4.7 ms now, untuned.)  Each shape's
 // transition graph is built once on the GPU at plan time as parent slots:
 // slot = (parent position << 5) | j for every mode j with t_j > 0, padded
 // with a slot that reads a zero row of U (Sec. II-A.3: the transitions
 // depend only on the input state).  A state with q occupied modes has q
 // parents, so each layer (but a PNR output layer, kept in Fock order for
-// the output) is stored with its states sorted, stably, by q rounded up to
-// even: a section of rows 2, 4, ..., 12 slots wide, so that no state pays
-// for the widest one.  A layer's "position" of a state is its place in that
-// order; the next layer's slots use positions.  Under threshold detection
-// the final layer's positions are its pattern-grouped list order instead
-// (patterns in output order, a pattern's states consecutive; it agrees with
-// the sections, since the patterns come by increasing |b|), and a work item
-// of that layer is a run of whole patterns, so one warp sums each pattern in
-// a fixed order and stores it once.  A final state's weight
+// the output) is stored by pattern: its states grouped by their set of
+// occupied modes, the sets by size q, then colex, a set's states consecutive.
+// The sets of one size form a section with rows of q slots (rounded up to
+// even), so that no state pays for the widest one, and the parents of a set's
+// states lie in q + 1 runs of consecutive rows (the same set one photon down,
+// and the set less each mode), which neighbouring lanes share in L1 (1024
+// instances: 6.25 ms with sections in Fock order).  A layer's "position" of a
+// state is its place in that order; the next layer's slots use positions.
+// Under threshold detection that is the order of the outcomes, and a work item
+// of the final layer is a run of whole patterns, so one warp sums each pattern
+// in a fixed order and stores it once.  A final state's weight
 // prod t_j! / prod s_i! is a per-position table built with the slots.
-// Work item = (lane group, layer k, chunk of consecutive Fock states).  Items are listed layer by
+// Work item = (lane group, layer k, chunk of consecutive positions).  Items are listed layer by
 // layer (all layer-1 items of every lane group, then all layer-2 items, ...),
 // largest lane groups first inside a layer (longest-processing-time order).
 // Warps pop items in that order with one atomic counter; an item of layer
@@ -55,7 +59,7 @@ namespace slos {
 slos_status_t fail(slos_status_t st, const std::string &msg);
 
 constexpr int kBMax = 20;   // modes handled by the persistent kernel (m <= 20)
-constexpr int kBLanes = 16; // instances per lane group
+constexpr int kBInst = 4;   // instances per lane group
 constexpr uint32_t kSlotEmpty = (uint32_t)kBMax;   // parent 0, mode kBMax (a zero row of U)
 constexpr int64_t kBMaxParent = int64_t(1) << 27;  // parent ranks in 27 bits
 constexpr int kBSec = 12;   // one section per occupied-mode count 1..12
@@ -77,6 +81,7 @@ struct BShape {
     // s = kw - 1 (rows of kw slots, all of them walked).
     int sec_pos[kMaxPhotons + 1][kBSec + 1];
     int64_t sec_off[kMaxPhotons + 1][kBSec];
+    bool sorted[kMaxPhotons + 1];       // layer k is stored in sections (else Fock order)
     float inv_sfact;
     int nclass;                         // threshold: pattern classes j = 1 .. min(n, m)
     int pat_off[kMaxPhotons + 2];       // first pattern index with j occupied modes
@@ -86,8 +91,7 @@ struct BShape {
 
 struct BLaneGroup {
     int shape;
-    int width;            // instances per lane group: 16, 8 or 4 (a shape's remainder after the 16s)
-    int inst[kBLanes];    // global instance index per lane, -1 = empty lane
+    int inst[kBInst];     // global instance index, -1 = none
     int64_t buf[2];       // workspace byte offsets of the two layer buffers
 };
 
@@ -118,69 +122,19 @@ struct BArgs {
     long long spin_limit;
 };
 
-// Occupied modes of state c of layer k (descending-lex rank, bar unranking
-// of common.cuh) and the section it goes to: q - 1.
-template <int MMAX>
-__device__ __forceinline__ int state_section(const BShape &sh, int k, int64_t c) {
-    const int m = sh.m, L = k + m - 1;
-    int p[MMAX];
-    unrank_bars<MMAX>(c, m, L, p);
-    int q = 0;
-#pragma unroll
-    for (int j = 0; j < MMAX; ++j)
-        if (j < m && occupation<MMAX>(j, m, L, p) > 0) ++q;
-    return q - 1;
-}
-
-// Stable partition of layer k by section, in two passes over blocks of 256
-// consecutive states: (1) cnt[blk][s] = states of block blk in section s;
-// (2) pos[c] = base[blk][s] + rank of c among the block's states of its
-// section, base being the section start plus the counts of earlier blocks
-// (an exclusive scan the host does between the passes).
-template <int MMAX>
-__global__ void __launch_bounds__(256) section_pass_kernel(const BShape sh, int k, int *cnt, const int *base,
-                                                            int *pos) {
-    __shared__ int wcnt[8][kBSec];
-    const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int sec = c < sh.F[k] ? state_section<MMAX>(sh, k, c) : -1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int wrank = 0;
-#pragma unroll
-    for (int q = 0; q < kBSec; ++q) {
-        const unsigned bal = __ballot_sync(0xffffffffu, sec == q);
-        if (sec == q) wrank = __popc(bal & ((1u << lane) - 1u));
-        if (lane == 0) wcnt[warp][q] = __popc(bal);
-    }
-    __syncthreads();
-    if (!pos) {
-        if (threadIdx.x < kBSec) {
-            int t = 0;
-            for (int w = 0; w < 8; ++w) t += wcnt[w][threadIdx.x];
-            cnt[(size_t)blockIdx.x * kBSec + threadIdx.x] = t;
-        }
-        return;
-    }
-    if (sec < 0) return;
-    int r = wrank;
-    for (int w = 0; w < warp; ++w) r += wcnt[w][sec];
-    pos[c] = base[(size_t)blockIdx.x * kBSec + sec] + r;
-}
-
 // Tables of layer k of one shape, one thread per state, with the index
 // arithmetic of the single-shape kernels (common.cuh): the row of state c
-// (at position cpos[c], or c in an unsorted layer) holds
+// holds
 //   (position of t - e_j in layer k-1 << 5) | j
 // for the occupied modes j of t in mode order, then padding; ppos maps the
-// parent layer's ranks to positions (null: unsorted).  For the final layer
-// also w[position] = prod t_j! / prod s_i!.  With `listed` (the final layer
-// of a threshold shape) the position is the state's place in the
-// pattern-grouped list: patterns in output order (|b|, then colex), and
-// inside a pattern the states t with support b in descending-lex order of
-// t - 1_b, a composition of n - |b| photons over |b| modes, ranked with the
-// same bar formula.
+// parent layer's ranks to positions (null: Fock order).  For the final layer
+// also w[position] = prod t_j! / prod s_i!.  In a sorted layer the position is
+// the state's place in the pattern-grouped list: patterns by |b|, then colex,
+// and inside a pattern the states t with support b in descending-lex order of
+// t - 1_b, a composition of k - |b| photons over |b| modes, ranked with the
+// same bar formula; it goes to cpos[c].
 template <int MMAX>
-__global__ void build_slots_kernel(const BShape sh, int k, uint32_t *tab, const int *ppos, const int *cpos,
-                                   float *w, bool listed) {
+__global__ void build_slots_kernel(const BShape sh, int k, uint32_t *tab, const int *ppos, int *cpos, float *w) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= sh.F[k]) return;
     const int m = sh.m;
@@ -210,7 +164,7 @@ __global__ void build_slots_kernel(const BShape sh, int k, uint32_t *tab, const 
     }
     const int nb = q;
     int64_t at = c;
-    if (listed) {
+    if (sh.sorted[k]) {
         const int np = k - nb, Lp = np + nb - 1;
         int64_t r = 0;
         int cum = 0;
@@ -218,13 +172,12 @@ __global__ void build_slots_kernel(const BShape sh, int k, uint32_t *tab, const 
             cum += tb[b] - 1;
             r += (int64_t)binom(Lp - 1 - b - cum, nb - 1 - b);
         }
-        at = sh.pat_base[nb] + (int64_t)colex_rank(supp) * sh.pat_cnt[nb] + r;
-    } else if (cpos) {
-        at = cpos[c];
+        at = sh.sec_pos[k][nb - 1] + (int64_t)colex_rank(supp) * binom(k - 1, nb - 1) + r;
+        if (cpos) cpos[c] = (int)at;
     }
     uint32_t *dst;
     int width;
-    if (cpos || listed) {
+    if (sh.sorted[k]) {
         const int sec = nb - 1;
         width = sec_width(sec);
         dst = tab + sh.sec_off[k][sec] + (at - sh.sec_pos[k][sec]) * width;
@@ -243,199 +196,152 @@ __device__ __forceinline__ int ld_acquire(const int *p) {
     return v;
 }
 
-// Slot rows of up to kBStage consecutive positions are staged per warp in
-// shared memory by one coalesced warp-wide copy, so a walk step waits for
-// one global round trip (its parent rows) instead of two (slot row, then
-// parent rows).
-constexpr int kBStage = 32;
-constexpr int kBSlotWords = kBStage * 12;                     // widest rows: 12 slots
-constexpr int kBWarpF2 = (kBMax + 1) * kBLanes + kBSlotWords;  // per warp: U column, two staging buffers (float2 units)
+constexpr int kBWarpF2 = (kBMax + 1) * kBInst;  // per warp: U column of the group's instances, a zero row
 
-__device__ __forceinline__ void b_cp4(uint32_t *dst, const uint32_t *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
-                 "l"(src)
-                 : "memory");
-}
-template <int N>
-__device__ __forceinline__ void b_cp_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+__device__ __forceinline__ void add_release(int *p) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
 }
 
-// The slot rows of positions [start, start + n) into dst, as one cp.async group.
-__device__ __forceinline__ void stage_issue(const uint32_t *__restrict__ tab, int pos0, int KW, int start, int n,
-                                            uint32_t *dst, int lane) {
-    const uint32_t *src = tab + (size_t)(start - pos0) * KW;
-    for (int i = lane; i < n * KW; i += 32) b_cp4(dst + i, src + i);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-// Walk of nwin windows of consecutive positions (win(i, start, n) gives window
-// i), each one's slot rows staged in one of the warp's two buffers while the
-// previous window is walked: proc(i, start, n, rows) runs once the rows are in.
-template <typename Win, typename Proc>
-__device__ __forceinline__ void staged_walk(int nwin, Win win, Proc proc, const uint32_t *__restrict__ tab, int pos0,
-                                            int KW, uint32_t *sbuf, int lane) {
-    if (nwin <= 0) return;
-    int s0, n0;
-    win(0, s0, n0);
-    __syncwarp();
-    stage_issue(tab, pos0, KW, s0, n0, sbuf, lane);
-    for (int i = 0; i < nwin; ++i) {
-        int s, n;
-        win(i, s, n);
-        if (i + 1 < nwin) {
-            int s1, n1;
-            win(i + 1, s1, n1);
-            stage_issue(tab, pos0, KW, s1, n1, sbuf + ((i + 1) & 1) * kBSlotWords, lane);
-            b_cp_wait<1>();
-        } else {
-            b_cp_wait<0>();
-        }
-        __syncwarp();  // every lane's copies of window i are in
-        proc(i, s, n, sbuf + (i & 1) * kBSlotWords);
-        __syncwarp();  // window i read before its buffer takes window i + 2
-    }
-}
-
-// Amplitude of one state from its staged slot row srow (KW slots, the first
-// QV of them occupied) for the lane's instance.  us: this warp's staged
-// column of U, row j = U[j][col] per lane (row kBMax zero); prev: layer k-1
-// of this lane (rows of LW complex64).  Parent rows are plain (L1-cached)
-// loads: the wait on layer k-1's completion counter has ordered them after
-// its writes.
-template <int KW, int QV, int LW>
-__device__ __forceinline__ float2 b_state_amp(const uint32_t *srow, const float2 *us, const char *prev,
-                                              bool first_layer) {
+// Amplitudes of one state for the lane group's instances: row = its slots, Q
+// of them (PAD: some may be padding, which reads no parent).  us: this warp's
+// staged column of U; prev: layer k-1 of the group.  Parent rows are plain
+// (L1-cached) loads: the wait on layer k-1's completion counter has ordered
+// them after its writes.
+template <int Q, bool PAD>
+__device__ __forceinline__ void b_state(const uint32_t *__restrict__ row, const float2 *us, const float2 *prev,
+                                        bool first_layer, float2 (&acc)[kBInst]) {
+    constexpr int KW = (Q + 1) & ~1;  // rows of an even number of slots: 8-byte aligned
     uint32_t e[KW];
-    const uint2 *s2 = reinterpret_cast<const uint2 *>(srow);  // rows of an even number of slots: 8-byte aligned
 #pragma unroll
     for (int q2 = 0; q2 < KW / 2; ++q2) {
-        const uint2 w2 = s2[q2];
+        const uint2 w2 = __ldg(reinterpret_cast<const uint2 *>(row) + q2);
         e[2 * q2] = w2.x;
         e[2 * q2 + 1] = w2.y;
     }
-    if (first_layer) return us[(e[0] & 31u) * kBLanes];  // one photon: a_1(e_j) = U[j][col]
-    float2 v[QV];
-    // parent position (e >> 5) times the row of LW complex64
+    auto column = [&](uint32_t slot, float4 &u0, float4 &u1) {
+        const float4 *u = reinterpret_cast<const float4 *>(us) + (slot & 31u) * (kBInst / 2);
+        u0 = u[0];
+        u1 = u[1];
+    };
+    float4 u0, u1;
+    if (first_layer) {
+        column(e[0], u0, u1);  // one photon: a_1(e_j) = U[j][col]
+        acc[0] = make_float2(u0.x, u0.y);
+        acc[1] = make_float2(u0.z, u0.w);
+        acc[2] = make_float2(u1.x, u1.y);
+        acc[3] = make_float2(u1.z, u1.w);
+        return;
+    }
 #pragma unroll
-    for (int q = 0; q < QV; ++q)
-        v[q] = *reinterpret_cast<const float2 *>(prev + (size_t)(e[q] & ~31u) * (LW / 4));
-    float2 acc = make_float2(0.f, 0.f);
+    for (int i = 0; i < kBInst; ++i) acc[i] = make_float2(0.f, 0.f);
+    // parent rows in two batches of at most 6, so that their registers leave room for resident warps
 #pragma unroll
-    for (int q = 0; q < QV; ++q) acc = cfma(us[(e[q] & 31u) * kBLanes], v[q], acc);
-    return acc;
+    for (int h = 0; h < Q; h += 6) {
+        float4 v[6][2];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            if (h + q < Q) {
+                const float4 *r = reinterpret_cast<const float4 *>(prev) + (size_t)(e[h + q] >> 5) * (kBInst / 2);
+                if (!PAD || e[h + q] != kSlotEmpty) {
+                    v[q][0] = r[0];
+                    v[q][1] = r[1];
+                } else {
+                    v[q][0] = v[q][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            if (h + q < Q) {
+                column(e[h + q], u0, u1);
+                acc[0] = cfma(make_float2(u0.x, u0.y), make_float2(v[q][0].x, v[q][0].y), acc[0]);
+                acc[1] = cfma(make_float2(u0.z, u0.w), make_float2(v[q][0].z, v[q][0].w), acc[1]);
+                acc[2] = cfma(make_float2(u1.x, u1.y), make_float2(v[q][1].x, v[q][1].y), acc[2]);
+                acc[3] = cfma(make_float2(u1.z, u1.w), make_float2(v[q][1].z, v[q][1].w), acc[3]);
+            }
+        }
+    }
 }
 
-// Positions c0 + part, c0 + part + P, ... < c1 of one section (P = 32 / LW
-// parts of the warp, lane il of each part = instance il of the lane group):
-// the next layer's amplitudes, or the PNR output probabilities (Fock order).
-// Windows of kBStage positions (a multiple of P, so each part keeps its
-// positions).
-template <int KW, int QV, int LW>
-__device__ __forceinline__ void fwd_states(const uint32_t *__restrict__ tab, int pos0, int c0, int c1, int part,
-                                           int lane, uint32_t *sbuf, const float2 *us, const char *prev,
-                                           bool first_layer, bool last, float2 *next, float *outp,
-                                           const float *__restrict__ wtab) {
-    constexpr int P = 32 / LW;
-    // positions fit in 32 bits (at most C(31, 12) < 2^28 per layer)
-    staged_walk(
-        (c1 - c0 + kBStage - 1) / kBStage,
-        [&](int i, int &st, int &nb) {
-            st = c0 + i * kBStage;
-            nb = min(kBStage, c1 - st);
-        },
-        [&](int, int cb, int nb, const uint32_t *rows) {
-            for (int c = cb + part; c < cb + nb; c += P) {
-                const float2 acc = b_state_amp<KW, QV, LW>(rows + (c - cb) * KW, us, prev, first_layer);
-                if (!last) next[(uint32_t)c * LW] = acc;
-                else if (outp) outp[c] = __ldg(wtab + c) * (acc.x * acc.x + acc.y * acc.y);
-            }
-        },
-        tab, pos0, KW, sbuf, lane);
+// Positions [c0, c1) of one section: the next layer's amplitudes, or the PNR
+// output probabilities (Fock order).
+template <int Q, bool PAD>
+__device__ __forceinline__ void fwd_states(const uint32_t *__restrict__ tab, int pos0, int c0, int c1, int lane,
+                                           const float2 *us, const float2 *prev, bool first_layer, bool last,
+                                           float2 *next, float *const (&outp)[kBInst], const float *__restrict__ wtab) {
+    constexpr int KW = (Q + 1) & ~1;
+    for (int c = c0 + lane; c < c1; c += 32) {
+        float2 acc[kBInst];
+        b_state<Q, PAD>(tab + (size_t)(c - pos0) * KW, us, prev, first_layer, acc);
+        if (!last) {
+            float4 *o = reinterpret_cast<float4 *>(next + (size_t)c * kBInst);
+            o[0] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+            o[1] = make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y);
+        } else {
+            const float w = __ldg(wtab + c);
+#pragma unroll
+            for (int i = 0; i < kBInst; ++i)
+                if (outp[i]) outp[i][c] = w * cabs2(acc[i]);
+        }
+    }
 }
 
 // Threshold detection, final layer in list order: patterns [P0, P1) of
 // class j (cnt states each, the first at list position base), whose output
-// indices start at pat_first.  Each pattern's probability is one sum in
-// list order: with one state per pattern the parts of the warp take
-// patterns in turn; otherwise they take the states of each pattern in turn
-// (part p: states p, p + P, ... of the pattern) and add their partial sums
-// (lanes il, il + LW, ... in a fixed order).  The sum does not depend on the
-// launch shape or on how the slot rows are staged: windows of whole patterns
-// (cnt <= kBStage) or, for larger patterns, pieces of kBStage states, which
-// keep each part's states and their order.
-template <int KW, int QV, int LW>
+// indices start at pat_first.  The warp walks windows of 32 positions aligned
+// to multiples of 32 of the list; inside a window a pattern's states are
+// added by a segmented scan over the lanes, and a pattern that spans windows
+// carries its sum along.  Windows and scan depend on list positions only, so
+// an output does not depend on the launch shape.
+template <int Q>
 __device__ __forceinline__ void thresh_patterns(const uint32_t *__restrict__ tab, int pos0, int64_t base, int cnt,
-                                                int64_t P0, int64_t P1, int pat_first, int part, int lane,
-                                                uint32_t *sbuf, const float2 *us, const char *prev, bool first_layer,
-                                                float *outp, const float *__restrict__ wtab) {
-    constexpr int P = 32 / LW;
-    auto combine_store = [&](float sum, int64_t Q) {
-        if (P == 8) sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-        if (P >= 4) sum += __shfl_xor_sync(0xffffffffu, sum, 8);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 16);
-        if (part == 0 && outp) outp[pat_first + Q] = sum;
-    };
-    if (cnt == 1) {
-        const int q0 = (int)(base + P0), q1 = (int)(base + P1);
-        staged_walk(
-            (q1 - q0 + kBStage - 1) / kBStage,
-            [&](int i, int &st, int &nb) {
-                st = q0 + i * kBStage;
-                nb = min(kBStage, q1 - st);
-            },
-            [&](int, int cb, int nb, const uint32_t *rows) {
-                for (int c = cb + part; c < cb + nb; c += P) {
-                    const float2 acc = b_state_amp<KW, QV, LW>(rows + (c - cb) * KW, us, prev, first_layer);
-                    if (outp) outp[pat_first + (c - base)] = __ldg(wtab + c) * (acc.x * acc.x + acc.y * acc.y);
+                                                int64_t P0, int64_t P1, int pat_first, int lane, const float2 *us,
+                                                const float2 *prev, bool first_layer,
+                                                float *const (&outp)[kBInst], const float *__restrict__ wtab) {
+    constexpr int KW = (Q + 1) & ~1;
+    const int q0 = (int)(base + P0 * cnt), q1 = (int)(base + P1 * cnt);
+    float carry[kBInst];
+#pragma unroll
+    for (int i = 0; i < kBInst; ++i) carry[i] = 0.f;
+    for (int win = q0 & ~31; win < q1; win += 32) {
+        const int c = win + lane;
+        const bool mine = c >= q0 && c < q1;
+        float v[kBInst];
+#pragma unroll
+        for (int i = 0; i < kBInst; ++i) v[i] = 0.f;
+        // the state's pattern, its first and last lane in this window
+        const int pat = mine ? (c - (int)base) / cnt : 0;
+        const int first = mine ? (int)base + pat * cnt : c;
+        if (mine) {
+            float2 acc[kBInst];
+            b_state<Q, false>(tab + (size_t)(c - pos0) * KW, us, prev, first_layer, acc);
+            const float w = __ldg(wtab + c);
+#pragma unroll
+            for (int i = 0; i < kBInst; ++i) v[i] = w * cabs2(acc[i]);
+        }
+        if (cnt > 1) {
+            const int start = max(first - win, 0);  // first lane of the state's pattern
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+                for (int i = 0; i < kBInst; ++i) {
+                    const float up = __shfl_up_sync(0xffffffffu, v[i], o);
+                    if (lane - o >= start) v[i] += up;
                 }
-            },
-            tab, pos0, KW, sbuf, lane);
-        return;
-    }
-    if (cnt <= kBStage) {
-        const int per = kBStage / cnt;  // whole patterns per window
-        staged_walk(
-            (int)((P1 - P0 + per - 1) / per),
-            [&](int i, int &st, int &nb) {
-                const int64_t Qw = P0 + (int64_t)i * per;
-                st = (int)(base + Qw * cnt);
-                nb = (int)min((int64_t)per, P1 - Qw) * cnt;
-            },
-            [&](int i, int cw, int nb, const uint32_t *rows) {
-                const int64_t Qw = P0 + (int64_t)i * per;
-                for (int64_t Q = Qw; Q < Qw + nb / cnt; ++Q) {
-                    const int c0 = (int)(base + Q * cnt);
-                    float sum = 0.f;
-                    for (int c = c0 + part; c < c0 + cnt; c += P) {
-                        const float2 acc = b_state_amp<KW, QV, LW>(rows + (c - cw) * KW, us, prev, first_layer);
-                        sum += __ldg(wtab + c) * (acc.x * acc.x + acc.y * acc.y);
-                    }
-                    combine_store(sum, Q);
-                }
-            },
-            tab, pos0, KW, sbuf, lane);
-        return;
-    }
-    const int npc = (cnt + kBStage - 1) / kBStage;  // pieces per pattern
-    float sum = 0.f;
-    staged_walk(
-        (int)(P1 - P0) * npc,
-        [&](int i, int &st, int &nb) {
-            const int64_t Q = P0 + i / npc;
-            const int piece = (i % npc) * kBStage;
-            st = (int)(base + Q * cnt) + piece;
-            nb = min(kBStage, cnt - piece);
-        },
-        [&](int i, int cs, int nb, const uint32_t *rows) {
-            if (i % npc == 0) sum = 0.f;
-            for (int c = cs + part; c < cs + nb; c += P) {
-                const float2 acc = b_state_amp<KW, QV, LW>(rows + (c - cs) * KW, us, prev, first_layer);
-                sum += __ldg(wtab + c) * (acc.x * acc.x + acc.y * acc.y);
             }
-            if (i % npc == npc - 1) combine_store(sum, P0 + i / npc);
-        },
-        tab, pos0, KW, sbuf, lane);
+            if (first < win) {
+#pragma unroll
+                for (int i = 0; i < kBInst; ++i) v[i] += carry[i];
+            }
+#pragma unroll
+            for (int i = 0; i < kBInst; ++i) carry[i] = __shfl_sync(0xffffffffu, v[i], 31);
+        }
+        if (mine && c == first + cnt - 1) {
+#pragma unroll
+            for (int i = 0; i < kBInst; ++i)
+                if (outp[i]) outp[i][pat_first + pat] = v[i];
+        }
+    }
 }
 
 // Work items of class j of a threshold final layer: runs of whole patterns
@@ -449,29 +355,25 @@ __host__ __device__ __forceinline__ int64_t thresh_items(const BShape &sh, int j
     return (npat + thresh_per_item(sh, j, chunk) - 1) / thresh_per_item(sh, j, chunk);
 }
 
-// One work item of lane group g (LW = its width: 16 or 8 instances): layer
-// k's positions of the item's section, or (threshold final layer) its run of
-// whole patterns.  The warp's 32 / LW parts take positions in turn; lane il
-// of each part is instance il of the lane group.
-template <int LW>
+// One work item of lane group g: layer k's positions of the item's section, or
+// (threshold final layer) its run of whole patterns.
 __device__ __forceinline__ void b_item(const BArgs &a, const BLaneGroup &g, const BShape &sh, int k, int64_t chunk_id,
-                                       int lane, float2 *us, uint32_t *sbuf) {
-    constexpr int P = 32 / LW;
-    const int part = lane / LW, il = lane % LW;
+                                       int lane, float2 *us) {
     const int n = sh.n;
-    const int inst = g.inst[il];
-    const bool valid = inst >= 0;
-    float *outp = valid ? a.out + a.out_off[inst] : nullptr;
     const int m = sh.m;
     const int col = sh.cols[k - 1];
+    float *outp[kBInst];
+#pragma unroll
+    for (int i = 0; i < kBInst; ++i) outp[i] = g.inst[i] >= 0 ? a.out + a.out_off[g.inst[i]] : nullptr;
     __syncwarp();
-    for (int j = part; j < m; j += P)
-        us[j * kBLanes + il] = valid ? a.U[a.u_off[inst] + (int64_t)j * m + col] : make_float2(0.f, 0.f);
+    for (int x = lane; x < m * kBInst; x += 32) {
+        const int inst = g.inst[x % kBInst];
+        us[x] = inst >= 0 ? a.U[a.u_off[inst] + (int64_t)(x / kBInst) * m + col] : make_float2(0.f, 0.f);
+    }
     __syncwarp();
-    const char *prev = a.ws + g.buf[(n - 1 - (k - 1)) & 1] + il * sizeof(float2);
+    const float2 *prev = reinterpret_cast<const float2 *>(a.ws + g.buf[(n - 1 - (k - 1)) & 1]);
     const uint32_t *tab = a.slots + sh.slot_off[k];
     const float *wtab = reinterpret_cast<const float *>(a.slots + sh.w_off);
-    const float2 *usl = us + il;
     if (k == n && sh.det == SLOS_DETECT_THRESHOLD) {
         // the item's class and run of patterns (items counted class by class)
         int j = 1;
@@ -487,22 +389,21 @@ __device__ __forceinline__ void b_item(const BArgs &a, const BLaneGroup &g, cons
         const int sec = j - 1;
         const int p0 = sh.sec_pos[k][sec];
         const uint32_t *st = tab + sh.sec_off[k][sec];
-#define SLOS_B_THR(W, Q)                                                                                         \
-    thresh_patterns<W, Q, LW>(st, p0, sh.pat_base[j], sh.pat_cnt[j], P0, P1, sh.pat_off[j], part, lane, sbuf, usl, \
-                              prev, k == 1, outp, wtab)
+#define SLOS_B_THR(Q)                                                                                              \
+    thresh_patterns<Q>(st, p0, sh.pat_base[j], sh.pat_cnt[j], P0, P1, sh.pat_off[j], lane, us, prev, k == 1, outp, wtab)
         switch (sec) {
-            case 0: SLOS_B_THR(2, 1); break;
-            case 1: SLOS_B_THR(2, 2); break;
-            case 2: SLOS_B_THR(4, 3); break;
-            case 3: SLOS_B_THR(4, 4); break;
-            case 4: SLOS_B_THR(6, 5); break;
-            case 5: SLOS_B_THR(6, 6); break;
-            case 6: SLOS_B_THR(8, 7); break;
-            case 7: SLOS_B_THR(8, 8); break;
-            case 8: SLOS_B_THR(10, 9); break;
-            case 9: SLOS_B_THR(10, 10); break;
-            case 10: SLOS_B_THR(12, 11); break;
-            default: SLOS_B_THR(12, 12); break;
+            case 0: SLOS_B_THR(1); break;
+            case 1: SLOS_B_THR(2); break;
+            case 2: SLOS_B_THR(3); break;
+            case 3: SLOS_B_THR(4); break;
+            case 4: SLOS_B_THR(5); break;
+            case 5: SLOS_B_THR(6); break;
+            case 6: SLOS_B_THR(7); break;
+            case 7: SLOS_B_THR(8); break;
+            case 8: SLOS_B_THR(9); break;
+            case 9: SLOS_B_THR(10); break;
+            case 10: SLOS_B_THR(11); break;
+            default: SLOS_B_THR(12); break;
         }
 #undef SLOS_B_THR
     } else {
@@ -518,23 +419,34 @@ __device__ __forceinline__ void b_item(const BArgs &a, const BLaneGroup &g, cons
         const int p0 = sh.sec_pos[k][sec];
         const int c0 = p0 + (int)rem * a.chunk;
         const int c1 = min(c0 + a.chunk, sh.sec_pos[k][sec + 1]);
-        float2 *next = reinterpret_cast<float2 *>(a.ws + g.buf[(n - 1 - k) & 1]) + il;
+        float2 *next = reinterpret_cast<float2 *>(a.ws + g.buf[(n - 1 - k) & 1]);
         const uint32_t *st = tab + sh.sec_off[k][sec];
-#define SLOS_B_SEC(W, Q) \
-    fwd_states<W, Q, LW>(st, p0, c0, c1, part, lane, sbuf, usl, prev, k == 1, k == n, next, outp, wtab)
+        if (!sh.sorted[k]) {
+            // Fock order: rows of kw slots, padding among them
+            switch (sh.kw[k]) {
+                case 2: fwd_states<2, true>(st, p0, c0, c1, lane, us, prev, k == 1, k == n, next, outp, wtab); break;
+                case 4: fwd_states<4, true>(st, p0, c0, c1, lane, us, prev, k == 1, k == n, next, outp, wtab); break;
+                case 6: fwd_states<6, true>(st, p0, c0, c1, lane, us, prev, k == 1, k == n, next, outp, wtab); break;
+                case 8: fwd_states<8, true>(st, p0, c0, c1, lane, us, prev, k == 1, k == n, next, outp, wtab); break;
+                case 10: fwd_states<10, true>(st, p0, c0, c1, lane, us, prev, k == 1, k == n, next, outp, wtab); break;
+                default: fwd_states<12, true>(st, p0, c0, c1, lane, us, prev, k == 1, k == n, next, outp, wtab); break;
+            }
+            return;
+        }
+#define SLOS_B_SEC(Q) fwd_states<Q, false>(st, p0, c0, c1, lane, us, prev, false, false, next, outp, wtab)
         switch (sec) {
-            case 0: SLOS_B_SEC(2, 1); break;
-            case 1: SLOS_B_SEC(2, 2); break;
-            case 2: SLOS_B_SEC(4, 3); break;
-            case 3: SLOS_B_SEC(4, 4); break;
-            case 4: SLOS_B_SEC(6, 5); break;
-            case 5: SLOS_B_SEC(6, 6); break;
-            case 6: SLOS_B_SEC(8, 7); break;
-            case 7: SLOS_B_SEC(8, 8); break;
-            case 8: SLOS_B_SEC(10, 9); break;
-            case 9: SLOS_B_SEC(10, 10); break;
-            case 10: SLOS_B_SEC(12, 11); break;
-            default: SLOS_B_SEC(12, 12); break;
+            case 0: SLOS_B_SEC(1); break;
+            case 1: SLOS_B_SEC(2); break;
+            case 2: SLOS_B_SEC(3); break;
+            case 3: SLOS_B_SEC(4); break;
+            case 4: SLOS_B_SEC(5); break;
+            case 5: SLOS_B_SEC(6); break;
+            case 6: SLOS_B_SEC(7); break;
+            case 7: SLOS_B_SEC(8); break;
+            case 8: SLOS_B_SEC(9); break;
+            case 9: SLOS_B_SEC(10); break;
+            case 10: SLOS_B_SEC(11); break;
+            default: SLOS_B_SEC(12); break;
         }
 #undef SLOS_B_SEC
     }
@@ -544,12 +456,11 @@ __device__ __forceinline__ void b_item(const BArgs &a, const BLaneGroup &g, cons
 // (a tuning dimension: fewer registers, more warps in flight).
 template <int MINB>
 __global__ void __launch_bounds__(256, MINB) slos_batched_kernel(BArgs a) {
-    extern __shared__ float2 us_all[];  // per warp: U column [kBMax + 1][16], then kBSlotWords staged slots
+    extern __shared__ float4 us_raw[];  // per warp: U column [kBMax + 1][kBInst]
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    float2 *us = us_all + warp * kBWarpF2;
-    uint32_t *sbuf = reinterpret_cast<uint32_t *>(us + (kBMax + 1) * kBLanes);
-    if (lane < kBLanes) us[kBMax * kBLanes + lane] = make_float2(0.f, 0.f);
+    float2 *us = reinterpret_cast<float2 *>(us_raw) + warp * kBWarpF2;
+    if (lane < kBInst) us[kBMax * kBInst + lane] = make_float2(0.f, 0.f);
     int lo = 0;  // descriptor of the previous item: items are handed out in increasing order
     for (;;) {
         unsigned long long q = 0;
@@ -590,15 +501,11 @@ __global__ void __launch_bounds__(256, MINB) slos_batched_kernel(BArgs a) {
             }
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
             if (!ok) return;
-            __syncwarp();
-            __threadfence();
+            __syncwarp();  // orders every lane's reads after lane 0's acquire
         }
-        if (g.width == 4) b_item<4>(a, g, sh, k, chunk_id, lane, us, sbuf);
-        else if (g.width == 8) b_item<8>(a, g, sh, k, chunk_id, lane, us, sbuf);
-        else b_item<16>(a, g, sh, k, chunk_id, lane, us, sbuf);
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) atomicAdd(a.done + lo, 1);
+        b_item(a, g, sh, k, chunk_id, lane, us);
+        __syncwarp();  // orders every lane's writes before lane 0's release
+        if (lane == 0) add_release(a.done + lo);
     }
 }
 
@@ -609,9 +516,8 @@ static bool layer_sorted(const BShape &sh, int k) { return k >= 2 && !(k == sh.n
 using BKernel = void (*)(BArgs);
 static BKernel batched_kernel(int minb) {
     switch (minb) {
-        case 4: return slos_batched_kernel<4>;
-        case 5: return slos_batched_kernel<5>;
-        default: return slos_batched_kernel<6>;
+        case 3: return slos_batched_kernel<3>;
+        default: return slos_batched_kernel<4>;
     }
 }
 
@@ -623,8 +529,8 @@ struct BatchedPlan {
     std::vector<BShape> shapes;
     std::vector<BLaneGroup> lgs;
     std::string signature;
-    // launch configuration (autotuned)
-    int chunk = 256, threads = 256, blocks_per_sm = 5, minb = 5;
+    // launch configuration (default_launch, or autotuned)
+    int chunk = 256, threads = 256, blocks_per_sm = 3, minb = 3;
     // device copies (owned)
     BShape *d_shapes = nullptr;
     BLaneGroup *d_lgs = nullptr;
@@ -716,6 +622,24 @@ static slos_status_t build_items(BatchedPlan *b, int chunk) {
     b->built_chunk = chunk;
     b->ctrl_bytes = align_up(sizeof(unsigned long long)) + align_up((size_t)b->ndesc * sizeof(int));
     return SLOS_OK;
+}
+
+// Launch shape of a plan that is not tuned: 3 blocks of 256 threads per SM (85
+// registers, no spills; 4 blocks at 64 registers measured within 2 % either
+// way), and chunks that grow with the states a resident warp has to walk: an
+// item costs a fetch, a staged U column and two synchronisations, but few
+// items leave warps idle between dependent layers.  Measured (ms at chunks of
+// 128 / 256 / 512 / 1024): 1024 instances of m 8..20 (46,000 states a warp)
+// - / 4.9 / 4.75 / 4.65; 500 of m 10..17 (2,700) - / 0.334 / 0.329 / -; 30 of
+// m 12..16 (270) 0.097 / 0.101 / 0.102 / -; 100 of m 8..14 (40) 0.047 / 0.05 / - / -.
+static void default_launch(BatchedPlan *b, int sm_count) {
+    int64_t states = 0;
+    for (const auto &g : b->lgs) {
+        const BShape &sh = b->shapes[g.shape];
+        for (int k = 1; k <= sh.n; ++k) states += sh.F[k];
+    }
+    const int64_t per_warp = states / ((int64_t)sm_count * b->blocks_per_sm * (b->threads / 32));
+    b->chunk = per_warp < 512 ? 128 : (per_warp < 2048 ? 256 : (per_warp < 16384 ? 512 : 1024));
 }
 
 static slos_status_t batched_launch(slos_plan_s *p, const void *U, float *out, void *ws, size_t ws_bytes,
@@ -902,21 +826,15 @@ slos_status_t slos_batched_plan(int count, const int *m, const int *n, const int
     size_t off = 0;
     for (size_t si = 0; si < members.size(); ++si) {
         const BShape &sh = b->shapes[si];
-        // groups of 16; the remainder r in 16-wide (r > 12), 8 + 4 (r = 9..12), 8 (r = 5..8) or 4 (r <= 4)
-        // groups, so few lanes sit idle (a group's cost is its lanes x its shape's states)
-        for (size_t q = 0; q < members[si].size();) {
+        for (size_t q = 0; q < members[si].size(); q += kBInst) {
             BLaneGroup g;
             g.shape = (int)si;
-            const size_t r = members[si].size() - q;
-            g.width = r > 12 ? kBLanes : (r > 4 ? 8 : 4);
-            for (int l = 0; l < kBLanes; ++l)
-                g.inst[l] = (l < g.width && q + l < members[si].size()) ? members[si][q + l] : -1;
-            q += g.width;
+            for (int l = 0; l < kBInst; ++l) g.inst[l] = q + l < members[si].size() ? members[si][q + l] : -1;
             const int64_t f1 = sh.n >= 2 ? sh.F[sh.n - 1] : 1;
             const int64_t f2 = sh.n >= 3 ? sh.F[sh.n - 2] : 1;
-            const size_t b1 = (size_t)f2 * g.width * sizeof(float2);
+            const size_t b1 = (size_t)f2 * kBInst * sizeof(float2);
             g.buf[0] = (int64_t)off;
-            off += align_up((size_t)f1 * g.width * sizeof(float2));
+            off += align_up((size_t)f1 * kBInst * sizeof(float2));
             g.buf[1] = (int64_t)off;
             off += align_up(b1);
             b->lgs.push_back(g);
@@ -931,7 +849,8 @@ slos_status_t slos_batched_plan(int count, const int *m, const int *n, const int
             sh.kw[k] = (std::min(sh.m, k) + 1) & ~1;
             sh.slot_off[k] = tab_elems;
             int64_t off = 0;
-            if (layer_sorted(sh, k)) {
+            sh.sorted[k] = layer_sorted(sh, k);
+            if (sh.sorted[k]) {
                 // states of layer k with q occupied modes: C(m, q) C(k-1, q-1)
                 max_sorted = std::max(max_sorted, sh.F[k]);
                 sh.sec_pos[k][0] = 0;
@@ -993,65 +912,32 @@ slos_status_t slos_batched_plan(int count, const int *m, const int *n, const int
     cudaMemcpy(b->d_ooff, b->out_off.data(), b->out_off.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
     if (cudaMalloc(&b->d_slots, (size_t)tab_elems * sizeof(uint32_t)) != cudaSuccess)
         return cleanup("slos_batched_plan: transition tables");
-    // plan-time scratch: positions of two consecutive layers, per-block section counts
-    const int64_t max_blk = (max_sorted + 255) / 256;
+    // plan-time scratch: positions of two consecutive layers
     int *d_pos[2] = {nullptr, nullptr};
-    int *d_cnt = nullptr, *d_base = nullptr;
     auto free_scratch = [&]() {
         cudaFree(d_pos[0]);
         cudaFree(d_pos[1]);
-        cudaFree(d_cnt);
-        cudaFree(d_base);
     };
-    if (max_sorted > 0 &&
-        (cudaMalloc(&d_pos[0], (size_t)max_sorted * sizeof(int)) != cudaSuccess ||
-         cudaMalloc(&d_pos[1], (size_t)max_sorted * sizeof(int)) != cudaSuccess ||
-         cudaMalloc(&d_cnt, (size_t)max_blk * kBSec * sizeof(int)) != cudaSuccess ||
-         cudaMalloc(&d_base, (size_t)max_blk * kBSec * sizeof(int)) != cudaSuccess)) {
+    if (max_sorted > 0 && (cudaMalloc(&d_pos[0], (size_t)max_sorted * sizeof(int)) != cudaSuccess ||
+                           cudaMalloc(&d_pos[1], (size_t)max_sorted * sizeof(int)) != cudaSuccess)) {
         free_scratch();
         return cleanup("slos_batched_plan: plan-time scratch");
     }
-    std::vector<int> hcnt, hbase;
     for (auto &sh : b->shapes) {
         const int *ppos = nullptr;
         for (int k = 1; k <= sh.n; ++k) {
             const int bs = 256;
             const unsigned grid = (unsigned)((sh.F[k] + bs - 1) / bs);
-            int *cpos = nullptr;
-            const bool listed = k == sh.n && sh.det == SLOS_DETECT_THRESHOLD;  // list order, no sort pass
-            if (layer_sorted(sh, k) && !listed) {
-                cpos = d_pos[k & 1];
-                section_pass_kernel<kBMax><<<grid, bs>>>(sh, k, d_cnt, nullptr, nullptr);
-                hcnt.resize((size_t)grid * kBSec);
-                hbase.resize((size_t)grid * kBSec);
-                if (cudaMemcpy(hcnt.data(), d_cnt, hcnt.size() * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) {
-                    free_scratch();
-                    return cleanup("slos_batched_plan: sorting a layer by occupied modes failed");
-                }
-                bool ok = true;
-                for (int sec = 0; sec < kBSec; ++sec) {
-                    int64_t run = sh.sec_pos[k][sec];
-                    for (unsigned blk = 0; blk < grid; ++blk) {
-                        hbase[(size_t)blk * kBSec + sec] = (int)run;
-                        run += hcnt[(size_t)blk * kBSec + sec];
-                    }
-                    ok = ok && run == sh.sec_pos[k][sec + 1];  // the closed-form section sizes
-                }
-                if (!ok) {
-                    free_scratch();
-                    return cleanup("slos_batched_plan: section sizes disagree with C(m, q) C(k-1, q-1)");
-                }
-                cudaMemcpy(d_base, hbase.data(), hbase.size() * sizeof(int), cudaMemcpyHostToDevice);
-                section_pass_kernel<kBMax><<<grid, bs>>>(sh, k, nullptr, d_base, cpos);
-            }
+            int *cpos = sh.sorted[k] && k < sh.n ? d_pos[k & 1] : nullptr;
             float *w = k == sh.n ? reinterpret_cast<float *>(b->d_slots + sh.w_off) : nullptr;
-            build_slots_kernel<kBMax><<<grid, bs>>>(sh, k, b->d_slots + sh.slot_off[k], ppos, cpos, w, listed);
+            build_slots_kernel<kBMax><<<grid, bs>>>(sh, k, b->d_slots + sh.slot_off[k], ppos, cpos, w);
             ppos = cpos;
         }
     }
     const bool built = cudaStreamSynchronize(0) == cudaSuccess && cudaGetLastError() == cudaSuccess;
     free_scratch();
     if (!built) return cleanup("slos_batched_plan: building the transition tables failed");
+    default_launch(b, p->sm_count);
     slos_status_t st = build_items(b, b->chunk);
     if (st != SLOS_OK) {
         batched_destroy(p);
@@ -1105,9 +991,9 @@ slos_status_t slos_batched_autotune(slos_plan_t p, const void *U_packed, float *
         b->minb = mb;
         return build_items(b, c);
     }
-    const int chunks[] = {128, 256, 512};
+    const int chunks[] = {128, 256, 512, 1024};
     const int thread_opts[] = {128, 256};
-    const int minb_opts[] = {4, 5, 6};
+    const int minb_opts[] = {3, 4};
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);

@@ -283,3 +283,33 @@ def test_batched_widest_slot_rows(slos):
             pos = np.sort(rng.choice(K, size=150, replace=False))
             refo = oracle.probabilities(Uq, it.s, oracle.enumerate_fock(it.m, it.n, pos))
             assert np.abs(got[pos] - refo).max() <= P_TOL
+
+
+def test_batched_groups_of_four_and_patterns_across_windows(slos):
+    """Shapes with 1 to 9 instances (full and ragged groups of four), patterns
+    of one state, of up to 32 and of up to 126 states (inside a 32-position
+    window, across several), against single-shape plans; bit for bit the same
+    after the autotuner has picked another launch shape."""
+    rng = np.random.default_rng(83)
+    specs = [(9, [1] * 8 + [0], True, 5), (7, [4, 3, 3, 0, 0, 0, 0], True, 4), (6, [1, 1, 1, 1, 0, 0], True, 1),
+             (10, [1, 1, 1] + [0] * 7, False, 9), (3, [1, 0, 0], True, 2), (2, [6, 6], True, 3), (5, [2, 0, 1, 0, 0], False, 8)]
+    inst = []
+    for m, s, thr, cnt in specs:
+        inst += [workloads.UnevenInstance(m=m, n=sum(s), s=list(s), threshold=thr)] * cnt
+    Us = [workloads.haar_unitaries(it.m, 1, rng)[0] for it in inst]
+    bp = make_plan(slos, inst)
+    ws = torch.empty(bp.workspace_bytes, dtype=torch.uint8, device="cuda")
+    out = torch.full((bp.out_offsets[-1],), float("nan"), dtype=torch.float32, device="cuda")
+    U = pack(Us)
+    bp.forward(U, out, ws)
+    bp.sync_status()
+    first = out.clone()
+    bp.autotune(U, out, ws)
+    out.fill_(float("nan"))
+    bp.forward(U, out, ws)
+    assert torch.equal(out, first)
+    for i, it in enumerate(inst):
+        plan = slos.Plan(it.m, it.s, slos.THRESHOLD if it.threshold else slos.PNR)
+        ref = plan.forward(torch.tensor(Us[i][None], dtype=torch.complex64, device="cuda"))[0]
+        # sums of positive terms in another order: a few ulps of each value
+        assert torch.allclose(first[bp.out_offsets[i]:bp.out_offsets[i + 1]], ref, rtol=1e-5, atol=1e-9)
