@@ -1410,7 +1410,10 @@ slos_status_t slos_plan_space(int m, int n, const int *input_state, slos_detecti
     }
     choose_fused(p);
     // the small leading layers on chip (Fock-space table plans: the child tables have no holes)
-    p->prefix_L = (p->tab.enabled && p->space == SLOS_SPACE_FOCK) ? slos_prefix_layers(p->m, p->n, p->F.data()) : 0;
+    if (p->tab.enabled && p->space == SLOS_SPACE_FOCK) {
+        p->prefix_L = slos_prefix_layers(p->m, p->n, p->F.data(), kPrefixInstBytes);
+        p->prefix_L_many = slos_prefix_layers(p->m, p->n, p->F.data(), kPrefixManyBytes);
+    }
     tst = build_encode_tables(p);
     if (tst != SLOS_OK) {
         free_tables(p);
@@ -1504,13 +1507,20 @@ static slos_status_t launch_layer_fwd(slos_plan_s *p, const Layout &Ly, char *ws
     return SLOS_OK;
 }
 
-// Prefix depth in use: the tuned one, else the largest that fits.
-static int prefix_layers(const slos_plan_s *p) { return p->tune_prefix_L >= 0 ? p->tune_prefix_L : p->prefix_L; }
+// Prefix depth in use for a batch: the tuned one, else the largest that fits,
+// of at most kPrefixManyBytes per instance once the batch gives every SM more
+// instances than it holds at once (training step kernels, m=12 n=6: batch 200,
+// depth 5 185 us, 4 194 us; batch 1000, depth 5 (60 KB) 434 us, 4 385 us, 3 393 us;
+// m=16 n=8, batch 256: depth 4 (45 KB) 2068 us, 3 2073 us).
+static int prefix_layers(const slos_plan_s *p, int batch) {
+    if (p->tune_prefix_L >= 0) return p->tune_prefix_L;
+    return (int64_t)batch > 2 * (int64_t)p->sm_count ? p->prefix_L_many : p->prefix_L;
+}
 
 static PrefixArgs prefix_args(const slos_plan_s *p, const float2 *U, int batch) {
     PrefixArgs pa;
     memset(&pa, 0, sizeof(pa));
-    const int L = prefix_layers(p);
+    const int L = prefix_layers(p, batch);
     pa.U = U;
     for (int k = 0; k <= L; ++k) pa.F[k] = (int)p->F[k];
     for (int k = 1; k <= L; ++k) {
@@ -1526,6 +1536,7 @@ static PrefixArgs prefix_args(const slos_plan_s *p, const float2 *U, int batch) 
     pa.L = L;
     pa.B = batch;
     pa.lanes = kLanes;
+    pa.sm_count = p->sm_count;
     pa.NI = slos_prefix_ni(p->m, L, p->F.data(), batch, p->sm_count);
     if (p->tune_prefix_ni > 0 && slos_prefix_bwd_smem(p->tune_prefix_ni, L, p->F.data()) <= kPrefixSmemLimit)
         pa.NI = p->tune_prefix_ni;
@@ -1639,9 +1650,9 @@ slos_status_t slos_forward(slos_plan_t p, const void *U, int batch, slos_output_
     }
     if (width == kLanes) SLOS_CUDA(cudaMemsetAsync(ws + Ly.counters, 0, kCounters * sizeof(int), s));
     int k0 = 1;
-    if (prefix_layers(p) >= 2) {
+    if (prefix_layers(p, batch) >= 2) {
         // kept layers of the prefix and its last layer (which layer L + 1 reads)
-        const int L = prefix_layers(p);
+        const int L = prefix_layers(p, batch);
         uint32_t want = 1u << L;
         for (int k = 1; k < L; ++k)
             if (save && p->stored[k]) want |= 1u << k;
@@ -1754,7 +1765,7 @@ slos_status_t slos_backward(slos_plan_t p, const void *U, int batch, slos_output
     int have_base = -1;  // segment currently recomputed (its kept base layer)
     ReduceArgs ra;
     memset(&ra, 0, sizeof(ra));
-    const int L = prefix_layers(p);
+    const int L = prefix_layers(p, batch);
     for (int k = n; k >= 1; --k) {
         const int kp = k - 1;
         int bx = Ly.bwd_blocks[k];  // CTAs per group of this layer's launch (dU partial rows)
@@ -1952,8 +1963,12 @@ slos_status_t slos_autotune(slos_plan_t p, const void *U, int batch, void *out, 
     // the default shape first: a candidate replaces it only when it is more
     // than 0.5 % faster, so timing noise does not move the choice
     std::vector<int> Ls;
-    for (int L = p->prefix_L; L >= 2; --L) Ls.push_back(L);
-    Ls.push_back(0);
+    p->tune_prefix_L = -1;
+    const int L_def = prefix_layers(p, batch);
+    Ls.push_back(L_def);
+    for (int L = p->prefix_L; L >= 2; --L)
+        if (L != L_def) Ls.push_back(L);
+    if (L_def != 0) Ls.push_back(0);
     const int res = slos_pair_resident_blocks(p->m);
     const int fwd_opts[] = {res, std::max(1, res - 2)};
     const int bwd_opts[] = {kSplitBwdMinBlocks, kSplitBwdMinBlocks - 1};
@@ -1970,7 +1985,7 @@ slos_status_t slos_autotune(slos_plan_t p, const void *U, int batch, void *out, 
         if (r != SLOS_OK) return r;
         return slos_backward(p, U, batch, SLOS_OUT_PROBS, dout_shared, 0, dU, workspace, workspace_bytes, stream);
     };
-    const int ni_def = slos_prefix_ni(p->m, p->prefix_L, p->F.data(), batch, p->sm_count);
+    const int ni_def = slos_prefix_ni(p->m, L_def, p->F.data(), batch, p->sm_count);
     std::vector<int> nis = {ni_def};  // the default instance count first, then the others
     for (int v : {1, 2, 4})
         if (v != ni_def) nis.push_back(v);
@@ -2023,7 +2038,7 @@ done:
 slos_status_t slos_plan_tuning(slos_plan_t p, int *prefix_layers_out, int *prefix_ni, int *fwd_blocks_per_sm,
                                int *bwd_blocks_per_sm) {
     if (!p || p->kind != 0) return fail(SLOS_ERR_INVALID_ARG, "slos_plan_tuning: not a single-shape plan");
-    if (prefix_layers_out) *prefix_layers_out = prefix_layers(p);
+    if (prefix_layers_out) *prefix_layers_out = p->tune_prefix_L >= 0 ? p->tune_prefix_L : p->prefix_L;
     if (prefix_ni) *prefix_ni = p->tune_prefix_ni;
     if (fwd_blocks_per_sm) *fwd_blocks_per_sm = p->tune_fwd_bps;
     if (bwd_blocks_per_sm) *bwd_blocks_per_sm = p->tune_bwd_bps;

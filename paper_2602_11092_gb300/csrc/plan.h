@@ -77,6 +77,7 @@ struct slos_plan_s {
     int fused_cap[2] = {1, 1};  // its buffer capacities (states per instance, even / odd layers)
     bool fused_sorted = false;  // walks the sorted layout (tab.fused) instead of Fock order
     int prefix_L = 0;           // layers 1..prefix_L run on chip in one launch each way (0: none)
+    int prefix_L_many = 0;      // the same for batches of many instances per SM
     // launch shapes picked by slos_autotune (negative / zero: the defaults)
     int tune_prefix_L = -1;     // prefix depth: 0 (none) or 2..prefix_L
     int tune_prefix_ni = 0;     // prefix instances per CTA: 1, 2 or 4

@@ -12,6 +12,7 @@ namespace slos {
 // Shared memory a prefix CTA may use, and the per-instance bound that picks L.
 constexpr size_t kPrefixSmemLimit = 200 * 1024;
 constexpr size_t kPrefixInstBytes = 100 * 1024;
+constexpr size_t kPrefixManyBytes = 48 * 1024;  // bound for batches of many instances per SM
 constexpr int kPrefixMaxNI = 4;
 constexpr int kPrefixThreads = 512;
 
@@ -31,11 +32,12 @@ struct PrefixArgs {
     int cap[2];                               // states per instance of the even / odd layer buffers
     int asum;                                 // backward: states of a_0..a_{L-1} per instance
     int m, L, B, NI;
+    int sm_count;
 };
 
-// Largest L (2 <= L <= n - 1) whose backward working set fits kPrefixInstBytes
-// per instance; 0 when no prefix of two or more layers fits.
-int slos_prefix_layers(int m, int n, const int64_t *F);
+// Largest L (2 <= L <= n - 1) whose backward working set fits `bytes` per
+// instance; 0 when no prefix of two or more layers fits.
+int slos_prefix_layers(int m, int n, const int64_t *F, size_t bytes);
 // Instances per CTA for a batch (1, 2 or 4).
 int slos_prefix_ni(int m, int L, const int64_t *F, int batch, int sm_count);
 size_t slos_prefix_fwd_smem(int NI, int L, const int64_t *F);

@@ -17,7 +17,12 @@
 //      G_{k-1}(t') = sum_j conj(U[j, c_k]) G_k(t' + e_j)
 //      dU[j, c_k]  = sum_{t'} conj(a_{k-1}(t')) G_k(t' + e_j)
 //   each dU column summed over the CTA in a fixed order and written as the
-//   layer's single partial row of the lane's instance.
+//   layer's single partial row of the lane's instance.  Bound by its chain of
+//   barriers and shuffles, not by its gathers: with every layer's sums reduced
+//   and added up between two barriers of their own, five shuffles a value, in
+//   512-thread CTAs, 1000 instances of m=12 n=6 took 65 us for 4 layers; with a
+//   reduce-scatter, one barrier a layer and CTAs sized to the layers 33 us
+//   (m=16 n=8, batch 256: 33 -> 22 us; m=8 n=4, batch 2000: 63 -> 14 us).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -53,11 +58,11 @@ size_t slos_prefix_bwd_smem(int NI, int L, const int64_t *F) {
     prefix_caps(L, F, cap);
     return prefix_us_bytes(NI, L) + (size_t)NI * (prefix_asum(L, F) + cap[0] + cap[1]) * sizeof(float2);
 }
-int slos_prefix_layers(int m, int n, const int64_t *F) {
+int slos_prefix_layers(int m, int n, const int64_t *F, size_t bytes) {
     if (m > kMaxModes) return 0;
     int best = 0;
     for (int L = 2; L <= n - 1; ++L)
-        if (slos_prefix_bwd_smem(1, L, F) <= kPrefixInstBytes) best = L;
+        if (slos_prefix_bwd_smem(1, L, F) <= bytes) best = L;
     return best;
 }
 int slos_prefix_ni(int m, int L, const int64_t *F, int batch, int sm_count) {
@@ -147,49 +152,50 @@ __global__ void __launch_bounds__(kPrefixThreads, 2) slos_fwd_prefix_kernel(Pref
     }
 }
 
-// Fixed-order CTA sums of the m complex values of every thread: each warp
-// reduces its values with shuffles, then thread j < m adds mode j over the
-// warps in warp order and writes dst[j].  red: [warps][kMaxModes].
+// Sum over the warp of each of the MM complex values of every lane, in a fixed
+// order, into red[2 * MM]: at each step a lane keeps the half of the values its
+// bit selects, so the values cost about one shuffle each instead of five.
 template <int MM>
-__device__ __forceinline__ void prefix_cta_sum_modes(float2 (&du)[MM], int m, float2 *red, float2 *dst) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void prefix_warp_sum(const float2 (&du)[MM], float *red) {
+    constexpr int N = (2 * MM + 31) / 32 * 32;
+    const int lane = threadIdx.x & 31;
+    float v[N];
 #pragma unroll
-    for (int j = 0; j < MM; ++j) {
-        if (j < m) {
+    for (int i = 0; i < N; ++i) v[i] = i < 2 * MM ? (i & 1 ? du[i / 2].y : du[i / 2].x) : 0.f;
+    int at = 0, n = N;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                du[j].x += __shfl_down_sync(0xffffffffu, du[j].x, o);
-                du[j].y += __shfl_down_sync(0xffffffffu, du[j].y, o);
+    for (int s = 16; s > 0; s >>= 1) {
+        n /= 2;
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) {
+            if (i < n) {
+                const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
             }
-            if (lane == 0) red[warp * kMaxModes + j] = du[j];
         }
+        at += up ? n : 0;
     }
-    __syncthreads();
-    if ((int)threadIdx.x < m) {
-        float2 t = make_float2(0.f, 0.f);
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            t.x += red[w * kMaxModes + threadIdx.x].x;
-            t.y += red[w * kMaxModes + threadIdx.x].y;
-        }
-        dst[threadIdx.x] = t;
-    }
-    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N / 32; ++i)
+        if (at + i < 2 * MM) red[at + i] = v[i];
 }
 
 // MM: a bound on m (16 or 24), the size of the per-thread dU accumulators.
+// One barrier per layer: the layer's G and its warps' dU sums are published
+// together, and the sums are added over the warps (in warp order) while the
+// next layer is walked, its sums going to the other half of `red`.
 template <int MM>
 __global__ void __launch_bounds__(kPrefixThreads, 2) slos_bwd_prefix_kernel(PrefixArgs a) {
     extern __shared__ float2 pf_sm[];
-    __shared__ float2 red[(kPrefixThreads / 32) * kMaxModes];
+    __shared__ float red[2][kPrefixMaxNI][kPrefixThreads / 32][2 * MM];
     const int NI = a.NI, L = a.L, m = a.m;
+    const int warp = threadIdx.x >> 5;
     float2 *us = pf_sm;                                  // [NI][L][kPfUsRow]
     float2 *as = us + (size_t)NI * L * kPfUsRow;         // [NI][asum]: a_0 .. a_{L-1}
     float2 *gbuf[2];                                     // G_k in gbuf[k & 1]: [NI][cap[k & 1]]
     gbuf[0] = as + (size_t)NI * a.asum;
     gbuf[1] = gbuf[0] + (size_t)NI * a.cap[0];
-    int aoff[kMaxPhotons + 1];
-    aoff[0] = 0;
-    for (int k = 1; k <= L; ++k) aoff[k] = aoff[k - 1] + a.F[k - 1];
     const int inst0 = blockIdx.x * NI;
     const int ni = min(NI, a.B - inst0);
     const int grp = inst0 / kLanes, l0 = inst0 % kLanes;
@@ -205,8 +211,10 @@ __global__ void __launch_bounds__(kPrefixThreads, 2) slos_bwd_prefix_kernel(Pref
     }
     __syncthreads();
     // a_1 .. a_{L-1}, recomputed
+    int aoff = 0;
     for (int k = 1; k < L; ++k) {
-        prefix_layer_kw(a, k, us, as + aoff[k - 1], a.asum, as + aoff[k], a.asum, ni, nullptr);
+        prefix_layer_kw(a, k, us, as + aoff, a.asum, as + aoff + a.F[k - 1], a.asum, ni, nullptr);
+        aoff += a.F[k - 1];
         __syncthreads();
     }
     for (int k = L; k >= 1; --k) {
@@ -215,48 +223,59 @@ __global__ void __launch_bounds__(kPrefixThreads, 2) slos_bwd_prefix_kernel(Pref
         const float2 *gk = gbuf[k & 1];
         float2 *gp = gbuf[(k - 1) & 1];
         const int capk = a.cap[k & 1], capp = a.cap[(k - 1) & 1];
-        for (int i = 0; i < ni; ++i) {
-            const float2 *u = us + (size_t)(i * L + k - 1) * kPfUsRow;
-            const float2 *ak = as + (size_t)i * a.asum + aoff[k - 1];
-            const float2 *gi = gk + (size_t)i * capk;
-            float2 du[MM];
+        // warps with a parent of this layer
+        const int nw = min((int)(blockDim.x >> 5), (Fp + 31) >> 5);
+        if (warp < nw) {
+            for (int i = 0; i < ni; ++i) {
+                const float2 *u = us + (size_t)(i * L + k - 1) * kPfUsRow;
+                const float2 *ak = as + (size_t)i * a.asum + aoff;
+                const float2 *gi = gk + (size_t)i * capk;
+                float2 du[MM];
 #pragma unroll
-            for (int j = 0; j < MM; ++j) du[j] = make_float2(0.f, 0.f);
-            for (int t = threadIdx.x; t < Fp; t += blockDim.x) {
-                const float2 av = ak[t];
-                float2 gacc = make_float2(0.f, 0.f);
-                // child ranks of parent t: rows of m entries, read as int4 when m % 4 == 0
-                if (m % 4 == 0) {
-                    const int4 *c4 = reinterpret_cast<const int4 *>(ct + (size_t)t * m);
+                for (int j = 0; j < MM; ++j) du[j] = make_float2(0.f, 0.f);
+                for (int t = threadIdx.x; t < Fp; t += blockDim.x) {
+                    const float2 av = ak[t];
+                    float2 gacc = make_float2(0.f, 0.f);
+                    // child ranks of parent t: rows of m entries, read as int4 when m % 4 == 0
+                    if (m % 4 == 0) {
+                        const int4 *c4 = reinterpret_cast<const int4 *>(ct + (size_t)t * m);
 #pragma unroll
-                    for (int j4 = 0; j4 < MM / 4; ++j4) {
-                        if (4 * j4 < m) {
-                            const int4 v = __ldg(c4 + j4);
-                            const int cx[4] = {v.x, v.y, v.z, v.w};
+                        for (int j4 = 0; j4 < MM / 4; ++j4) {
+                            if (4 * j4 < m) {
+                                const int4 v = __ldg(c4 + j4);
+                                const int cx[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                            for (int i4 = 0; i4 < 4; ++i4) {
-                                const int j = 4 * j4 + i4;
-                                const float2 g = gi[cx[i4]];
+                                for (int i4 = 0; i4 < 4; ++i4) {
+                                    const int j = 4 * j4 + i4;
+                                    const float2 g = gi[cx[i4]];
+                                    gacc = cfma_conj_a(u[j], g, gacc);
+                                    du[j] = cfma_conj_a(av, g, du[j]);
+                                }
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < MM; ++j) {
+                            if (j < m) {
+                                const float2 g = gi[__ldg(ct + (size_t)t * m + j)];
                                 gacc = cfma_conj_a(u[j], g, gacc);
                                 du[j] = cfma_conj_a(av, g, du[j]);
                             }
                         }
                     }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < MM; ++j) {
-                        if (j < m) {
-                            const float2 g = gi[__ldg(ct + (size_t)t * m + j)];
-                            gacc = cfma_conj_a(u[j], g, gacc);
-                            du[j] = cfma_conj_a(av, g, du[j]);
-                        }
-                    }
+                    if (k >= 2) gp[(size_t)i * capp + t] = gacc;
                 }
-                if (k >= 2) gp[(size_t)i * capp + t] = gacc;
+                prefix_warp_sum<MM>(du, red[k & 1][i][warp]);
             }
-            prefix_cta_sum_modes(du, m, red, a.dUpart[k] + ((size_t)grp * kLanes + l0 + i) * m);
         }
         __syncthreads();
+        for (int x = threadIdx.x; x < ni * 2 * m; x += blockDim.x) {
+            const int i = x / (2 * m), f = x % (2 * m);
+            float s = 0.f;
+            for (int w = 0; w < nw; ++w) s += red[k & 1][i][w][f];
+            reinterpret_cast<float *>(a.dUpart[k] + ((size_t)grp * kLanes + l0 + i) * m)[f] = s;
+        }
+        aoff -= k >= 2 ? a.F[k - 2] : 0;
     }
 }
 
@@ -272,6 +291,15 @@ cudaError_t slos_prefix_init() {
                                 (int)kPrefixSmemLimit);
 }
 
+// Threads of a prefix CTA: the full 512 while the grid is too small to fill the
+// GPU otherwise, fewer when its layers (`states` in the widest one walked) do
+// not feed 512 and more CTAs per SM hide each other's latencies.
+static int prefix_threads(const PrefixArgs &a, int states) {
+    const int ctas = (a.B + a.NI - 1) / a.NI;
+    if (ctas <= 2 * a.sm_count) return kPrefixThreads;
+    return states <= 160 ? 128 : (states <= 820 ? 256 : kPrefixThreads);
+}
+
 static size_t prefix_smem_args(const PrefixArgs &a, bool bwd) {
     return (size_t)a.NI * a.L * kPfUsRow * sizeof(float2) +
            (size_t)a.NI * ((bwd ? a.asum : 0) + a.cap[0] + a.cap[1]) * sizeof(float2);
@@ -280,7 +308,7 @@ static size_t prefix_smem_args(const PrefixArgs &a, bool bwd) {
 cudaError_t slos_launch_prefix_fwd(const PrefixArgs &a, cudaStream_t s) {
     const size_t sm = prefix_smem_args(a, false);
     if (sm > kPrefixSmemLimit || a.NI < 1 || a.lanes % a.NI != 0) return cudaErrorInvalidValue;
-    slos_fwd_prefix_kernel<<<(a.B + a.NI - 1) / a.NI, kPrefixThreads, sm, s>>>(a);
+    slos_fwd_prefix_kernel<<<(a.B + a.NI - 1) / a.NI, prefix_threads(a, a.F[a.L] / 2), sm, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -288,10 +316,11 @@ cudaError_t slos_launch_prefix_bwd(const PrefixArgs &a, cudaStream_t s) {
     const size_t sm = prefix_smem_args(a, true);
     if (sm > kPrefixSmemLimit || a.NI < 1 || kLanes % a.NI != 0) return cudaErrorInvalidValue;
     const int grid = (a.B + a.NI - 1) / a.NI;
+    const int threads = prefix_threads(a, a.F[a.L - 1]);
     if (a.m <= 16)
-        slos_bwd_prefix_kernel<16><<<grid, kPrefixThreads, sm, s>>>(a);
+        slos_bwd_prefix_kernel<16><<<grid, threads, sm, s>>>(a);
     else
-        slos_bwd_prefix_kernel<kMaxModes><<<grid, kPrefixThreads, sm, s>>>(a);
+        slos_bwd_prefix_kernel<kMaxModes><<<grid, threads, sm, s>>>(a);
     return cudaGetLastError();
 }
 
