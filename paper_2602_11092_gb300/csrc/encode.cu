@@ -165,17 +165,23 @@ __global__ void __launch_bounds__(256) encode_split_b_kernel(const float2 *A, in
     }
 }
 
-// Real-form operand A of the GEMM for batch rows [b0, b0 + rows), one block
+// Real-form operand A of the GEMM for batch rows [b0, b0 + rows), T threads
 // per row: [rows][K2], cols s -> Re X[b][s] / g_s, K + s -> Im X[b][s] / g_s,
 // the padding columns 2K .. K2-1 zero; scaled and split into hi and lo copies.
-// rowscale[r] = 1 over the row's scale.
+// rowscale[r] = 1 over the row's scale.  T = 32 (a warp per row, no barrier)
+// up to kSplitWarpRow values, a block per row beyond (1657 rows of 56: a block
+// each cost 3 us more than a warp each).
 constexpr int kSplitThreads = 256;
 constexpr int kSplitKeep = 8;  // values per thread kept in registers between the maximum and the split
+constexpr int64_t kSplitWarpRow = 32 * kSplitKeep;
+template <int T>
 __global__ void __launch_bounds__(kSplitThreads) encode_split_a_kernel(const float2 *X, const float *g, int64_t b0,
-                                                                       int64_t K, int64_t K2, __half *ahi, __half *alo,
-                                                                       float *rowscale) {
+                                                                       int rows, int64_t K, int64_t K2, __half *ahi,
+                                                                       __half *alo, float *rowscale) {
     __shared__ unsigned int red[kSplitThreads / 32];
-    const int64_t r = blockIdx.x;
+    const int64_t r = (int64_t)blockIdx.x * (kSplitThreads / T) + threadIdx.x / T;
+    if (r >= rows) return;  // whole warps (T = 32) or nobody
+    const int tid = threadIdx.x % T;
     const float2 *x = X + (b0 + r) * K;
     auto value = [&](int64_t s) {
         const float2 v = x[s];
@@ -187,17 +193,19 @@ __global__ void __launch_bounds__(kSplitThreads) encode_split_a_kernel(const flo
     unsigned int top = 0u;
 #pragma unroll
     for (int i = 0; i < kSplitKeep; ++i) {
-        const int64_t s = threadIdx.x + (int64_t)i * kSplitThreads;
+        const int64_t s = tid + (int64_t)i * T;
         keep[i] = s < K ? value(s) : make_float2(0.f, 0.f);
         top = max(top, bits(keep[i]));
     }
-    const int64_t rest = threadIdx.x + (int64_t)kSplitKeep * kSplitThreads;
-    for (int64_t s = rest; s < K; s += kSplitThreads) top = max(top, bits(value(s)));
+    const int64_t rest = tid + (int64_t)kSplitKeep * T;
+    for (int64_t s = rest; s < K; s += T) top = max(top, bits(value(s)));
     top = __reduce_max_sync(0xffffffffu, top);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
-    __syncthreads();
+    if (T > 32) {
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+        __syncthreads();
 #pragma unroll
-    for (int w = 0; w < kSplitThreads / 32; ++w) top = max(top, red[w]);
+        for (int w = 0; w < T / 32; ++w) top = max(top, red[w]);
+    }
     const int ex = split_exponent(top);
     const float sc = pow2f(ex);
     __half *h = ahi + r * K2, *l = alo + r * K2;
@@ -212,12 +220,12 @@ __global__ void __launch_bounds__(kSplitThreads) encode_split_a_kernel(const flo
     };
 #pragma unroll
     for (int i = 0; i < kSplitKeep; ++i) {
-        const int64_t s = threadIdx.x + (int64_t)i * kSplitThreads;
+        const int64_t s = tid + (int64_t)i * T;
         if (s < K) put(s, keep[i]);
     }
-    for (int64_t s = rest; s < K; s += kSplitThreads) put(s, value(s));
-    for (int64_t c = 2 * K + threadIdx.x; c < K2; c += kSplitThreads) h[c] = l[c] = __float2half_rn(0.f);
-    if (threadIdx.x == 0) rowscale[r] = pow2f(-ex);
+    for (int64_t s = rest; s < K; s += T) put(s, value(s));
+    for (int64_t c = 2 * K + tid; c < K2; c += T) h[c] = l[c] = __float2half_rn(0.f);
+    if (tid == 0) rowscale[r] = pow2f(-ex);
 }
 
 // FP16 matrix [rows][cols] (row stride ld elements, a multiple of 8), box
@@ -375,8 +383,12 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
         const int rows = std::min(kEncodeChunk, batch - b0);
         {
             ProfScope ps("slos_encode_split", 0.0, s);
-            encode_split_a_kernel<<<(unsigned)rows, kSplitThreads, 0, s>>>(Xd, p->tab.gfact, b0, K, K2, ahi, alo,
-                                                                           rowscale);
+            if (K <= kSplitWarpRow)
+                encode_split_a_kernel<32><<<(unsigned)((rows + 7) / 8), kSplitThreads, 0, s>>>(
+                    Xd, p->tab.gfact, b0, rows, K, K2, ahi, alo, rowscale);
+            else
+                encode_split_a_kernel<kSplitThreads><<<(unsigned)rows, kSplitThreads, 0, s>>>(
+                    Xd, p->tab.gfact, b0, rows, K, K2, ahi, alo, rowscale);
             if ((e = cudaGetLastError()) != cudaSuccess)
                 return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
         }
