@@ -127,19 +127,14 @@ def _ptr(t: torch.Tensor | None):
     return None if t is None else t.data_ptr()
 
 
-_cuda_ready = False
-
-
 def _stream(stream=None):
     """The stream's handle; by default the current device's current stream
     (read as a handle: building a torch.cuda.Stream object takes 3 us, more
     than a launch)."""
     if stream is not None:
         return stream.cuda_stream
-    global _cuda_ready
-    if not _cuda_ready:
+    if not torch.cuda.is_initialized():
         torch.cuda.init()
-        _cuda_ready = True
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 

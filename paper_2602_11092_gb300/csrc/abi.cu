@@ -1584,6 +1584,10 @@ static int narrow_width(const slos_plan_s *p, int batch) {
         if (p->fused_threads == 1024) return width;
         return p->F[p->n] >= 2000 && batch >= 4 ? width : kLanes;
     }
+    // a CTA of these kernels serves one group of four: few states leave most of
+    // it idle (m=5 n=2, 15 states: batch 8192 9.9 us / 16.6, 32768 24.9 / 18.5;
+    // m=8 n=2, 36 states, 32768: 28 / 29), and the grid ends at 65535 groups
+    if (batch > (p->F[p->n] < 32 ? 16384 : 65535 * 4)) return kLanes;
     const int64_t most = p->det == SLOS_DETECT_PNR ? (int64_t)1 << 25 : 6500000;
     return (int64_t)batch * p->F[p->n] <= most ? width : kLanes;
 }

@@ -436,6 +436,22 @@ def test_backward_threshold(slos, m, n, B):
         assert np.linalg.norm(dU[b] - ref) / np.linalg.norm(ref) <= G_TOL
 
 
+@pytest.mark.parametrize("m,s,B", [(4, [1, 0, 1, 0], 16384), (4, [1, 0, 1, 0], 16385), (6, [1, 0, 1, 0, 1, 0], 262140),
+                                   (6, [1, 0, 1, 0, 1, 0], 262141)])
+def test_threshold_forward_of_very_many_small_instances(slos, m, s, B):
+    """Either side of the two limits on the batch of the lane = state kernels
+    (few states, and one grid row per group of four): the first and the last
+    instances of the batch against the same instances alone."""
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    U = torch.randn(B, m, m, 2, generator=gen, device="cuda") * 0.3
+    U = torch.view_as_complex(U)
+    plan = slos.Plan(m, s, slos.THRESHOLD)
+    got = plan.forward(U)
+    for part in (slice(0, 5), slice(B - 6, B)):
+        # the same sums of positive terms, up to their order
+        assert torch.allclose(got[part], plan.forward(U[part].contiguous()), rtol=1e-5, atol=1e-9)
+
+
 @pytest.mark.parametrize("m,n,kind,B", [(4, 2, "probs", 1), (8, 4, "probs", 65), (8, 4, "amps", 33), (16, 4, "threshold", 33),
                                         (9, 6, "threshold", 31), (3, 8, "threshold", 2), (17, 3, "amps", 5)])
 def test_output_gradient_rows_shared_or_per_instance(slos, m, n, kind, B):
