@@ -91,11 +91,18 @@ int sm_count() {
     return g_sm_count[dev];
 }
 
+// Products without bias or activation (the only ones use_pairs sends to single CTAs).
+template <int EPI>
+constexpr bool kPlain = EPI == TC_F32 || EPI == TC_F32_ACCUM;
+
 template <int EPI>
 cudaError_t set_attr() {
-    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(tc_gemm_persist_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(tc_gemm_pair_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
+    if constexpr (kPlain<EPI>) {
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(tc_gemm_persist_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    }
+    return e;
 }
 
 cudaError_t init_attrs() {
@@ -112,6 +119,29 @@ cudaError_t init_attrs() {
     return cudaSuccess;
 }
 
+int64_t gemm_tiles(int M, int N, int rows) { return (int64_t)((N + BN - 1) / BN) * ((M + rows - 1) / rows); }
+
+// Pairs but for plain products of at most one wave of 128 x 256 tiles, where one
+// CTA's MMAs run a little ahead of a pair's (us, pairs / single: 2048 x 2048 x
+// 16384 101 / 96, 64 x 2048 x 2048 17.1 / 15.6); with a bias or GELU the epilogue
+// decides (128 x 12376 x 2048 19.9 / 21.7, 128 x 2048 x 288 13.5 / 15.3).
+bool use_pairs(int epi, int M, int N) {
+    const bool plain = epi == TC_F32 || epi == TC_F32_ACCUM;
+    return !(plain && gemm_tiles(M, N, BM) <= sm_count());
+}
+
+// Persistent CTAs, one per SM (the shared-memory ring allows no second).
+template <int EPI>
+void launch_gemm(bool pair, const CUtensorMap &ta, const CUtensorMap &tb, const TcArgs &g, cudaStream_t s) {
+    if (!kPlain<EPI> || pair) {
+        const unsigned pairs = (unsigned)std::min<int64_t>(gemm_tiles(g.M, g.N, 2 * BM), std::max(1, sm_count() / 2));
+        tc_gemm_pair_kernel<EPI><<<2 * pairs, kPairThreads, kPairSmem, s>>>(ta, tb, g);
+    } else if constexpr (kPlain<EPI>) {
+        const unsigned grid = (unsigned)std::min<int64_t>(gemm_tiles(g.M, g.N, BM), sm_count());
+        tc_gemm_persist_kernel<EPI><<<grid, kPersistThreads, SMEM_BYTES, s>>>(ta, tb, g);
+    }
+}
+
 // C[M][N] = A[M][K] . B[N][K]^T with epilogue EPI.  lda/ldb in elements.
 slos_status_t gemm(int epi, int M, int N, int K, const __nv_bfloat16 *A, int64_t lda, const __nv_bfloat16 *Bm,
                    int64_t ldb, void *C, int ldc, const float *bias, __nv_bfloat16 *aux, cudaStream_t s) {
@@ -123,7 +153,8 @@ slos_status_t gemm(int epi, int M, int N, int K, const __nv_bfloat16 *A, int64_t
     cudaError_t e = init_attrs();
     if (e != cudaSuccess) return fail(SLOS_ERR_CUDA, std::string("GEMM attributes: ") + cudaGetErrorString(e));
     CUtensorMap ta, tb;
-    if (!make_map(&ta, A, M, K, lda, BM) || !make_map(&tb, Bm, N, K, ldb, BN))
+    const bool pair = use_pairs(epi, M, N);
+    if (!make_map(&ta, A, M, K, lda, BM) || !make_map(&tb, Bm, N, K, ldb, pair ? BN / 2 : BN))
         return fail(SLOS_ERR_CUDA, "cuTensorMapEncodeTiled failed");
     TcArgs g;
     g.M = M;
@@ -137,17 +168,13 @@ slos_status_t gemm(int epi, int M, int N, int K, const __nv_bfloat16 *A, int64_t
     g.colscale = nullptr;
     g.rowscale = nullptr;
     g.amps = 0;
-    // persistent CTAs, one per SM (the shared-memory ring allows no second)
-    const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-    const unsigned grid = (unsigned)std::min<int64_t>(tiles, sm_count());
     ProfScope ps("tc_gemm", 2.0 * M * N * K, s);  // flops, not bytes
-    constexpr int T = kPersistThreads;
     switch (epi) {
-        case TC_F32: tc_gemm_persist_kernel<TC_F32><<<grid, T, SMEM_BYTES, s>>>(ta, tb, g); break;
-        case TC_F32_BIAS: tc_gemm_persist_kernel<TC_F32_BIAS><<<grid, T, SMEM_BYTES, s>>>(ta, tb, g); break;
-        case TC_GELU: tc_gemm_persist_kernel<TC_GELU><<<grid, T, SMEM_BYTES, s>>>(ta, tb, g); break;
-        case TC_GELU_BWD: tc_gemm_persist_kernel<TC_GELU_BWD><<<grid, T, SMEM_BYTES, s>>>(ta, tb, g); break;
-        case TC_F32_ACCUM: tc_gemm_persist_kernel<TC_F32_ACCUM><<<grid, T, SMEM_BYTES, s>>>(ta, tb, g); break;
+        case TC_F32: launch_gemm<TC_F32>(pair, ta, tb, g, s); break;
+        case TC_F32_BIAS: launch_gemm<TC_F32_BIAS>(pair, ta, tb, g, s); break;
+        case TC_GELU: launch_gemm<TC_GELU>(pair, ta, tb, g, s); break;
+        case TC_GELU_BWD: launch_gemm<TC_GELU_BWD>(pair, ta, tb, g, s); break;
+        case TC_F32_ACCUM: launch_gemm<TC_F32_ACCUM>(pair, ta, tb, g, s); break;
         default: return fail(SLOS_ERR_INVALID_ARG, "GEMM epilogue");
     }
     e = cudaGetLastError();

@@ -3,22 +3,19 @@
 // tc_gemm_split_kernel (end of the file) multiplies FP32-accurate operands
 // given as pairs of FP16 copies, with the same stage rows of 128 bytes (64
 // 16-bit elements), swizzle and descriptors.
-// Two kernels share the pipeline below: tc_gemm_kernel (one tile per CTA) and
-// tc_gemm_persist_kernel (one CTA per SM over many tiles, two accumulators,
-// the epilogue of one tile overlapping the next tile's MMAs), which the
-// library launches.
+// Two kernels share the pipeline below, both persistent over many tiles:
+// tc_gemm_pair_kernel (256 x 256 tiles on CTA pairs) and tc_gemm_persist_kernel
+// (128 x 256 tiles, one CTA each; surrogate.cu's use_pairs says when).
 //
-// One CTA = 128 threads computes one 128 x 256 output tile.
-//   warp 0, lane 0: TMA producer.  cp.async.bulk.tensor loads 128x64 tiles of
-//                   A and B (128-byte swizzle) into a 4-stage ring; each stage
+//   TMA producer:   cp.async.bulk.tensor loads tiles of A and B, 64 values of K
+//                   wide (128-byte swizzle), into a ring of stages; each stage
 //                   has a `full` mbarrier (transaction bytes) and an `empty`
 //                   mbarrier (arrived by tcgen05.commit when the MMAs that
 //                   read the stage are done).
-//   warp 1, lane 0: MMA issuer.  Four tcgen05.mma.kind::f16 (K = 16 each) per
-//                   stage into one 128 x 256 FP32 accumulator in TMEM
-//                   (256 of the SM's 512 TMEM columns).
-//   all 4 warps:    epilogue.  tcgen05.ld 32x32b: warp w reads TMEM lanes
-//                   32w..32w+31 (= output rows), 16 columns per load.
+//   MMA issuer:     four tcgen05.mma.kind::f16 (K = 16 each) per stage into one
+//                   of two FP32 accumulators in TMEM.
+//   epilogue warps: tcgen05.ld 32x32b of the other accumulator: warp w reads
+//                   TMEM lanes 32 (w % 4) .. + 31 (= output rows).
 // Every mbarrier wait has an iteration limit; a wait that runs out sets the
 // error word, the CTA still frees its TMEM and returns.
 #pragma once
@@ -36,7 +33,6 @@ constexpr int A_TILE = BM * BK * 2;  // bytes
 constexpr int B_TILE = BN * BK * 2;
 constexpr int STAGE_BYTES = A_TILE + B_TILE;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
-constexpr uint32_t TMEM_COLS = BN;
 constexpr long long kWaitLimit = 1ll << 22;  // tries; a few seconds at most
 
 enum TcEpi : int {
@@ -244,107 +240,6 @@ __device__ __forceinline__ void tc_store16(const TcArgs &g, int row, int col0, f
     }
 }
 
-template <int EPI>
-__global__ void __launch_bounds__(128, 1)
-    tc_gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, TcArgs g) {
-    extern __shared__ uint8_t smem_tc[];
-    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_tc) + 1023) & ~uintptr_t(1023));
-    uint8_t *sA = base;
-    uint8_t *sB = base + STAGES * A_TILE;
-    uint64_t *full = reinterpret_cast<uint64_t *>(sB + STAGES * B_TILE);
-    uint64_t *empty = full + STAGES;
-    uint64_t *done = empty + STAGES;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int nk = (g.K + BK - 1) / BK;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(full + s, 1);
-            mbar_init(empty + s, 1);
-        }
-        mbar_init(done, 1);
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-
-    if (warp == 0 && lane == 0) {
-        // producer
-        int issued = 0;
-        for (int kt = 0; kt < nk; ++kt) {
-            const int s = kt % STAGES;
-            const uint32_t ph = (kt / STAGES) & 1;
-            if (kt >= STAGES && !mbar_wait(empty + s, ph ^ 1)) {
-                atomicExch(g.err, 1);
-                *abort_flag = 1;
-                break;
-            }
-            if (*abort_flag) break;
-            mbar_expect_tx(full + s, STAGE_BYTES);
-            tma_load_2d(sA + s * A_TILE, &ta, kt * BK, m0, full + s);
-            tma_load_2d(sB + s * B_TILE, &tb, kt * BK, n0, full + s);
-            issued = kt + 1;
-        }
-        // never leave with copies in flight: wait (bounded) for the last loads
-        for (int kt = (issued > STAGES ? issued - STAGES : 0); kt < issued; ++kt)
-            mbar_wait(full + (kt % STAGES), (kt / STAGES) & 1);
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer
-        for (int kt = 0; kt < nk; ++kt) {
-            const int s = kt % STAGES;
-            const uint32_t ph = (kt / STAGES) & 1;
-            if (*abort_flag || !mbar_wait(full + s, ph)) {
-                atomicExch(g.err, 2);
-                *abort_flag = 1;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t a0 = smem_u32(sA + s * A_TILE), b0 = smem_u32(sB + s * B_TILE);
-#pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-                mma_bf16(tmem, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), (kt > 0 || kk > 0) ? 1u : 0u);
-            mma_commit(empty + s);
-        }
-        mma_commit(done);  // arrives once every MMA issued above has completed
-    }
-    __syncwarp();
-    // epilogue
-    const bool ok = __all_sync(0xffffffffu, mbar_wait(done, 0) && !*abort_flag);
-    if (!ok && lane == 0) atomicExch(g.err, 3);
-    tc_fence_after();
-    const int row = m0 + warp * 32 + lane;
-    if (ok) {
-        // 16 consecutive outputs per thread per TMEM load: one row segment,
-        // written with 16-byte stores when the row stride allows it
-        const bool vec = (g.ldc % 8) == 0;
-#pragma unroll 1
-        for (int c = 0; c < BN; c += 16) {
-            float v[16];
-            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
-            tc_store16<EPI>(g, row, n0 + c, v, vec);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
-    }
-}
-
-
 // Persistent variant: one CTA per SM walks the output tiles t = blockIdx.x,
 // blockIdx.x + gridDim.x, ... (row-major over 128 x 256 tiles, so the CTAs
 // running together share A rows in L2).  Six warps:
@@ -497,6 +392,355 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kPersistTmemCols)
+                     : "memory");
+    }
+}
+
+// ---------------------------------------------------------------- CTA pairs
+// tc_gemm_pair_kernel: the persistent pipeline on CTA pairs (cta_group::2).
+// A pair shares a 256 x 256 tile: each CTA stages its 128 rows of A and half of
+// the 256 rows of B, the pair's MMA reads both halves of B, and each CTA holds
+// its 128 rows of the accumulator: 32 KB per CTA and 64 of K, where a 128 x 256
+// tile of one CTA takes 48 KB.  What bounds it is the MMAs: 0.36 us per 64 of K (1760 TFLOP/s over 76
+// pairs), 0.38 with the loads; four stages instead of six cost 4 %.  A
+// thread reads a row of outputs from TMEM; written as it stands that is 16 bytes
+// to each of 32 rows an instruction, so the epilogue warps turn their outputs in
+// shared memory first (eight warps: four fell behind the MMAs, sixteen were no
+// faster).  Measured, us for this kernel / one CTA a tile:
+// 16384 x 12376 x 2048 with bias 545 / 632 (1525 TFLOP/s), 12800 x 8000 x 768
+// with bias 131 / 242, 16384 x 2048 x 2048 with GELU 116 / 123 and K = 288 60 / 86
+// (GELU's arithmetic keeps the epilogue behind the MMAs), 8192^3 684 / 741.
+//
+// Roles as in tc_gemm_persist_kernel, with these differences: the even CTA
+// (rank 0) issues the MMAs of both and owns the `full` barriers, on which the
+// loads of both CTAs complete, and the `tempty` ones, on which the epilogue
+// warps of both arrive; the MMAs' commits arrive on the `empty` and `tfull`
+// barriers of both.  A CTA leaves only after the other has passed its last
+// barrier, so no arrival or operand read meets a CTA that is gone.
+constexpr int kPairEpiWarps = 8;
+constexpr int kPairThreads = 64 + 32 * kPairEpiWarps;
+constexpr int kPairStages = 6;
+constexpr int kPairStageBytes = 2 * BM * BK * 2;  // per CTA: 128 rows of A, 128 rows of B
+constexpr int kPairBox = 32 * 128;                // an epilogue warp's transposition buffer: 32 rows of 128 bytes
+constexpr int kPairSmem = kPairStages * kPairStageBytes + kPairEpiWarps * kPairBox + 1024 + 256;
+constexpr uint32_t kIdescPair =
+    (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
+
+// Address of this CTA's shared variable in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// Bounded wait on a barrier that threads of both CTAs arrive on.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity) {
+    for (long long i = 0; i < kWaitLimit; ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+// Load into this CTA's shared memory that completes on a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_pair(void *dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
+        "[%2];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y)
+        : "memory");
+}
+__device__ __forceinline__ void mma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(kIdescPair), "r"(accumulate)
+        : "memory");
+}
+// Arrival on this barrier of both CTAs once the MMAs issued so far have completed.
+__device__ __forceinline__ void mma_commit_pair(uint64_t *bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+__device__ __forceinline__ float2 unpack_bf16(uint32_t x) {
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x));
+}
+
+// Epilogue of 32 rows x 32 columns by a warp, columns col0 .. col0 + 31 all
+// inside the matrix, rows and bias 16-byte aligned: v holds row row0 + lane.
+// The block is turned in `box` (32 rows of eight 16-byte slots, slot q of row r
+// at q ^ (r & 7), free of bank conflicts both ways), so that eight lanes
+// write a row's 128 bytes (64 of C and 64 of Z for the bf16 outputs); a thread
+// writing its own row sends 16 bytes to each of 32 rows an instruction.
+template <int EPI>
+__device__ __forceinline__ void pair_store32(const TcArgs &g, int row0, int col0, int lane, float (&v)[32], uint4 *box) {
+    constexpr bool kBf16 = EPI == TC_GELU || EPI == TC_GELU_BWD;
+    if (EPI == TC_F32_BIAS || EPI == TC_GELU) {
+        const float4 *b = reinterpret_cast<const float4 *>(g.bias + col0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 x = __ldg(b + i);
+            v[4 * i] += x.x;
+            v[4 * i + 1] += x.y;
+            v[4 * i + 2] += x.z;
+            v[4 * i + 3] += x.w;
+        }
+    }
+    const int sw = lane & 7;
+    uint4 *mine = box + lane * 8;
+    if (EPI == TC_GELU_BWD) {
+        // Z of the block: four lanes a row
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = 8 * i + (lane >> 2), q = lane & 3;
+            if (row0 + r < g.M)
+                box[r * 8 + (q ^ (r & 7))] =
+                    *(reinterpret_cast<const uint4 *>(g.aux + (int64_t)(row0 + r) * g.ldc + col0) + q);
+        }
+        __syncwarp();
+    }
+    if (!kBf16) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            mine[q ^ sw] = make_uint4(__float_as_uint(v[4 * q]), __float_as_uint(v[4 * q + 1]),
+                                      __float_as_uint(v[4 * q + 2]), __float_as_uint(v[4 * q + 3]));
+    } else {
+        // slots 0-3: Z, 4-7: C
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            uint32_t z[4], c[4];
+            if (EPI == TC_GELU_BWD) {
+                const uint4 zz = mine[q ^ sw];
+                z[0] = zz.x;
+                z[1] = zz.y;
+                z[2] = zz.z;
+                z[3] = zz.w;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float a = v[8 * q + 2 * i], b = v[8 * q + 2 * i + 1];
+                if (EPI == TC_GELU) z[i] = pack_bf16(a, b);
+                const float2 zf = unpack_bf16(z[i]);
+                c[i] = EPI == TC_GELU ? pack_bf16(gelu_f(zf.x), gelu_f(zf.y))
+                                      : pack_bf16(a * gelu_grad(zf.x), b * gelu_grad(zf.y));
+            }
+            if (EPI == TC_GELU) mine[q ^ sw] = make_uint4(z[0], z[1], z[2], z[3]);
+            mine[(q + 4) ^ sw] = make_uint4(c[0], c[1], c[2], c[3]);
+        }
+    }
+    __syncwarp();
+    const int q = lane & 7;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = 4 * i + (lane >> 3);
+        if (row0 + r >= g.M) break;
+        const int64_t o = (int64_t)(row0 + r) * g.ldc + col0;
+        uint4 x = box[r * 8 + (q ^ (r & 7))];
+        if (!kBf16) {
+            uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<float *>(g.C) + o) + q;
+            if (EPI == TC_F32_ACCUM) {
+                const uint4 old = *dst;
+                x.x = __float_as_uint(__uint_as_float(x.x) + __uint_as_float(old.x));
+                x.y = __float_as_uint(__uint_as_float(x.y) + __uint_as_float(old.y));
+                x.z = __float_as_uint(__uint_as_float(x.z) + __uint_as_float(old.z));
+                x.w = __float_as_uint(__uint_as_float(x.w) + __uint_as_float(old.w));
+            }
+            *dst = x;
+        } else if (q >= 4) {
+            *(reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(g.C) + o) + (q - 4)) = x;
+        } else if (EPI == TC_GELU) {
+            *(reinterpret_cast<uint4 *>(g.aux + o) + q) = x;
+        }
+    }
+    __syncwarp();
+}
+
+template <int EPI>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+    tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, TcArgs g) {
+    extern __shared__ uint8_t smem_tc[];
+    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_tc) + 1023) & ~uintptr_t(1023));
+    uint8_t *boxes = base + kPairStages * kPairStageBytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(boxes + kPairEpiWarps * kPairBox);
+    uint64_t *empty = full + kPairStages;
+    uint64_t *tfull = empty + kPairStages;  // [2]
+    uint64_t *tempty = tfull + 2;           // [2]
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tempty + 2);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+    const int nk = (g.K + BK - 1) / BK;
+    const int ntn = (g.N + BN - 1) / BN;
+    const int ntiles = ((g.M + 2 * BM - 1) / (2 * BM)) * ntn;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kPairStages; ++s) {
+            mbar_init(full + s, 1);
+            mbar_init(empty + s, 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(tfull + a, 1);
+            mbar_init(tempty + a, 2 * kPairEpiWarps);
+        }
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(kPersistTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();  // both CTAs' barriers are initialised and their tensor memory is allocated
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // producer
+            uint32_t it = 0;
+            for (int t = pair; t < ntiles && !*abort_flag; t += npairs) {
+                const int m0 = (t / ntn) * 2 * BM + rank * BM, n0 = (t % ntn) * BN + rank * (BN / 2);
+                for (int kt = 0; kt < nk; ++kt, ++it) {
+                    const int s = it % kPairStages;
+                    const uint32_t ph = (it / kPairStages) & 1;
+                    if (it >= (uint32_t)kPairStages && !mbar_wait(empty + s, ph ^ 1)) {
+                        atomicExch(g.err, 1);
+                        *abort_flag = 1;
+                        break;
+                    }
+                    if (*abort_flag) break;
+                    if (rank == 0) mbar_expect_tx(full + s, 2 * kPairStageBytes);
+                    const uint32_t bar = cluster_addr(full + s, 0);
+                    uint8_t *st = base + s * kPairStageBytes;
+                    tma_load_pair(st, &ta, kt * BK, m0, bar);
+                    tma_load_pair(st + A_TILE, &tb, kt * BK, n0, bar);
+                }
+            }
+            // never leave with copies in flight: wait (bounded) until the last stages have been consumed
+            for (uint32_t q = (it > (uint32_t)kPairStages ? it - kPairStages : 0); q < it; ++q)
+                if (!mbar_wait(empty + (q % kPairStages), (q / kPairStages) & 1)) break;
+        }
+    } else if (warp == 1) {
+        if (lane == 0 && rank == 0) {
+            // MMA issuer of the pair
+            uint32_t it = 0;
+            int j = 0;
+            for (int t = pair; t < ntiles && !*abort_flag; t += npairs, ++j) {
+                const int acc = j & 1;
+                const int use = j >> 1;  // this accumulator's use count
+                if (use > 0 && !mbar_wait_cluster(tempty + acc, (use - 1) & 1)) {
+                    atomicExch(g.err, 4);
+                    *abort_flag = 1;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)(acc * BN);
+                for (int kt = 0; kt < nk; ++kt, ++it) {
+                    const int s = it % kPairStages;
+                    const uint32_t ph = (it / kPairStages) & 1;
+                    if (*abort_flag || !mbar_wait_cluster(full + s, ph)) {
+                        atomicExch(g.err, 2);
+                        *abort_flag = 1;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t a0 = smem_u32(base + s * kPairStageBytes), b0 = a0 + A_TILE;
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk)
+                        mma_pair(d, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), (kt > 0 || kk > 0) ? 1u : 0u);
+                    mma_commit_pair(empty + s);
+                }
+                if (*abort_flag) break;
+                mma_commit_pair(tfull + acc);  // arrives once this tile's MMAs have completed
+            }
+        }
+    } else {
+        // epilogue warps: this CTA's 128 rows, a quarter of them and a slice of the columns each
+        constexpr int kCols = BN * 4 / kPairEpiWarps;
+        const int q = warp & 3, c0 = ((warp - 2) >> 2) * kCols;
+        const bool vec = (g.ldc % 8) == 0 && ((reinterpret_cast<uintptr_t>(g.C) | reinterpret_cast<uintptr_t>(g.aux) |
+                                               reinterpret_cast<uintptr_t>(g.bias)) & 15) == 0;
+        uint4 *box = reinterpret_cast<uint4 *>(boxes + (warp - 2) * kPairBox);
+        int j = 0;
+        for (int t = pair; t < ntiles; t += npairs, ++j) {
+            const int acc = j & 1;
+            const bool ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(tfull + acc, (j >> 1) & 1));
+            if (!ok) {
+                if (lane == 0) {
+                    atomicExch(g.err, 3);
+                    *abort_flag = 1;
+                }
+                break;
+            }
+            tc_fence_after();
+            const int row0 = (t / ntn) * 2 * BM + rank * BM + q * 32, n0 = (t % ntn) * BN;
+            const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
+#pragma unroll 1
+            for (int c = c0; c < c0 + kCols; c += 32) {
+                if (row0 >= g.M || n0 + c >= g.N) break;
+                if (vec && n0 + c + 32 <= g.N) {
+                    float v[32];
+                    tmem_ld32(src + (uint32_t)c, v);
+                    pair_store32<EPI>(g, row0, n0 + c, lane, v, box);
+                } else {
+#pragma unroll 1
+                    for (int h = 0; h < 32; h += 16) {
+                        float v[16];
+                        tmem_ld16(src + (uint32_t)(c + h), v);
+                        tc_store16<EPI>(g, row0 + lane, n0 + c + h, v, vec);
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(cluster_addr(tempty + acc, 0));
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();  // the other CTA's loads, arrivals and tensor-memory reads are done too
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kPersistTmemCols)
                      : "memory");
     }
 }

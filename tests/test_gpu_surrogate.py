@@ -213,3 +213,22 @@ def test_softmax_row_lengths_and_alignment(K, offset):
     pd = p.astype(np.float64)
     kl = (pd * (np.log(np.where(pd > 0, pd, 1.0)) - np.log(ref)[None, :])).sum(axis=1)
     assert np.abs(losses.cpu().numpy() - kl).max() <= 2e-5
+
+
+@pytest.mark.parametrize("M,N,K", [(136, 8, 8), (256, 136, 64), (257, 256, 72), (384, 264, 392), (393, 129, 448),
+                                   (20000, 300, 520)])
+def test_gemm_tiles_of_cta_pairs(M, N, K):
+    """The 256 x 256 tiles of CTA pairs: one row past the first CTA's half, a
+    second CTA with rows or operand rows wholly outside, K within one stage,
+    around the ring's six and beyond, pairs that walk several tiles.  The sums
+    are exact: operands and bias are small integers, so any product lost,
+    doubled or misplaced shows."""
+    from paper_2602_11092_gb300 import surrogate as S
+    gen = torch.Generator().manual_seed(M + N + K)
+    A = torch.randint(-8, 9, (M, K), generator=gen).to(torch.bfloat16).cuda()
+    Bm = torch.randint(-8, 9, (N, K), generator=gen).to(torch.bfloat16).cuda()
+    bias = torch.randint(-8, 9, (N,), generator=gen).float().cuda()
+    C = torch.full((M, N), float("nan"), device="cuda")
+    S.gemm(A, Bm, S.GEMM_F32_BIAS, C=C, bias=bias)
+    S.sync_status()
+    assert torch.equal(C.double(), A.double() @ Bm.double().T + bias.double())
