@@ -26,7 +26,8 @@
 // copy of X needs a fixed workspace.
 //
 // One call, 4096 states of 2002 amplitudes: 818 us with TF32 operands (GEMM
-// 645, splits and their clearing 110, transfer matrix 47), 441 us now (315, 67, 43).
+// 645, splits and their clearing 110, transfer matrix 47), 441 us with FP16
+// pairs on single CTAs (315, 67, 43), 369 us with the tiles of CTA pairs.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -52,16 +53,23 @@ constexpr int kTransferThreads = 256;
 constexpr int kTransferRows = 4;  // input columns per block: they share the slot rows of the outputs
 
 // Layer k of the transfer matrix.  colmax (the last layer): per output t the
-// largest |re|, |im| over the inputs, as the bits of a non-negative float
-// (zeroed before the launch).
+// largest |re|, |im| over the inputs, as the bits of a non-negative float; the
+// layer before clears it (`clear`, nclear entries: a memset of its own cost 3 us
+// a call).
 template <int KW>
 __global__ void __launch_bounds__(kTransferThreads)
     transfer_kernel(const float2 *U, int m, const uint32_t *slots, const uint32_t *colinfo, int64_t Fk, int64_t Fp,
-                    const float2 *prev, float2 *cur, int first, unsigned int *colmax) {
+                    const float2 *prev, float2 *cur, int first, unsigned int *colmax, unsigned int *clear,
+                    int64_t nclear) {
     __shared__ float2 uc[kTransferRows][32];  // column c of U, zero past m (padding slots name mode kMaxModes)
     __shared__ int64_t from[kTransferRows];
     const int64_t s0 = (int64_t)blockIdx.y * kTransferRows;
     const int rows = (int)min((int64_t)kTransferRows, Fk - s0);
+    if (clear) {
+        const int64_t step = (int64_t)gridDim.x * gridDim.y * kTransferThreads;
+        for (int64_t i = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kTransferThreads + threadIdx.x; i < nclear; i += step)
+            clear[i] = 0u;
+    }
     if (threadIdx.x < kTransferRows * 32) {
         const int r = threadIdx.x >> 5, j = threadIdx.x & 31;
         if (r < rows) {
@@ -332,7 +340,7 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
     unsigned int *colmax = reinterpret_cast<unsigned int *>(ws + L.colmax);
     const float2 *Ud = reinterpret_cast<const float2 *>(U);
     cudaError_t e;
-    if ((e = cudaMemsetAsync(colmax, 0, (size_t)p->K * sizeof(unsigned int), s)) != cudaSuccess)
+    if (n == 1 && (e = cudaMemsetAsync(colmax, 0, (size_t)p->K * sizeof(unsigned int), s)) != cudaSuccess)
         return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
     {
         ProfScope ps("slos_transfer", 0.0, s);
@@ -342,12 +350,12 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
             const float2 *prev = k >= 2 ? buf[(n - k + 1) & 1] : nullptr;
             dim3 grid((unsigned)((Fk + kTransferThreads - 1) / kTransferThreads),
                       (unsigned)((Fk + kTransferRows - 1) / kTransferRows));
-            unsigned int *top = k == n ? colmax : nullptr;
+            unsigned int *top = k == n ? colmax : nullptr, *clr = k == n - 1 ? colmax : nullptr;
             const uint32_t *sl = p->tab.layer[k].slots, *ci = p->tab.layer[k].colinfo;
             switch (p->tab.layer[k].kw) {
-                case 4: transfer_kernel<4><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top); break;
-                case 8: transfer_kernel<8><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top); break;
-                default: transfer_kernel<12><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top); break;
+                case 4: transfer_kernel<4><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top, clr, p->K); break;
+                case 8: transfer_kernel<8><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top, clr, p->K); break;
+                default: transfer_kernel<12><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top, clr, p->K); break;
             }
             if ((e = cudaGetLastError()) != cudaSuccess)
                 return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
@@ -374,9 +382,8 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
             return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
         attr_done[dev] = true;
     }
-    CUtensorMap mah, mal, mbh, mbl;
-    if (!make_map_f16(&mbh, bhi, 2 * K, K2, K2, tc::kSpBN) || !make_map_f16(&mbl, blo, 2 * K, K2, K2, tc::kSpBN) ||
-        !make_map_f16(&mah, ahi, kEncodeChunk, K2, K2, tc::BM) || !make_map_f16(&mal, alo, kEncodeChunk, K2, K2, tc::BM))
+    CUtensorMap mah, mal;
+    if (!make_map_f16(&mah, ahi, kEncodeChunk, K2, K2, tc::BM) || !make_map_f16(&mal, alo, kEncodeChunk, K2, K2, tc::BM))
         return fail(SLOS_ERR_CUDA, "slos_encoded_forward: cuTensorMapEncodeTiled failed");
     const float2 *Xd = reinterpret_cast<const float2 *>(X);
     for (int b0 = 0; b0 < batch; b0 += kEncodeChunk) {
@@ -392,20 +399,24 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
             if ((e = cudaGetLastError()) != cudaSuccess)
                 return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
         }
-        tc::TcArgs g;
+        const int pairs = std::max(1, p->sm_count / 2);
+        tc::SplitArgs g;
         memset(&g, 0, sizeof(g));
         g.M = rows;
         g.N = (int)(2 * K);
         g.K = (int)K2;
-        g.ldc = (int)K;
+        g.bn = tc::split_columns(g.M, g.N, pairs);
         g.C = output == SLOS_OUT_AMPS ? (void *)(reinterpret_cast<float2 *>(out) + (int64_t)b0 * K)
                                       : (void *)(reinterpret_cast<float *>(out) + (int64_t)b0 * K);
         g.colscale = colscale;
         g.rowscale = rowscale;
         g.amps = output == SLOS_OUT_AMPS ? 1 : 0;
         g.err = p->d_status + 2;
-        const int64_t tiles = (int64_t)((g.N + tc::kSpBN - 1) / tc::kSpBN) * ((rows + tc::BM - 1) / tc::BM);
-        const unsigned grid = (unsigned)std::min<int64_t>(tiles, p->sm_count);
+        CUtensorMap mbh, mbl;
+        if (!make_map_f16(&mbh, bhi, 2 * K, K2, K2, g.bn / 2) || !make_map_f16(&mbl, blo, 2 * K, K2, K2, g.bn / 2))
+            return fail(SLOS_ERR_CUDA, "slos_encoded_forward: cuTensorMapEncodeTiled failed");
+        const int64_t tiles = (int64_t)((g.N + g.bn - 1) / g.bn) * ((rows + 2 * tc::BM - 1) / (2 * tc::BM));
+        const unsigned grid = 2 * (unsigned)std::min<int64_t>(tiles, pairs);
         ProfScope ps("slos_encode_gemm", 3.0 * 2.0 * rows * (double)g.N * (double)K2, s);  // flops
         tc::tc_gemm_split_kernel<<<grid, tc::kSpThreads, tc::kSpSmem, s>>>(mah, mbh, mal, mbl, g);
         if ((e = cudaGetLastError()) != cudaSuccess)

@@ -165,9 +165,6 @@ slos_status_t gemm(int epi, int M, int N, int K, const __nv_bfloat16 *A, int64_t
     g.bias = bias;
     g.aux = aux;
     g.err = err_ptr();
-    g.colscale = nullptr;
-    g.rowscale = nullptr;
-    g.amps = 0;
     ProfScope ps("tc_gemm", 2.0 * M * N * K, s);  // flops, not bytes
     switch (epi) {
         case TC_F32: launch_gemm<TC_F32>(pair, ta, tb, g, s); break;

@@ -41,8 +41,6 @@ enum TcEpi : int {
     TC_GELU = 2,       // Z = acc + bias[n] (bf16, aux), C = gelu(Z) (bf16)
     TC_GELU_BWD = 3,   // C = acc * gelu'(Z), Z = aux (bf16 in), C bf16
     TC_F32_ACCUM = 4,  // C += acc                        (float)
-    TC_ENCODE = 5,     // columns (2t, 2t+1) = (re, im) of output t: psi = rowscale[row] colscale[t] (re + i im);
-                       //   C float |psi|^2, or complex64 psi when amps (row stride ldc outputs)
 };
 
 struct TcArgs {
@@ -52,9 +50,6 @@ struct TcArgs {
     const float *bias;    // [N]
     __nv_bfloat16 *aux;   // [M][ldc] (Z for TC_GELU out, TC_GELU_BWD in)
     int *err;             // error word (device)
-    const float *colscale;  // TC_ENCODE: [N / 2]
-    const float *rowscale;  // TC_ENCODE: [M]
-    int amps;               // TC_ENCODE: complex64 output
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -155,22 +150,6 @@ __device__ __forceinline__ float gelu_grad(float z) {
 // accumulator values of row `row`, columns col0 .. col0 + 15.
 template <int EPI>
 __device__ __forceinline__ void tc_store16(const TcArgs &g, int row, int col0, float (&v)[16], bool vec) {
-    if (EPI == TC_ENCODE) {
-        if (row < g.M) {
-            const float rs = g.rowscale[row];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int t = col0 / 2 + i;
-                if (2 * t >= g.N) break;
-                const float c = g.colscale[t];
-                const float re = v[2 * i] * rs * c, im = v[2 * i + 1] * rs * c;  // rs a power of two
-                const int64_t o = (int64_t)row * g.ldc + t;
-                if (g.amps) reinterpret_cast<float2 *>(g.C)[o] = make_float2(re, im);
-                else reinterpret_cast<float *>(g.C)[o] = re * re + im * im;
-            }
-        }
-        return;
-    }
     if (row < g.M && col0 < g.N) {
         const int64_t o0 = (int64_t)row * g.ldc + col0;
         if (EPI == TC_F32_BIAS || EPI == TC_GELU) {
@@ -756,15 +735,18 @@ namespace tc {
 // operand value is scaled by a power of two of its row and split into two FP16
 // numbers, v = hi + lo (22 significant bits), and the product is
 // A_hi B_hi + A_hi B_lo + A_lo B_hi (the dropped lo lo term is ~2^-22 of it).
+// Columns 2t and 2t + 1 are re and im of output t: psi(row, t) = rowscale[row]
+// colscale[t] (re + i im); stored as |psi|^2, or as psi (complex64).
 //
-// A stage holds the hi and the lo tile of both operands for 64 values of K and
-// feeds all three products from them (12 MMAs).  The loads bound a GEMM of
-// 128 x 256 tiles here: one product per pair of tiles needs 96 bytes per clock
-// and SM at full tensor rate, against the 56 or so that the L2 delivers, the
-// shared stage 64.  TF32 operands in three passes over hi and lo copies, the
-// form before, need twice the MMAs (K = 8 each at half rate) and one load per
-// product: 645 us for 4096 x 2002 complex (611 TFLOP/s of MMA work),
-// 315 us now (1250 TFLOP/s).
+// CTA pairs as in tc_gemm_pair_kernel, tiles of 256 x bn; a stage holds the hi
+// and the lo tile of both operands for 64 values of K and feeds all three
+// products from them (12 MMAs).  Bound by the MMAs, so what is left to choose
+// is how evenly the tiles fill the pairs: bn (split_columns) is the multiple of
+// 32 up to 256 with the least waves x columns.  One call of encoded_forward, us,
+// with 128 x 256 tiles of single CTAs (two stages, outputs written a row a
+// thread) / now: 4096 states of 2002 amplitudes 441 / 371 (2 x 2002 columns in
+// tiles of 224 fill 3.8 of 4 waves, of 256 3.4), 120 of 120 33 / 26, 16 of 56
+// 25 / 23.
 //
 // The tensor core's FP32 accumulation does not round to nearest: over the
 // ~1500 MMAs of a long K its errors pile up in one direction (measured:
@@ -772,48 +754,103 @@ namespace tc {
 // accumulator took all of them).  So the K sum is taken in chunks of
 // kSpChunkStages stages: each chunk accumulates into one of two TMEM buffers
 // while the epilogue warps move the other buffer's finished chunk into FP32
-// registers (half a row, 128 columns, per thread; round-to-nearest adds).
-// Roles: warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue (TMEM lane
-// quarter = warp % 4, columns 0-127 for warps 2-5 and 128-255 for warps 6-9).
-// Waits are bounded as above.
-constexpr int kSpBN = 256;
-constexpr int kSpStages = 2;
+// registers (half a row, up to 128 columns, per thread; round-to-nearest adds).
+// Roles: warp 0 TMA producer, warp 1 MMA issuer (of the even CTA), warps 2-9
+// epilogue (TMEM lane quarter = warp % 4, the first half of the columns for
+// warps 2-5 and the second for warps 6-9).  Waits are bounded as above.
+constexpr int kSpStages = 3;
 constexpr int kSpChunkStages = 2;  // 24 MMAs per chunk
 constexpr int kSpThreads = 320;
 constexpr int kSpEpiWarps = 8;
-constexpr int kSpATile = BM * 128, kSpBTile = kSpBN * 128;  // bytes: 128-byte rows
-constexpr int kSpStageBytes = 2 * (kSpATile + kSpBTile);    // A hi, A lo, B hi, B lo
-constexpr int kSpSmem = kSpStages * kSpStageBytes + 1024 + 256;
-constexpr uint32_t kSpTmemCols = 2 * kSpBN;
-// kind::f16 with A and B FP16 (bits 7-9 = 0, 10-12 = 0), otherwise as kIdesc.
-constexpr uint32_t kIdescF16 = (1u << 4) | ((uint32_t)(kSpBN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+constexpr int kSpTile = BM * 128;             // bytes of 128 rows of an operand
+constexpr int kSpStageBytes = 4 * kSpTile;    // A hi, A lo, B hi, B lo
+constexpr int kSpBox = 32 * 9 * 8;            // an epilogue warp's block of 32 rows x 8 outputs, padded
+constexpr int kSpSmem = kSpStages * kSpStageBytes + kSpEpiWarps * kSpBox + 1024 + 256;
+constexpr uint32_t kSpTmemCols = 2 * BN;
 
-__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+struct SplitArgs {
+    int M, N, K;  // N = 2 x outputs
+    int bn;       // columns of a tile: a multiple of 32, at most 256
+    void *C;      // [M][N / 2] float or complex64
+    int amps;
+    const float *colscale, *rowscale;
+    int *err;
+};
+
+// Columns of a tile for M x N outputs on `pairs` CTA pairs: the least time of
+// waves x (columns + 32; the fixed cost of a wave in columns), the widest of equals.
+inline int split_columns(int M, int N, int pairs) {
+    int best = BN;
+    int64_t least = INT64_MAX;
+    for (int bn = BN; bn >= 32; bn -= 32) {
+        const int64_t tiles = (int64_t)((N + bn - 1) / bn) * ((M + 2 * BM - 1) / (2 * BM));
+        const int64_t cost = (tiles + pairs - 1) / pairs * (bn + 32);
+        if (cost < least) {
+            least = cost;
+            best = bn;
+        }
+    }
+    return best;
+}
+
+__device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(kIdescF16), "r"(accumulate)
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
-static __global__ void __launch_bounds__(kSpThreads, 1)
+// 32 rows x 16 columns (8 outputs) by a warp: v holds row row0 + lane.  Turned
+// in `box` so that eight lanes write a row's eight outputs.
+__device__ __forceinline__ void split_store(const SplitArgs &g, int row0, int col0, int lane, const float *v,
+                                            float2 *box) {
+    const int t0 = col0 / 2, outs = g.N / 2;
+    const float rs = row0 + lane < g.M ? __ldg(g.rowscale + row0 + lane) : 0.f;
+    float *boxf = reinterpret_cast<float *>(box);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float c = t0 + i < outs ? __ldg(g.colscale + t0 + i) : 0.f;
+        const float re = v[2 * i] * rs * c, im = v[2 * i + 1] * rs * c;  // rs a power of two
+        if (g.amps) box[lane * 9 + i] = make_float2(re, im);
+        else boxf[lane * 9 + i] = re * re + im * im;
+    }
+    __syncwarp();
+    const int i = lane & 7;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        const int r = 4 * p + (lane >> 3);
+        if (row0 + r < g.M && t0 + i < outs) {
+            const int64_t o = (int64_t)(row0 + r) * outs + t0 + i;
+            if (g.amps) reinterpret_cast<float2 *>(g.C)[o] = box[r * 9 + i];
+            else reinterpret_cast<float *>(g.C)[o] = boxf[r * 9 + i];
+        }
+    }
+    __syncwarp();
+}
+
+static __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1)
     tc_gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                          const __grid_constant__ CUtensorMap ta_lo, const __grid_constant__ CUtensorMap tb_lo,
-                         TcArgs g) {
+                         SplitArgs g) {
     extern __shared__ uint8_t smem_tc[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_tc) + 1023) & ~uintptr_t(1023));
-    uint64_t *full = reinterpret_cast<uint64_t *>(base + kSpStages * kSpStageBytes);
+    uint8_t *boxes = base + kSpStages * kSpStageBytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(boxes + kSpEpiWarps * kSpBox);
     uint64_t *empty = full + kSpStages;
     uint64_t *cfull = empty + kSpStages;  // [2] a chunk's MMAs are done
-    uint64_t *cempty = cfull + 2;         // [2] the epilogue has taken the chunk
+    uint64_t *cempty = cfull + 2;         // [2] the epilogue warps of both CTAs have taken the chunk
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(cempty + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+    const int bn = g.bn;
     const int nk = (g.K + BK - 1) / BK;
     const int nchunks = (nk + kSpChunkStages - 1) / kSpChunkStages;
-    const int ntn = (g.N + kSpBN - 1) / kSpBN;
-    const int ntiles = ((g.M + BM - 1) / BM) * ntn;
+    const int ntn = (g.N + bn - 1) / bn;
+    const int ntiles = ((g.M + 2 * BM - 1) / (2 * BM)) * ntn;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kSpStages; ++s) {
@@ -822,28 +859,30 @@ static __global__ void __launch_bounds__(kSpThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(cfull + a, 1);
-            mbar_init(cempty + a, kSpEpiWarps);
+            mbar_init(cempty + a, 2 * kSpEpiWarps);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(kSpTmemCols)
                      : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
+    cluster_sync();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
         if (lane == 0) {
             // producer: every stage of every tile, in order
+            const uint32_t bytes = 2u * 2u * (uint32_t)(kSpTile + bn / 2 * 128);  // of both CTAs
             uint32_t it = 0;
-            for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
-                const int m0 = (t / ntn) * BM, n0 = (t % ntn) * kSpBN;
+            for (int t = pair; t < ntiles && !*abort_flag; t += npairs) {
+                const int m0 = (t / ntn) * 2 * BM + rank * BM, n0 = (t % ntn) * bn + rank * (bn / 2);
                 for (int kt = 0; kt < nk; ++kt, ++it) {
                     const int s = it % kSpStages;
                     const uint32_t ph = (it / kSpStages) & 1;
@@ -853,67 +892,72 @@ static __global__ void __launch_bounds__(kSpThreads, 1)
                         break;
                     }
                     if (*abort_flag) break;
+                    if (rank == 0) mbar_expect_tx(full + s, bytes);
+                    const uint32_t bar = cluster_addr(full + s, 0);
                     uint8_t *st = base + s * kSpStageBytes;
-                    mbar_expect_tx(full + s, kSpStageBytes);
-                    tma_load_2d(st, &ta, kt * BK, m0, full + s);
-                    tma_load_2d(st + 2 * kSpATile, &tb, kt * BK, n0, full + s);
-                    tma_load_2d(st + 2 * kSpATile + kSpBTile, &tb_lo, kt * BK, n0, full + s);
-                    tma_load_2d(st + kSpATile, &ta_lo, kt * BK, m0, full + s);
+                    tma_load_pair(st, &ta, kt * BK, m0, bar);
+                    tma_load_pair(st + 2 * kSpTile, &tb, kt * BK, n0, bar);
+                    tma_load_pair(st + 3 * kSpTile, &tb_lo, kt * BK, n0, bar);
+                    tma_load_pair(st + kSpTile, &ta_lo, kt * BK, m0, bar);
                 }
             }
+            // never leave with copies in flight: wait (bounded) until the last stages have been consumed
             for (uint32_t q = (it > (uint32_t)kSpStages ? it - kSpStages : 0); q < it; ++q)
-                mbar_wait(full + (q % kSpStages), (q / kSpStages) & 1);
+                if (!mbar_wait(empty + (q % kSpStages), (q / kSpStages) & 1)) break;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // MMA issuer: chunk c of the CTA's walk goes to buffer c & 1
-            uint32_t it = 0, c = 0;
-            for (int t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
-                for (int ch = 0; ch < nchunks && !*abort_flag; ++ch, ++c) {
+        if (lane == 0 && rank == 0) {
+            // FP32 accumulator (bits 4-5 = 1), A and B FP16 (0), N >> 3 (bits 17-22), M >> 4 (bits 24-28)
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
+            uint32_t it = 0, c = 0;  // stages and chunks over all tiles
+            for (int t = pair; t < ntiles && !*abort_flag; t += npairs) {
+                for (int ch = 0; ch < nchunks; ++ch, ++c) {
                     const int b = c & 1;
                     const uint32_t use = c >> 1;
-                    if (use > 0 && !mbar_wait(cempty + b, (use - 1) & 1)) {
+                    if (use > 0 && !mbar_wait_cluster(cempty + b, (use - 1) & 1)) {
                         atomicExch(g.err, 4);
                         *abort_flag = 1;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(b * kSpBN);
+                    const uint32_t d = tmem + (uint32_t)(b * BN);
                     const int k1 = min(nk, (ch + 1) * kSpChunkStages);
                     for (int kt = ch * kSpChunkStages; kt < k1; ++kt, ++it) {
                         const int s = it % kSpStages;
                         const uint32_t ph = (it / kSpStages) & 1;
-                        if (*abort_flag || !mbar_wait(full + s, ph)) {
+                        if (*abort_flag || !mbar_wait_cluster(full + s, ph)) {
                             atomicExch(g.err, 2);
                             *abort_flag = 1;
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t ah = smem_u32(base + s * kSpStageBytes), al = ah + kSpATile;
-                        const uint32_t bh = ah + 2 * kSpATile, bl = bh + kSpBTile;
+                        const uint32_t ah = smem_u32(base + s * kSpStageBytes), al = ah + kSpTile;
+                        const uint32_t bh = ah + 2 * kSpTile, bl = ah + 3 * kSpTile;
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
                             const uint64_t dah = sw128_desc(ah + kk * 32), dal = sw128_desc(al + kk * 32);
                             const uint64_t dbh = sw128_desc(bh + kk * 32), dbl = sw128_desc(bl + kk * 32);
-                            mma_f16(d, dal, dbh, (kt > ch * kSpChunkStages || kk > 0) ? 1u : 0u);
-                            mma_f16(d, dah, dbl, 1u);
-                            mma_f16(d, dah, dbh, 1u);
+                            mma_f16_pair(d, dal, dbh, idesc, (kt > ch * kSpChunkStages || kk > 0) ? 1u : 0u);
+                            mma_f16_pair(d, dah, dbl, idesc, 1u);
+                            mma_f16_pair(d, dah, dbh, idesc, 1u);
                         }
-                        mma_commit(empty + s);
+                        mma_commit_pair(empty + s);
                     }
                     if (*abort_flag) break;
-                    mma_commit(cfull + b);
+                    mma_commit_pair(cfull + b);
                 }
             }
         }
     } else {
-        // epilogue warps: each thread sums 128 columns of its row over the chunks
-        constexpr int HC = kSpBN / 2;
+        // epilogue warps: each thread sums half of its row's columns over the chunks
+        constexpr int HC = BN / 2;
+        const int hn = bn / 2;  // columns of a half, a multiple of 16
         const int q = warp & 3;
         const int hc = (warp - 2) >> 2;  // column half
+        float2 *box = reinterpret_cast<float2 *>(boxes + (warp - 2) * kSpBox);
         uint32_t c = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        for (int t = pair; t < ntiles && ok; t += npairs) {
             float acc[HC];
 #pragma unroll
             for (int i = 0; i < HC; ++i) acc[i] = 0.f;
@@ -928,35 +972,34 @@ static __global__ void __launch_bounds__(kSpThreads, 1)
                     break;
                 }
                 tc_fence_after();
-                const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * kSpBN + hc * HC);
+                const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + hc * hn);
 #pragma unroll
                 for (int c16 = 0; c16 < HC; c16 += 16) {
-                    float v[16];
-                    tmem_ld16(src + (uint32_t)c16, v);
+                    if (c16 < hn) {
+                        float v[16];
+                        tmem_ld16(src + (uint32_t)c16, v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[c16 + i] += v[i];
+                        for (int i = 0; i < 16; ++i) acc[c16 + i] += v[i];
+                    }
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(cempty + b);
+                if (lane == 0) mbar_arrive_cluster(cluster_addr(cempty + b, 0));
             }
             if (!ok) break;
-            const int m0 = (t / ntn) * BM, n0 = (t % ntn) * kSpBN + hc * HC;
-            const int row = m0 + q * 32 + lane;
+            const int row0 = (t / ntn) * 2 * BM + rank * BM + q * 32, n0 = (t % ntn) * bn + hc * hn;
 #pragma unroll
-            for (int c16 = 0; c16 < HC; c16 += 16) {
-                float v[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = acc[c16 + i];
-                tc_store16<TC_ENCODE>(g, row, n0 + c16, v, false);
-            }
+            for (int c16 = 0; c16 < HC; c16 += 16)
+                if (c16 < hn && n0 + c16 < g.N && row0 < g.M) split_store(g, row0, n0 + c16, lane, acc + c16, box);
         }
     }
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
+    cluster_sync();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSpTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSpTmemCols) : "memory");
     }
 }
 

@@ -119,3 +119,24 @@ def test_encoded_rows_and_outputs_of_any_scale(slos, m, n, B):
     bound = 4e-6 * np.sqrt(K) * norm[:, None] * size[None, :]
     assert np.all(np.abs(amps - ref) <= bound + 1e-44)
     assert np.all(amps[B // 2] == 0)
+
+
+@pytest.mark.parametrize("m,n,B", [(3, 1, 1), (6, 3, 130), (7, 3, 257), (8, 4, 513), (9, 4, 40), (10, 4, 300), (9, 5, 1100)])
+@pytest.mark.parametrize("kind", ["amps", "probs"])
+def test_encoded_tile_widths(slos, m, n, B, kind):
+    """Output counts and batches whose tiles take widths from 32 to 256
+    columns, ragged in both directions and odd row lengths, against the FP64
+    product with the transfer matrix."""
+    rng = np.random.default_rng(m * 100 + B)
+    plan = slos.Plan(m, [n] + [0] * (m - 1))
+    basis = oracle.enumerate_fock(m, n)
+    U = workloads.haar_unitaries(m, 1, rng)[0].astype(np.complex64)
+    X = rand_states(rng, B, plan.n_outputs).astype(np.complex64)
+    out = slos.AMPS if kind == "amps" else slos.PROBS
+    got = plan.encoded_forward(torch.tensor(U, device="cuda"), torch.tensor(X, device="cuda"), out).cpu().numpy()
+    ref = X.astype(np.complex128) @ oracle.transfer_matrix(U.astype(np.complex128), basis).T
+    # the split's 2^-22 and the FP32 recursion and sums, on amplitudes of norm 1
+    if kind == "amps":
+        assert np.abs(got - ref).max() <= 4e-6
+    else:
+        assert np.abs(got - np.abs(ref) ** 2).max() <= 8e-6
