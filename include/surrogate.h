@@ -33,7 +33,8 @@ typedef struct surr_model_s *surr_model_t;
 
 /* Tensor-core GEMM (tcgen05 + TMA + TMEM): C[M][N] = A[M][K] . B[N][K]^T with
  * A, B BF16 row-major (row strides lda, ldb elements; K, lda, ldb multiples
- * of 8; 16-byte aligned), FP32 accumulation.  Epilogue `epi`:
+ * of 8; 16-byte aligned), FP32 accumulation; C, bias and aux need only their
+ * elements' alignment.  Epilogue `epi`:
  *   0: C = acc (float [M][ldc])          1: C = acc + bias[n] (float)
  *   2: aux = bf16(acc + bias[n]), C = bf16(gelu(aux))   (GELU, tanh form)
  *   3: C = bf16(acc * gelu'(aux))         4: C += acc (float)

@@ -339,7 +339,8 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
     } else {
         // epilogue warps
         const int q = warp & 3;
-        const bool vec = (g.ldc % 8) == 0;
+        // 16-byte stores where every row of C starts on a 16-byte boundary (its epilogues touch only C)
+        const bool vec = (g.ldc % 8) == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
         int j = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++j) {
             const int acc = j & 1;

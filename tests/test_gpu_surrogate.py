@@ -232,3 +232,25 @@ def test_gemm_tiles_of_cta_pairs(M, N, K):
     S.gemm(A, Bm, S.GEMM_F32_BIAS, C=C, bias=bias)
     S.sync_status()
     assert torch.equal(C.double(), A.double() @ Bm.double().T + bias.double())
+
+
+@pytest.mark.parametrize("M,N", [(256, 264), (5000, 2304)])  # one wave of single CTAs, CTA pairs over several tiles
+@pytest.mark.parametrize("off", [0, 1, 2, 4])
+def test_plain_gemm_with_an_output_on_any_float(M, N, off):
+    """Plain and accumulating products into a C that starts `off` floats past
+    a 16-byte boundary: vector stores only where its rows allow them.  Exact:
+    small integers."""
+    from paper_2602_11092_gb300 import surrogate as S
+    K = 72
+    gen = torch.Generator().manual_seed(M + off)
+    A = torch.randint(-8, 9, (M, K), generator=gen).to(torch.bfloat16).cuda()
+    Bm = torch.randint(-8, 9, (N, K), generator=gen).to(torch.bfloat16).cuda()
+    ref = A.double() @ Bm.double().T
+    buf = torch.full((M * N + 8,), 3.0, device="cuda")
+    C = buf[off:off + M * N].view(M, N)
+    S.gemm(A, Bm, S.GEMM_F32, C=C)
+    assert torch.equal(C.double(), ref)
+    S.gemm(A, Bm, S.GEMM_F32_ACCUM, C=C)
+    S.sync_status()
+    assert torch.equal(C.double(), 2 * ref)
+    assert torch.all(buf[:off] == 3.0) and torch.all(buf[off + M * N:] == 3.0)
