@@ -332,7 +332,8 @@ slos_status_t slos_batched_plan(int count, const int *m, const int *n, const int
                                 const slos_detection_t *detection, slos_plan_t *out);
 
 /* u_offsets / out_offsets: host arrays of count + 1 int64 (the last entry is
- * the total).  workspace_bytes: device scratch for slos_batched_forward. */
+ * the total).  workspace_bytes: device scratch for slos_batched_forward, at
+ * any address. */
 slos_status_t slos_batched_query(slos_plan_t plan, int64_t *u_offsets, int64_t *out_offsets,
                                  size_t *workspace_bytes);
 

@@ -60,6 +60,7 @@ slos_status_t fail(slos_status_t st, const std::string &msg);
 
 constexpr int kBMax = 20;   // modes handled by the persistent kernel (m <= 20)
 constexpr int kBInst = 4;   // instances per lane group
+constexpr size_t kBRowBytes = kBInst * sizeof(float2);  // a state of a lane group: one 32-byte sector
 constexpr uint32_t kSlotEmpty = (uint32_t)kBMax;   // parent 0, mode kBMax (a zero row of U)
 constexpr int64_t kBMaxParent = int64_t(1) << 27;  // parent ranks in 27 bits
 constexpr int kBSec = 12;   // one section per occupied-mode count 1..12
@@ -648,8 +649,11 @@ static slos_status_t batched_launch(slos_plan_s *p, const void *U, float *out, v
     slos_status_t st = build_items(b, chunk);
     if (st != SLOS_OK) return st;
     const size_t need = b->layer_bytes + b->ctrl_bytes;
-    if (ws_bytes < need || !ws) return fail(SLOS_ERR_INVALID_ARG, "slos_batched_forward: workspace too small");
-    char *w = reinterpret_cast<char *>(ws);
+    // layer rows are read as float4 and are one sector each: start at the workspace's first sector boundary
+    char *w = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(ws) + kBRowBytes - 1) & ~uintptr_t(kBRowBytes - 1));
+    const size_t skipped = (size_t)(w - reinterpret_cast<char *>(ws));
+    if (!ws || ws_bytes < skipped + need)
+        return fail(SLOS_ERR_INVALID_ARG, "slos_batched_forward: workspace too small");
     unsigned long long *head = reinterpret_cast<unsigned long long *>(w + b->layer_bytes);
     int *done = reinterpret_cast<int *>(w + b->layer_bytes + align_up(sizeof(unsigned long long)));
     cudaError_t e;
@@ -956,7 +960,8 @@ slos_status_t slos_batched_query(slos_plan_t p, int64_t *u_offsets, int64_t *out
     if (out_offsets) memcpy(out_offsets, b->out_off.data(), b->out_off.size() * sizeof(int64_t));
     if (workspace_bytes) {
         // enough for the largest chunk the autotuner tries (smallest chunk = most descriptors is the same count)
-        *workspace_bytes = b->layer_bytes + align_up(sizeof(unsigned long long)) +
+        // (and room to start on a sector boundary)
+        *workspace_bytes = kBRowBytes + b->layer_bytes + align_up(sizeof(unsigned long long)) +
                            align_up((size_t)b->lgs.size() * (kMaxPhotons + 1) * sizeof(int));
     }
     return SLOS_OK;

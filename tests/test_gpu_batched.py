@@ -313,3 +313,24 @@ def test_batched_groups_of_four_and_patterns_across_windows(slos):
         ref = plan.forward(torch.tensor(Us[i][None], dtype=torch.complex64, device="cuda"))[0]
         # sums of positive terms in another order: a few ulps of each value
         assert torch.allclose(first[bp.out_offsets[i]:bp.out_offsets[i + 1]], ref, rtol=1e-5, atol=1e-9)
+
+
+@pytest.mark.parametrize("off", [1, 8, 16, 24, 32])
+def test_uneven_workspace_on_any_address(slos, off):
+    """A workspace of the queried size at any address (cudaMalloc's alignment
+    is not asked for): the layer rows start at its first sector boundary, the
+    outputs are the same bit for bit; a workspace too small is refused."""
+    inst = [workloads.UnevenInstance(m, n, workloads.even_mode_input(m, n), thr)
+            for m, n, thr in [(6, 3, False), (8, 4, True), (10, 5, False), (6, 3, False)]]
+    rng = np.random.default_rng(off)
+    U = pack([workloads.haar_unitaries(it.m, 1, rng)[0] for it in inst])
+    bp = make_plan(slos, inst)
+    buf = torch.empty(bp.workspace_bytes + 64, dtype=torch.uint8, device="cuda")
+    ref = torch.empty(bp.out_offsets[-1], device="cuda")
+    got = torch.full_like(ref, -1.0)
+    bp.forward(U, ref, buf)
+    bp.forward(U, got, buf[off:off + bp.workspace_bytes])
+    bp.sync_status()
+    assert torch.equal(ref, got)
+    with pytest.raises(slos.SlosError):
+        bp.forward(U, got, buf[off:off + 64])
