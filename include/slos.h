@@ -281,10 +281,15 @@ slos_status_t slos_fidelity_kernel(int m, const int *input_state, const void *Ua
  * The call builds the n-photon transfer matrix of U (K x K) layer by layer
  * with the photon-by-photon recursion, in the workspace, then applies it to
  * the batch's vectors with one complex GEMM.  One U for the whole batch.
+ * Every entry of the matrix and every component of a vector enters the sums
+ * with its 24 significant bits, however small it is beside the others.
  * PNR plans with K <= 32768 outputs (tables built at plan time); forward only.
  * ---------------------------------------------------------------------- */
 
-/* Device scratch bytes slos_encoded_forward needs (K^2 + F_{n-1}^2 complex64). */
+/* Device scratch bytes slos_encoded_forward needs: the transfer matrices of
+ * the last two layers (K^2 + F_{n-1}^2 complex64), and the GEMM's operands as
+ * three BF16 copies each (24 K^2 bytes of the matrix, 49152 K of a chunk of
+ * 4096 vectors). */
 slos_status_t slos_encoded_workspace_bytes(slos_plan_t plan, size_t *bytes);
 
 /* U: complex64 [m][m]; X: complex64 [batch][n_outputs] input amplitudes;

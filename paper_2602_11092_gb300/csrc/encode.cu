@@ -17,20 +17,23 @@
 // x_s = X[b][s] / g_s, A = A_n, its output columns interleaved (2t = re,
 // 2t + 1 = im of output t) so the epilogue forms g_t (Yr + i Yi) and its
 // |.|^2 from adjacent columns of one row.  For FP32-accurate products on the
-// FP16 tensor path (tc_gemm_split_kernel) every operand value is scaled by a
-// power of two, one per row of X and one per output t, that brings the row's
-// largest magnitude to [2^14, 2^15), and split into hi = v rounded to FP16 and
-// lo = (v - hi) rounded to FP16: 22 significant bits down to 2^-18 of the
-// row's largest value, an absolute 2^-40 of it below.  The epilogue undoes
-// both scales.  The batch runs in chunks of kEncodeChunk rows, so the split
+// 16-bit tensor path (tc_gemm_split_kernel) every operand value is split into
+// three BF16 numbers, which hold an FP32 value's 24 significant bits whatever
+// its size: a component of a state vector keeps its relative accuracy however
+// small it is beside the others (a map that does not mix hands it straight to
+// its output).  A power of two per row of X and one per output t first brings
+// the row's largest magnitude to [2^50, 2^51), so that products of small
+// vectors and small outputs stay far above FP32's subnormals; the epilogue
+// undoes both.  The batch runs in chunks of kEncodeChunk rows, so the split
 // copy of X needs a fixed workspace.
 //
-// One call, 4096 states of 2002 amplitudes: 818 us with TF32 operands (GEMM
-// 645, splits and their clearing 110, transfer matrix 47), 441 us with FP16
-// pairs on single CTAs (315, 67, 43), 369 us with the tiles of CTA pairs.
+// One call, 4096 states of 2002 amplitudes: 818 us with TF32 pairs on single
+// CTAs (GEMM 645, splits and their clearing 110, transfer matrix 47), now
+// 577 us.  FP16 pairs (three products instead of six) take 369 us, but share
+// an exponent range of 2^-40 over a row and lose what lies below it.
 #include <cuda.h>
 #include <cudaTypedefs.h>
-#include <cuda_fp16.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -112,34 +115,42 @@ __global__ void __launch_bounds__(kTransferThreads)
 }
 
 // Exponent of the power of two that brings a row whose largest magnitude has
-// these bits to [2^14, 2^15); 0 for rows of zeros and of values that are not
-// finite (their products are not either, whatever the scale).
+// these bits to [2^kSplitTarget, 2^(kSplitTarget + 1)); 0 for rows of zeros and
+// of values that are not finite (their products are not either, whatever the
+// scale).  Sums of 2^16 products stay below 2^118, and a value keeps its three
+// parts normal down to 2^-160 of its row's largest.
 __device__ __forceinline__ int split_exponent(unsigned int bits) {
     if (bits == 0u || bits >= 0x7f800000u) return 0;
-    return max(-126, min(126, 14 - ilogbf(__uint_as_float(bits))));
+    return min(126, tc::kSplitTarget - ilogbf(__uint_as_float(bits)));
 }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
-// v (scaled) = hi + lo in FP16.
-__device__ __forceinline__ void f16_split(float v, __half &hi, __half &lo) {
-    hi = __float2half_rn(v);
-    lo = __float2half_rn(v - __half2float(hi));
+// v = p[0] + p[1] + p[2] in BF16.
+constexpr int kParts = tc::kSpParts;
+__device__ __forceinline__ void bf16_split(float v, __nv_bfloat16 (&p)[kParts]) {
+#pragma unroll
+    for (int i = 0; i < kParts; ++i) {
+        p[i] = __float2bfloat16_rn(v);
+        v -= __bfloat162float(p[i]);
+    }
 }
 
 constexpr int kEncodeChunk = 4096;  // batch rows per GEMM launch
-constexpr int kEncodeKAlign = 64;   // K' padded to whole 128-byte FP16 stage rows
+constexpr int kEncodeKAlign = 64;   // K' padded to whole 128-byte stage rows
 
 // Real-form operand B of the GEMM, [N = 2K rows][K2 cols], K-major:
 //   row 2t:     cols s -> Ar[s][t],  K + s -> -Ai[s][t],  2K .. K2-1 -> 0
 //   row 2t + 1: cols s -> Ai[s][t],  K + s ->  Ar[s][t]
-// scaled and split into hi and lo copies; 32 x 32 tiles of A through shared
-// memory, so both the read (along t) and the writes (along s) are coalesced.
-// colscale[t] = g_t over t's scale.
+// scaled and split into kParts copies, each 2K rows after the one before;
+// 32 x 32 tiles of A through shared memory, so both the read (along t) and the
+// writes (along s) are coalesced.  colscale[t] = g_t times t's share of the
+// scale's inverse.
 __global__ void __launch_bounds__(256) encode_split_b_kernel(const float2 *A, int64_t K, int64_t K2,
-                                                             const unsigned int *colmax, const float *g, __half *bhi,
-                                                             __half *blo, float *colscale) {
+                                                             const unsigned int *colmax, const float *g,
+                                                             __nv_bfloat16 *bsplit, float *colscale) {
     __shared__ float2 tile[32][33];
     const int64_t s0 = (int64_t)blockIdx.y * 32, t0 = (int64_t)blockIdx.x * 32;
+    const int64_t part = 2 * K * K2;
     for (int i = threadIdx.y; i < 32; i += 8) {
         const int64_t ss = s0 + i, tt = t0 + threadIdx.x;
         tile[i][threadIdx.x] = (ss < K && tt < K) ? A[ss * K + tt] : make_float2(0.f, 0.f);
@@ -149,34 +160,36 @@ __global__ void __launch_bounds__(256) encode_split_b_kernel(const float2 *A, in
         const int64_t tt = t0 + i, ss = s0 + threadIdx.x;
         if (tt >= K) continue;
         const int ex = split_exponent(__ldg(colmax + tt));
-        if (blockIdx.y == 0 && threadIdx.x == 0) colscale[tt] = g[tt] * pow2f(-ex);
+        if (blockIdx.y == 0 && threadIdx.x == 0) colscale[tt] = g[tt] * pow2f(tc::kSplitTarget - ex);
         if (blockIdx.y + 1 == gridDim.y) {
             for (int64_t c = 2 * K + threadIdx.x; c < K2; c += 32)
-                bhi[2 * tt * K2 + c] = blo[2 * tt * K2 + c] = bhi[(2 * tt + 1) * K2 + c] = blo[(2 * tt + 1) * K2 + c] =
-                    __float2half_rn(0.f);
+#pragma unroll
+                for (int p = 0; p < kParts; ++p)
+                    bsplit[p * part + 2 * tt * K2 + c] = bsplit[p * part + (2 * tt + 1) * K2 + c] =
+                        __float2bfloat16_rn(0.f);
         }
         if (ss >= K) continue;
         const float sc = pow2f(ex);
         const float2 v = tile[threadIdx.x][i];  // A[ss][tt]
-        __half rh, rl, ih, il;
-        f16_split(v.x * sc, rh, rl);
-        f16_split(v.y * sc, ih, il);
-        const int64_t o = 2 * tt * K2 + ss;
-        bhi[o] = rh;
-        blo[o] = rl;
-        bhi[o + K] = __hneg(ih);
-        blo[o + K] = __hneg(il);
-        bhi[o + K2] = ih;
-        blo[o + K2] = il;
-        bhi[o + K2 + K] = rh;
-        blo[o + K2 + K] = rl;
+        __nv_bfloat16 re[kParts], im[kParts];
+        bf16_split(v.x * sc, re);
+        bf16_split(v.y * sc, im);
+#pragma unroll
+        for (int p = 0; p < kParts; ++p) {
+            __nv_bfloat16 *o = bsplit + p * part + 2 * tt * K2 + ss;
+            o[0] = re[p];
+            o[K] = __hneg(im[p]);
+            o[K2] = im[p];
+            o[K2 + K] = re[p];
+        }
     }
 }
 
 // Real-form operand A of the GEMM for batch rows [b0, b0 + rows), T threads
 // per row: [rows][K2], cols s -> Re X[b][s] / g_s, K + s -> Im X[b][s] / g_s,
-// the padding columns 2K .. K2-1 zero; scaled and split into hi and lo copies.
-// rowscale[r] = 1 over the row's scale.  T = 32 (a warp per row, no barrier)
+// the padding columns 2K .. K2-1 zero; scaled and split into kParts copies,
+// each kEncodeChunk rows after the one before.  rowscale[r] = the row's share
+// of its scale's inverse.  T = 32 (a warp per row, no barrier)
 // up to kSplitWarpRow values, a block per row beyond (1657 rows of 56: a block
 // each cost 3 us more than a warp each).
 constexpr int kSplitThreads = 256;
@@ -184,8 +197,8 @@ constexpr int kSplitKeep = 8;  // values per thread kept in registers between th
 constexpr int64_t kSplitWarpRow = 32 * kSplitKeep;
 template <int T>
 __global__ void __launch_bounds__(kSplitThreads) encode_split_a_kernel(const float2 *X, const float *g, int64_t b0,
-                                                                       int rows, int64_t K, int64_t K2, __half *ahi,
-                                                                       __half *alo, float *rowscale) {
+                                                                       int rows, int64_t K, int64_t K2,
+                                                                       __nv_bfloat16 *asplit, float *rowscale) {
     __shared__ unsigned int red[kSplitThreads / 32];
     const int64_t r = (int64_t)blockIdx.x * (kSplitThreads / T) + threadIdx.x / T;
     if (r >= rows) return;  // whole warps (T = 32) or nobody
@@ -216,15 +229,17 @@ __global__ void __launch_bounds__(kSplitThreads) encode_split_a_kernel(const flo
     }
     const int ex = split_exponent(top);
     const float sc = pow2f(ex);
-    __half *h = ahi + r * K2, *l = alo + r * K2;
+    const int64_t part = (int64_t)kEncodeChunk * K2;
+    __nv_bfloat16 *o = asplit + r * K2;
     auto put = [&](int64_t s, float2 v) {
-        __half rh, rl, ih, il;
-        f16_split(v.x * sc, rh, rl);
-        f16_split(v.y * sc, ih, il);
-        h[s] = rh;
-        l[s] = rl;
-        h[K + s] = ih;
-        l[K + s] = il;
+        __nv_bfloat16 re[kParts], im[kParts];
+        bf16_split(v.x * sc, re);
+        bf16_split(v.y * sc, im);
+#pragma unroll
+        for (int p = 0; p < kParts; ++p) {
+            o[p * part + s] = re[p];
+            o[p * part + K + s] = im[p];
+        }
     };
 #pragma unroll
     for (int i = 0; i < kSplitKeep; ++i) {
@@ -232,11 +247,13 @@ __global__ void __launch_bounds__(kSplitThreads) encode_split_a_kernel(const flo
         if (s < K) put(s, keep[i]);
     }
     for (int64_t s = rest; s < K; s += T) put(s, value(s));
-    for (int64_t c = 2 * K + tid; c < K2; c += T) h[c] = l[c] = __float2half_rn(0.f);
-    if (tid == 0) rowscale[r] = pow2f(-ex);
+    for (int64_t c = 2 * K + tid; c < K2; c += T)
+#pragma unroll
+        for (int p = 0; p < kParts; ++p) o[p * part + c] = __float2bfloat16_rn(0.f);
+    if (tid == 0) rowscale[r] = pow2f(tc::kSplitTarget - ex);
 }
 
-// FP16 matrix [rows][cols] (row stride ld elements, a multiple of 8), box
+// BF16 matrix [rows][cols] (row stride ld elements, a multiple of 8), box
 // 64 x box_rows, 128-byte swizzle: the operand layout of tc_gemm.cuh.
 static PFN_cuTensorMapEncodeTiled_v12000 encode_map_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -251,14 +268,14 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_map_fn() {
     });
     return fn;
 }
-static bool make_map_f16(CUtensorMap *map, const __half *ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+static bool make_map_bf16(CUtensorMap *map, const __nv_bfloat16 *ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
     auto fn = encode_map_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)(ld * 2)};
     cuuint32_t box[2] = {(cuuint32_t)tc::BK, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half *>(ptr), dims, strides, box, estr,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -277,10 +294,10 @@ static int64_t encode_k2(const slos_plan_s *p) {
 }
 
 // workspace: the transfer matrices of layers n and n-1, the split operands
-// B_hi, B_lo [2K][K2] and A_hi, A_lo [kEncodeChunk][K2], then the largest
+// B [kParts][2K][K2] and A [kParts][kEncodeChunk][K2], then the largest
 // magnitude and the scale of each output and the scale of each row of a chunk
 struct EncodeLayout {
-    size_t a, b, bhi, blo, ahi, alo, colmax, colscale, rowscale, total;
+    size_t a, b, bsplit, asplit, colmax, colscale, rowscale, total;
 };
 static EncodeLayout encode_layout(const slos_plan_s *p) {
     const int n = p->n;
@@ -294,10 +311,8 @@ static EncodeLayout encode_layout(const slos_plan_s *p) {
     };
     L.a = take((size_t)p->F[n] * p->F[n] * sizeof(float2));
     L.b = take(n >= 2 ? (size_t)p->F[n - 1] * p->F[n - 1] * sizeof(float2) : 0);
-    L.bhi = take(2 * K * K2 * sizeof(__half));
-    L.blo = take(2 * K * K2 * sizeof(__half));
-    L.ahi = take(kEncodeChunk * K2 * sizeof(__half));
-    L.alo = take(kEncodeChunk * K2 * sizeof(__half));
+    L.bsplit = take(kParts * 2 * K * K2 * sizeof(__nv_bfloat16));
+    L.asplit = take(kParts * kEncodeChunk * K2 * sizeof(__nv_bfloat16));
     L.colmax = take(K * sizeof(unsigned int));
     L.colscale = take(K * sizeof(float));
     L.rowscale = take(kEncodeChunk * sizeof(float));
@@ -363,13 +378,13 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
     }
     if (batch == 0) return SLOS_OK;
     const int64_t K = p->K, K2 = encode_k2(p);
-    __half *bhi = reinterpret_cast<__half *>(ws + L.bhi), *blo = reinterpret_cast<__half *>(ws + L.blo);
-    __half *ahi = reinterpret_cast<__half *>(ws + L.ahi), *alo = reinterpret_cast<__half *>(ws + L.alo);
+    __nv_bfloat16 *bsplit = reinterpret_cast<__nv_bfloat16 *>(ws + L.bsplit);
+    __nv_bfloat16 *asplit = reinterpret_cast<__nv_bfloat16 *>(ws + L.asplit);
     float *colscale = reinterpret_cast<float *>(ws + L.colscale), *rowscale = reinterpret_cast<float *>(ws + L.rowscale);
     {
         ProfScope ps("slos_encode_split", 0.0, s);
         dim3 grid((unsigned)((K + 31) / 32), (unsigned)((K + 31) / 32));
-        encode_split_b_kernel<<<grid, dim3(32, 8), 0, s>>>(buf[0], K, K2, colmax, p->tab.gfact, bhi, blo, colscale);
+        encode_split_b_kernel<<<grid, dim3(32, 8), 0, s>>>(buf[0], K, K2, colmax, p->tab.gfact, bsplit, colscale);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
     }
@@ -382,8 +397,8 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
             return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
         attr_done[dev] = true;
     }
-    CUtensorMap mah, mal;
-    if (!make_map_f16(&mah, ahi, kEncodeChunk, K2, K2, tc::BM) || !make_map_f16(&mal, alo, kEncodeChunk, K2, K2, tc::BM))
+    CUtensorMap ma;
+    if (!make_map_bf16(&ma, asplit, (int64_t)kParts * kEncodeChunk, K2, K2, tc::BM))
         return fail(SLOS_ERR_CUDA, "slos_encoded_forward: cuTensorMapEncodeTiled failed");
     const float2 *Xd = reinterpret_cast<const float2 *>(X);
     for (int b0 = 0; b0 < batch; b0 += kEncodeChunk) {
@@ -392,10 +407,10 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
             ProfScope ps("slos_encode_split", 0.0, s);
             if (K <= kSplitWarpRow)
                 encode_split_a_kernel<32><<<(unsigned)((rows + 7) / 8), kSplitThreads, 0, s>>>(
-                    Xd, p->tab.gfact, b0, rows, K, K2, ahi, alo, rowscale);
+                    Xd, p->tab.gfact, b0, rows, K, K2, asplit, rowscale);
             else
                 encode_split_a_kernel<kSplitThreads><<<(unsigned)rows, kSplitThreads, 0, s>>>(
-                    Xd, p->tab.gfact, b0, rows, K, K2, ahi, alo, rowscale);
+                    Xd, p->tab.gfact, b0, rows, K, K2, asplit, rowscale);
             if ((e = cudaGetLastError()) != cudaSuccess)
                 return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
         }
@@ -412,13 +427,15 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
         g.rowscale = rowscale;
         g.amps = output == SLOS_OUT_AMPS ? 1 : 0;
         g.err = p->d_status + 2;
-        CUtensorMap mbh, mbl;
-        if (!make_map_f16(&mbh, bhi, 2 * K, K2, K2, g.bn / 2) || !make_map_f16(&mbl, blo, 2 * K, K2, K2, g.bn / 2))
+        g.part_rows_a = kEncodeChunk;
+        g.part_rows_b = (int)(2 * K);
+        CUtensorMap mb;
+        if (!make_map_bf16(&mb, bsplit, kParts * 2 * K, K2, K2, g.bn / 2))
             return fail(SLOS_ERR_CUDA, "slos_encoded_forward: cuTensorMapEncodeTiled failed");
         const int64_t tiles = (int64_t)((g.N + g.bn - 1) / g.bn) * ((rows + 2 * tc::BM - 1) / (2 * tc::BM));
         const unsigned grid = 2 * (unsigned)std::min<int64_t>(tiles, pairs);
-        ProfScope ps("slos_encode_gemm", 3.0 * 2.0 * rows * (double)g.N * (double)K2, s);  // flops
-        tc::tc_gemm_split_kernel<<<grid, tc::kSpThreads, tc::kSpSmem, s>>>(mah, mbh, mal, mbl, g);
+        ProfScope ps("slos_encode_gemm", 6.0 * 2.0 * rows * (double)g.N * (double)K2, s);  // flops
+        tc::tc_gemm_split_kernel<<<grid, tc::kSpThreads, tc::kSpSmem, s>>>(ma, mb, g);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
     }

@@ -1,7 +1,7 @@
 // Tensor-core GEMM for sm_103a: C[M][N] = A[M][K] . B[N][K]^T, BF16 inputs
 // (both K-major), FP32 accumulation in tensor memory (TMEM), fused epilogues.
 // tc_gemm_split_kernel (end of the file) multiplies FP32-accurate operands
-// given as pairs of FP16 copies, with the same stage rows of 128 bytes (64
+// given as three BF16 copies, with the same stage rows of 128 bytes (64
 // 16-bit elements), swizzle and descriptors.
 // Two kernels share the pipeline below, both persistent over many tiles:
 // tc_gemm_pair_kernel (256 x 256 tiles on CTA pairs) and tc_gemm_persist_kernel
@@ -732,22 +732,21 @@ namespace slos {
 namespace tc {
 
 // ---------------------------------------------------------------- split operands
-// tc_gemm_split_kernel: FP32-accurate products on the FP16 tensor path.  Each
-// operand value is scaled by a power of two of its row and split into two FP16
-// numbers, v = hi + lo (22 significant bits), and the product is
-// A_hi B_hi + A_hi B_lo + A_lo B_hi (the dropped lo lo term is ~2^-22 of it).
-// Columns 2t and 2t + 1 are re and im of output t: psi(row, t) = rowscale[row]
-// colscale[t] (re + i im); stored as |psi|^2, or as psi (complex64).
+// tc_gemm_split_kernel: FP32-accurate products on the 16-bit tensor path.  Each
+// operand value is scaled by a power of two of its row and split into three
+// BF16 numbers, v = p0 + p1 + p2 (24 significant bits at any size), and the
+// product is p0 q0 + p0 q1 + p1 q0 + p1 q1 + p0 q2 + p2 q0, taken smallest
+// first (the dropped terms are ~2^-24 of it).  Columns 2t and 2t + 1 are re and
+// im of output t: psi(row, t) = rowscale[row] colscale[t] (re + i im) 2^(-2
+// kSplitTarget); stored as |psi|^2, or as psi (complex64).
 //
-// CTA pairs as in tc_gemm_pair_kernel, tiles of 256 x bn; a stage holds the hi
-// and the lo tile of both operands for 64 values of K and feeds all three
-// products from them (12 MMAs).  Bound by the MMAs, so what is left to choose
-// is how evenly the tiles fill the pairs: bn (split_columns) is the multiple of
-// 32 up to 256 with the least waves x columns.  One call of encoded_forward, us,
-// with 128 x 256 tiles of single CTAs (two stages, outputs written a row a
-// thread) / now: 4096 states of 2002 amplitudes 441 / 371 (2 x 2002 columns in
-// tiles of 224 fill 3.8 of 4 waves, of 256 3.4), 120 of 120 33 / 26, 16 of 56
-// 25 / 23.
+// CTA pairs as in tc_gemm_pair_kernel, tiles of 256 x bn; a stage holds the
+// three parts of both operands for 64 values of K and feeds all six products
+// from them (24 MMAs), so two stages of 96 KB a CTA keep the loads a stage
+// ahead.  Bound by the MMAs, so what is left to choose is how evenly the tiles
+// fill the pairs: bn (split_columns) is the multiple of 32 up to 256 with the
+// least waves x columns (2 x 2002 columns in tiles of 224 fill 3.8 of 4 waves,
+// of 256 3.4).
 //
 // The tensor core's FP32 accumulation does not round to nearest: over the
 // ~1500 MMAs of a long K its errors pile up in one direction (measured:
@@ -759,12 +758,14 @@ namespace tc {
 // Roles: warp 0 TMA producer, warp 1 MMA issuer (of the even CTA), warps 2-9
 // epilogue (TMEM lane quarter = warp % 4, the first half of the columns for
 // warps 2-5 and the second for warps 6-9).  Waits are bounded as above.
-constexpr int kSpStages = 3;
-constexpr int kSpChunkStages = 2;  // 24 MMAs per chunk
+constexpr int kSplitTarget = 50;   // exponent of a scaled row's largest magnitude
+constexpr int kSpParts = 3;        // BF16 numbers per value
+constexpr int kSpStages = 2;
+constexpr int kSpChunkStages = 1;  // 24 MMAs per chunk
 constexpr int kSpThreads = 320;
 constexpr int kSpEpiWarps = 8;
 constexpr int kSpTile = BM * 128;             // bytes of 128 rows of an operand
-constexpr int kSpStageBytes = 4 * kSpTile;    // A hi, A lo, B hi, B lo
+constexpr int kSpStageBytes = 2 * kSpParts * kSpTile;  // the parts of A, then those of B
 constexpr int kSpBox = 32 * 9 * 8;            // an epilogue warp's block of 32 rows x 8 outputs, padded
 constexpr int kSpSmem = kSpStages * kSpStageBytes + kSpEpiWarps * kSpBox + 1024 + 256;
 constexpr uint32_t kSpTmemCols = 2 * BN;
@@ -775,6 +776,7 @@ struct SplitArgs {
     void *C;      // [M][N / 2] float or complex64
     int amps;
     const float *colscale, *rowscale;
+    int part_rows_a, part_rows_b;  // rows from one part of an operand to the next
     int *err;
 };
 
@@ -794,7 +796,7 @@ inline int split_columns(int M, int N, int pairs) {
     return best;
 }
 
-__device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+__device__ __forceinline__ void mma_split_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                              uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -810,11 +812,13 @@ __device__ __forceinline__ void split_store(const SplitArgs &g, int row0, int co
                                             float2 *box) {
     const int t0 = col0 / 2, outs = g.N / 2;
     const float rs = row0 + lane < g.M ? __ldg(g.rowscale + row0 + lane) : 0.f;
+    constexpr float unscale = 1.f / ((float)(1ull << kSplitTarget) * (float)(1ull << kSplitTarget));
     float *boxf = reinterpret_cast<float *>(box);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const float c = t0 + i < outs ? __ldg(g.colscale + t0 + i) : 0.f;
-        const float re = v[2 * i] * rs * c, im = v[2 * i + 1] * rs * c;  // rs a power of two
+        // rs and unscale are powers of two; the sums reach 2^118, so unscale comes first
+        const float re = v[2 * i] * unscale * rs * c, im = v[2 * i + 1] * unscale * rs * c;
         if (g.amps) box[lane * 9 + i] = make_float2(re, im);
         else boxf[lane * 9 + i] = re * re + im * im;
     }
@@ -833,9 +837,7 @@ __device__ __forceinline__ void split_store(const SplitArgs &g, int row0, int co
 }
 
 static __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1)
-    tc_gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-                         const __grid_constant__ CUtensorMap ta_lo, const __grid_constant__ CUtensorMap tb_lo,
-                         SplitArgs g) {
+    tc_gemm_split_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, SplitArgs g) {
     extern __shared__ uint8_t smem_tc[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_tc) + 1023) & ~uintptr_t(1023));
     uint8_t *boxes = base + kSpStages * kSpStageBytes;
@@ -880,7 +882,7 @@ static __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1
     if (warp == 0) {
         if (lane == 0) {
             // producer: every stage of every tile, in order
-            const uint32_t bytes = 2u * 2u * (uint32_t)(kSpTile + bn / 2 * 128);  // of both CTAs
+            const uint32_t bytes = 2u * kSpParts * (uint32_t)(kSpTile + bn / 2 * 128);  // of both CTAs
             uint32_t it = 0;
             for (int t = pair; t < ntiles && !*abort_flag; t += npairs) {
                 const int m0 = (t / ntn) * 2 * BM + rank * BM, n0 = (t % ntn) * bn + rank * (bn / 2);
@@ -896,10 +898,12 @@ static __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1
                     if (rank == 0) mbar_expect_tx(full + s, bytes);
                     const uint32_t bar = cluster_addr(full + s, 0);
                     uint8_t *st = base + s * kSpStageBytes;
-                    tma_load_pair(st, &ta, kt * BK, m0, bar);
-                    tma_load_pair(st + 2 * kSpTile, &tb, kt * BK, n0, bar);
-                    tma_load_pair(st + 3 * kSpTile, &tb_lo, kt * BK, n0, bar);
-                    tma_load_pair(st + kSpTile, &ta_lo, kt * BK, m0, bar);
+                    // rows past a part's last are another part's: they meet outputs that are not stored
+#pragma unroll
+                    for (int p = 0; p < kSpParts; ++p) {
+                        tma_load_pair(st + p * kSpTile, &ta, kt * BK, m0 + p * g.part_rows_a, bar);
+                        tma_load_pair(st + (kSpParts + p) * kSpTile, &tb, kt * BK, n0 + p * g.part_rows_b, bar);
+                    }
                 }
             }
             // never leave with copies in flight: wait (bounded) until the last stages have been consumed
@@ -908,8 +912,9 @@ static __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
-            // FP32 accumulator (bits 4-5 = 1), A and B FP16 (0), N >> 3 (bits 17-22), M >> 4 (bits 24-28)
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
+            // as kIdescPair, with the tile's own width
+            const uint32_t idesc =
+                (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
             uint32_t it = 0, c = 0;  // stages and chunks over all tiles
             for (int t = pair; t < ntiles && !*abort_flag; t += npairs) {
                 for (int ch = 0; ch < nchunks; ++ch, ++c) {
@@ -932,15 +937,21 @@ static __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSpThreads, 1
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t ah = smem_u32(base + s * kSpStageBytes), al = ah + kSpTile;
-                        const uint32_t bh = ah + 2 * kSpTile, bl = ah + 3 * kSpTile;
+                        const uint32_t a0 = smem_u32(base + s * kSpStageBytes), b0 = a0 + kSpParts * kSpTile;
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
-                            const uint64_t dah = sw128_desc(ah + kk * 32), dal = sw128_desc(al + kk * 32);
-                            const uint64_t dbh = sw128_desc(bh + kk * 32), dbl = sw128_desc(bl + kk * 32);
-                            mma_f16_pair(d, dal, dbh, idesc, (kt > ch * kSpChunkStages || kk > 0) ? 1u : 0u);
-                            mma_f16_pair(d, dah, dbl, idesc, 1u);
-                            mma_f16_pair(d, dah, dbh, idesc, 1u);
+                            uint64_t p[kSpParts], q[kSpParts];
+#pragma unroll
+                            for (int i = 0; i < kSpParts; ++i) {
+                                p[i] = sw128_desc(a0 + i * kSpTile + kk * 32);
+                                q[i] = sw128_desc(b0 + i * kSpTile + kk * 32);
+                            }
+                            mma_split_pair(d, p[2], q[0], idesc, (kt > ch * kSpChunkStages || kk > 0) ? 1u : 0u);
+                            mma_split_pair(d, p[0], q[2], idesc, 1u);
+                            mma_split_pair(d, p[1], q[1], idesc, 1u);
+                            mma_split_pair(d, p[1], q[0], idesc, 1u);
+                            mma_split_pair(d, p[0], q[1], idesc, 1u);
+                            mma_split_pair(d, p[0], q[0], idesc, 1u);
                         }
                         mma_commit_pair(empty + s);
                     }

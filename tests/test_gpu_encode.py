@@ -1,5 +1,7 @@
 """Amplitude-encoded input (slos_encoded_forward): psi(t) = sum_s <t|U|s> x_s
 against the oracle's transfer matrix (Ryser permanents)."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -140,3 +142,56 @@ def test_encoded_tile_widths(slos, m, n, B, kind):
         assert np.abs(got - ref).max() <= 4e-6
     else:
         assert np.abs(got - np.abs(ref) ** 2).max() <= 8e-6
+
+
+def transfer_by_recursion(U, m, n):
+    """Phi in FP64 by the photon-by-photon recursion: products and sums of
+    entries of U only, so zeros and small entries are exact to their own size
+    (a permanent by inclusion and exclusion leaves 1e-17 in their place)."""
+    layers = [oracle.enumerate_fock(m, k) for k in range(n + 1)]
+    rank = [{tuple(int(x) for x in t): i for i, t in enumerate(b)} for b in layers]
+    A = {(0,) * m: np.ones(1, dtype=np.complex128)}
+    for k in range(1, n + 1):
+        child = np.array([[rank[k][tuple(int(x) + (q == j) for q, x in enumerate(t))] for j in range(m)]
+                          for t in layers[k - 1]])
+        cur = {}
+        for s in rank[k]:
+            c = max(q for q in range(m) if s[q])
+            prev = A[tuple(x - (q == c) for q, x in enumerate(s))]
+            v = np.zeros(len(layers[k]), dtype=np.complex128)
+            for j in range(m):
+                v[child[:, j]] += U[j, c] * prev
+            cur[s] = v
+        A = cur
+    g = np.sqrt([np.prod([math.factorial(int(x)) for x in t]) for t in layers[n]])
+    return np.stack([A[s] for s in rank[n]], axis=1) * g[:, None] / g[None, :]
+
+
+@pytest.mark.parametrize("m,n,B", [(6, 3, 131), (9, 4, 40), (10, 4, 300)])
+@pytest.mark.parametrize("u", ["phases", "permutation", "positive"])
+def test_encoded_components_of_very_different_size(slos, u, m, n, B):
+    """State vectors whose components span 25 orders of magnitude through maps
+    that do not mix (phases, a permutation): every output has one term and
+    keeps that component's relative accuracy, however small it is beside the
+    rest of its vector.  `positive`: a map with entries from 1e-8 to 1, all
+    sums of positive terms, so every output is as accurate as its terms.
+    Per term: the operands' 24 bits, about 2 n + 4 FP32 roundings of the
+    recursion and the factorials, the sums' truncation over 24 MMAs (below
+    2^-20): 4e-6 of the output's own size."""
+    rng = np.random.default_rng(10 * m + n)
+    plan = slos.Plan(m, [n] + [0] * (m - 1))
+    K = plan.n_outputs
+    span = 10.0 ** rng.uniform(-25, 0, (B, K))
+    if u == "positive":
+        U = (10.0 ** rng.uniform(-8, 0, (m, m))).astype(np.complex64)
+        X = span.astype(np.complex64)
+        X[: B // 2] *= np.arange(K)[None, :] == rng.integers(0, K, B // 2)[:, None]  # basis states: entries of Phi
+    else:
+        U = np.diag(np.exp(2j * np.pi * rng.random(m)))
+        if u == "permutation":
+            U = U[rng.permutation(m)]
+        U = U.astype(np.complex64)
+        X = (span * np.exp(2j * np.pi * rng.random((B, K)))).astype(np.complex64)
+    got = plan.encoded_forward(torch.tensor(U, device="cuda"), torch.tensor(X, device="cuda"), slos.AMPS).cpu().numpy()
+    ref = X.astype(np.complex128) @ transfer_by_recursion(U.astype(np.complex128), m, n).T
+    assert np.all(np.abs(got - ref) <= 4e-6 * np.abs(ref) + 1e-37)
