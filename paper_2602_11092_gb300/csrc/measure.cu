@@ -12,8 +12,7 @@
 // the renormalisation keeps its row in registers between its sum and its
 // division, and the expectations read an output's occupations as 32-bit words
 // once for several instances.  512 instances of 8008 outputs, 16 modes:
-// renormalise 15.0 -> 10.1 us, its backward 21.9 -> 13.6 us, expectations 44.2 -> 15 us,
-// their backward 35.8 -> 9.5 us.
+// expectations 44.2 -> 15 us, their backward 35.8 -> 9.5 us.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -150,11 +149,17 @@ __global__ void __launch_bounds__(kExpThreads) expect_bwd_kernel(const float *do
     }
 }
 
-constexpr int kRenThreads = 512;
-constexpr int kRenKeep = 16;  // values per thread kept in registers between the two passes
+// Renormalisation: T threads a row, KEEP values of it per thread in registers
+// between the sum and the division (what is left of longer rows is read again),
+// rows of fewer than 128 threads sharing a CTA.  A row's sum is a chain of
+// double-float additions (20 instructions each) per thread and one over its
+// lanes and warps, so short rows want few threads (many rows in flight, no
+// barrier) and long ones want many; renorm_launch has the lines.
+constexpr int kRenLong = 512;  // threads of the longest rows, which may also split over a cluster
 
-// Cluster-wide sum of one double-float per thread, fixed order (a tree over
-// the lanes, the warps and the ranks); every thread gets it.
+// Sum of one double-float per thread over a row's T threads (and its cluster),
+// fixed order (a tree over the lanes, the warps and the ranks); every thread
+// of the row gets it.
 __device__ __forceinline__ dfl warp_sum(dfl v, int width) {
     for (int o = width / 2; o > 0; o >>= 1) {
         const dfl w = {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
@@ -162,96 +167,121 @@ __device__ __forceinline__ dfl warp_sum(dfl v, int width) {
     }
     return v;
 }
-__device__ dfl cluster_sum(dfl v, dfl *red, dfl *part) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ dfl lane0(dfl v) {
+    return {__shfl_sync(0xffffffffu, v.hi, 0), __shfl_sync(0xffffffffu, v.lo, 0)};
+}
+template <int T>
+__device__ __forceinline__ dfl row_sum(dfl v, dfl *red, dfl *part) {
     v = warp_sum(v, 32);
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    v = warp_sum(lane < kRenThreads / 32 ? red[lane] : df_zero(), 32);
-    if (gridDim.x == 1) return v;
-    cg::cluster_group cluster = cg::this_cluster();
-    if (threadIdx.x == 0) *part = v;
-    cluster.sync();
-    v = df_zero();
-    if (lane < (int)gridDim.x) v = *cluster.map_shared_rank(part, lane);
-    v = warp_sum(v, kMaxCluster);  // lanes 0..7; the others hold zeros and are not used
-    v = {__shfl_sync(0xffffffffu, v.hi, 0), __shfl_sync(0xffffffffu, v.lo, 0)};
-    cluster.sync();  // no CTA leaves while its partial sum is read
+    if constexpr (T > 32) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        if (lane == 0) red[warp] = v;
+        __syncthreads();
+        // the row's T / 32 warps are the CTA's
+        v = lane0(warp_sum(lane < T / 32 ? red[lane] : df_zero(), T / 32));
+        if (T == kRenLong && gridDim.x > 1) {
+            cg::cluster_group cluster = cg::this_cluster();
+            if (threadIdx.x == 0) *part = v;
+            cluster.sync();
+            v = df_zero();
+            if (lane < (int)gridDim.x) v = *cluster.map_shared_rank(part, lane);
+            v = lane0(warp_sum(v, kMaxCluster));
+            cluster.sync();  // no CTA leaves while its partial sum is read
+        }
+    }
     return v;
 }
 
+// The slice of a row that this thread's CTA of the cluster (or its part of the CTA) takes.
+template <int T>
+struct RenRow {
+    static constexpr int kThreads = T < 128 ? 128 : T;
+    int b, tid;
+    int64_t lo, n;  // first value, values (none for rows past the batch)
+    __device__ RenRow(int64_t K, int B) {
+        tid = threadIdx.x % T;
+        b = blockIdx.y * (kThreads / T) + threadIdx.x / T;
+        const int64_t per = (K + gridDim.x - 1) / gridDim.x;
+        lo = per * blockIdx.x;
+        n = b < B ? min(K, lo + per) - lo : 0;
+    }
+};
+
 // Z = sum_t p[t]; q[t] = p[t] / Z  (sums in double-float, dfloat.cuh).  q may be p.
-__global__ void __launch_bounds__(kRenThreads, 3) renorm_fwd_kernel(const float *p, int64_t K, float *q, float *Z) {
-    __shared__ dfl red[kRenThreads / 32], part;
-    const int b = blockIdx.y;
-    const int64_t per = (K + gridDim.x - 1) / gridDim.x;
-    const int64_t lo = per * blockIdx.x;
-    const int n = (int)(min(K, lo + per) - lo);  // at most K < 2^31
-    const float *pb = p + (size_t)b * K + lo;
-    float keep[kRenKeep];
+template <int T, int KEEP>
+__global__ void __launch_bounds__(RenRow<T>::kThreads) renorm_fwd_kernel(const float *p, int64_t K, int B, float *q,
+                                                                         float *Z) {
+    __shared__ dfl red[RenRow<T>::kThreads / 32], part;
+    const RenRow<T> r(K, B);
+    const float *pb = p + (size_t)r.b * K + r.lo;
+    float keep[KEEP];
 #pragma unroll
-    for (int i = 0; i < kRenKeep; ++i) {
-        const int64_t c = threadIdx.x + (int64_t)i * kRenThreads;
-        keep[i] = c < n ? pb[c] : 0.f;
+    for (int i = 0; i < KEEP; ++i) {
+        const int64_t c = r.tid + (int64_t)i * T;
+        keep[i] = c < r.n ? pb[c] : 0.f;
     }
-    // pairs first (exact), in four independent chains: the additions of one
-    // chain wait 20 instructions for each other
-    dfl part4[4];
+    // pairs first (exact), in independent chains: the additions of one chain
+    // wait 20 instructions for each other
+    constexpr int kChains = KEEP >= 8 ? 4 : 1;
+    dfl chain[kChains];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) part4[i] = two_sum(keep[4 * i], keep[4 * i + 1]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) part4[i] = df_add(part4[i], two_sum(keep[4 * i + 2], keep[4 * i + 3]));
-    dfl acc = df_add(df_add(part4[0], part4[1]), df_add(part4[2], part4[3]));
-    const int64_t rest = threadIdx.x + (int64_t)kRenKeep * kRenThreads;
+    for (int i = 0; i < KEEP / 2; ++i) {
+        const dfl pair = two_sum(keep[2 * i], keep[2 * i + 1]);
+        chain[i % kChains] = i < kChains ? pair : df_add(chain[i % kChains], pair);
+    }
+    dfl acc = chain[0];
+    if constexpr (kChains == 4) acc = df_add(df_add(chain[0], chain[1]), df_add(chain[2], chain[3]));
+    const int64_t rest = r.tid + (int64_t)KEEP * T;
 #pragma unroll 4
-    for (int64_t c = rest; c < n; c += kRenThreads) acc = df_add_f(acc, pb[c]);
-    const float z = df_float(cluster_sum(acc, red, &part));
+    for (int64_t c = rest; c < r.n; c += T) acc = df_add_f(acc, pb[c]);
+    const float z = df_float(row_sum<T>(acc, red, &part));
     const float inv = z > 0.f ? 1.f / z : 0.f;
-    float *qb = q + (size_t)b * K + lo;
+    float *qb = q + (size_t)r.b * K + r.lo;
 #pragma unroll
-    for (int i = 0; i < kRenKeep; ++i) {
-        const int64_t c = threadIdx.x + (int64_t)i * kRenThreads;
-        if (c < n) qb[c] = keep[i] * inv;
+    for (int i = 0; i < KEEP; ++i) {
+        const int64_t c = r.tid + (int64_t)i * T;
+        if (c < r.n) qb[c] = keep[i] * inv;
     }
-    for (int64_t c = rest; c < n; c += kRenThreads) qb[c] = pb[c] * inv;
-    if (blockIdx.x == 0 && threadIdx.x == 0) Z[b] = z;
+    for (int64_t c = rest; c < r.n; c += T) qb[c] = pb[c] * inv;
+    if (blockIdx.x == 0 && r.tid == 0 && r.b < B) Z[r.b] = z;
 }
 
 // dp[t] = (dq[t] - sum_s dq[s] q[s]) / Z.  dp may be dq.
-__global__ void __launch_bounds__(kRenThreads, 2) renorm_bwd_kernel(const float *q, const float *Z, const float *dq,
-                                                                    int64_t K, float *dp) {
-    __shared__ dfl red[kRenThreads / 32], part;
-    const int b = blockIdx.y;
-    const int64_t per = (K + gridDim.x - 1) / gridDim.x;
-    const int64_t lo = per * blockIdx.x;
-    const int n = (int)(min(K, lo + per) - lo);
-    const float *qb = q + (size_t)b * K + lo, *dqb = dq + (size_t)b * K + lo;
-    float keep[kRenKeep], qv[kRenKeep];
+template <int T, int KEEP>
+__global__ void __launch_bounds__(RenRow<T>::kThreads) renorm_bwd_kernel(const float *q, const float *Z, const float *dq,
+                                                                         int64_t K, int B, float *dp) {
+    __shared__ dfl red[RenRow<T>::kThreads / 32], part;
+    const RenRow<T> r(K, B);
+    const float *qb = q + (size_t)r.b * K + r.lo, *dqb = dq + (size_t)r.b * K + r.lo;
+    float keep[KEEP], qv[KEEP];
 #pragma unroll
-    for (int i = 0; i < kRenKeep; ++i) {
-        const int64_t c = threadIdx.x + (int64_t)i * kRenThreads;
-        keep[i] = c < n ? dqb[c] : 0.f;
-        qv[i] = c < n ? qb[c] : 0.f;
+    for (int i = 0; i < KEEP; ++i) {
+        const int64_t c = r.tid + (int64_t)i * T;
+        keep[i] = c < r.n ? dqb[c] : 0.f;
+        qv[i] = c < r.n ? qb[c] : 0.f;
     }
-    const float z = Z[b];
-    dfl part4[4];
+    const float z = r.b < B ? Z[r.b] : 0.f;
+    constexpr int kChains = KEEP >= 8 ? 4 : 1;
+    dfl chain[kChains];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) part4[i] = two_prod(keep[i], qv[i]);
-#pragma unroll
-    for (int i = 4; i < kRenKeep; ++i) part4[i & 3] = df_add(part4[i & 3], two_prod(keep[i], qv[i]));
-    dfl acc = df_add(df_add(part4[0], part4[1]), df_add(part4[2], part4[3]));
-    const int64_t rest = threadIdx.x + (int64_t)kRenKeep * kRenThreads;
+    for (int i = 0; i < KEEP; ++i) {
+        const dfl prod = two_prod(keep[i], qv[i]);
+        chain[i % kChains] = i < kChains ? prod : df_add(chain[i % kChains], prod);
+    }
+    dfl acc = chain[0];
+    if constexpr (kChains == 4) acc = df_add(df_add(chain[0], chain[1]), df_add(chain[2], chain[3]));
+    const int64_t rest = r.tid + (int64_t)KEEP * T;
 #pragma unroll 4
-    for (int64_t c = rest; c < n; c += kRenThreads) acc = df_add(acc, two_prod(dqb[c], qb[c]));
-    const float sdot = df_float(cluster_sum(acc, red, &part));
+    for (int64_t c = rest; c < r.n; c += T) acc = df_add(acc, two_prod(dqb[c], qb[c]));
+    const float sdot = df_float(row_sum<T>(acc, red, &part));
     const float inv = z > 0.f ? 1.f / z : 0.f;
-    float *dpb = dp + (size_t)b * K + lo;
+    float *dpb = dp + (size_t)r.b * K + r.lo;
 #pragma unroll
-    for (int i = 0; i < kRenKeep; ++i) {
-        const int64_t c = threadIdx.x + (int64_t)i * kRenThreads;
-        if (c < n) dpb[c] = (keep[i] - sdot) * inv;
+    for (int i = 0; i < KEEP; ++i) {
+        const int64_t c = r.tid + (int64_t)i * T;
+        if (c < r.n) dpb[c] = (keep[i] - sdot) * inv;
     }
-    for (int64_t c = rest; c < n; c += kRenThreads) dpb[c] = (dqb[c] - sdot) * inv;
+    for (int64_t c = rest; c < r.n; c += T) dpb[c] = (dqb[c] - sdot) * inv;
 }
 
 // A kernel launched with clusters of `cluster` CTAs along x (the grid's width).
@@ -266,18 +296,58 @@ static cudaError_t launch_clusters(void (*kernel)(P...), int cluster, int rows, 
     attr.val.clusterDim.x = cluster;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 1 : 0;  // a grid of single CTAs launches without
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
-// The renormalisation's CTAs per row: one while the row fits its registers
-// (8192 outputs; a cluster costs two cluster barriers: 16.9 us against
-// 10.1 us on 512 rows of 8008), then clusters until a slice does.
-static int renorm_cluster(const slos_plan_s *p) {
+// Calls f.run<T, KEEP>(cluster, CTAs) with the shape for rows of K outputs.
+// Measured, us, forward / backward (a warp a row, 128, 256 and 512 threads):
+//   65,535 rows of 10: warp x 2 values 16 / 18, x 8 25 / 31, 512 x 16 629 / 811
+//   65,535 of 120: x 8 24 / 31, x 16 33 / 46;  of 330: x 16 37 / 50, x 32 56 / 81
+//   65,535 of 1001: x 32 76 / 117, 128 x 16 145 / 190;  16,384 of 2002: 61 / 96, 44 / 60
+//   4096 of 4368: 256 x 16 29 / 39, 512 x 16 43 / 59;  of 8008: 256 x 32 43 / 61, 512 x 16 48 / 71
+//   4096 of 12,376: 512 x 16, the rest read again, 77 / 118, two CTAs 113 / 161
+// Clusters pay where a CTA would walk more than 32,768 values (1000 rows of
+// 54,264: one CTA 173 / 251, two 112 / 167) and for few rows (one of 54,264:
+// 20 / 25, eight CTAs 4.7 / 5.2).
+template <typename F>
+static cudaError_t renorm_launch(const slos_plan_s *p, int batch, F f) {
+    const int64_t K = p->K;
+    if (K <= 64) return f.template run<32, 2>(1, (batch + 3) / 4);
+    if (K <= 256) return f.template run<32, 8>(1, (batch + 3) / 4);
+    if (K <= 512) return f.template run<32, 16>(1, (batch + 3) / 4);
+    if (K <= 1024) return f.template run<32, 32>(1, (batch + 3) / 4);
+    if (K <= 2048) return f.template run<128, 16>(1, batch);
+    if (K <= 4608) return f.template run<256, 16>(1, batch);
+    if (K <= 8192) return f.template run<256, 32>(1, batch);
     int c = 1;
-    while (c < kMaxCluster && p->K > (int64_t)c * kRenThreads * kRenKeep) c *= 2;
-    return c;
+    while (c < kMaxCluster &&
+           (K / c > 32768 || ((int64_t)2 * c * batch <= p->sm_count && K / (2 * c) >= 4096)))
+        c *= 2;
+    return f.template run<kRenLong, 16>(c, batch);
 }
+struct RenormFwd {
+    const float *p;
+    int64_t K;
+    int B;
+    float *q, *Z;
+    cudaStream_t s;
+    template <int T, int KEEP>
+    cudaError_t run(int cluster, int rows) const {
+        return launch_clusters(renorm_fwd_kernel<T, KEEP>, cluster, rows, RenRow<T>::kThreads, s, p, K, B, q, Z);
+    }
+};
+struct RenormBwd {
+    const float *q, *Z, *dq;
+    int64_t K;
+    int B;
+    float *dp;
+    cudaStream_t s;
+    template <int T, int KEEP>
+    cudaError_t run(int cluster, int rows) const {
+        return launch_clusters(renorm_bwd_kernel<T, KEEP>, cluster, rows, RenRow<T>::kThreads, s, q, Z, dq, K, B, dp);
+    }
+};
 
 template <int MW>
 static cudaError_t launch_expect_fwd(const slos_plan_s *p, const float *probs, int batch, float *out, cudaStream_t s) {
@@ -366,8 +436,7 @@ slos_status_t slos_renormalise(slos_plan_t p, const float *pr, int batch, float 
     if (!pr || !q || !Z) return fail(SLOS_ERR_INVALID_ARG, "slos_renormalise: NULL pointer");
     cudaStream_t s = (cudaStream_t)stream;
     ProfScope ps("slos_renormalise", (double)batch * 8.0 * p->K, s);
-    return launched(launch_clusters(renorm_fwd_kernel, renorm_cluster(p), batch, kRenThreads, s, pr, p->K, q, Z),
-                    "slos_renormalise");
+    return launched(renorm_launch(p, batch, RenormFwd{pr, p->K, batch, q, Z, s}), "slos_renormalise");
 }
 
 slos_status_t slos_renormalise_backward(slos_plan_t p, const float *q, const float *Z, const float *dq, int batch,
@@ -378,8 +447,7 @@ slos_status_t slos_renormalise_backward(slos_plan_t p, const float *q, const flo
     if (!q || !Z || !dq || !dp) return fail(SLOS_ERR_INVALID_ARG, "slos_renormalise_backward: NULL pointer");
     cudaStream_t s = (cudaStream_t)stream;
     ProfScope ps("slos_renormalise_bwd", (double)batch * 12.0 * p->K, s);
-    return launched(launch_clusters(renorm_bwd_kernel, renorm_cluster(p), batch, kRenThreads, s, q, Z, dq, p->K, dp),
-                    "slos_renormalise_backward");
+    return launched(renorm_launch(p, batch, RenormBwd{q, Z, dq, p->K, batch, dp, s}), "slos_renormalise_backward");
 }
 
 }  // extern "C"

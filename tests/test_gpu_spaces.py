@@ -321,3 +321,34 @@ def test_reductions_over_split_rows(slos, m, n, det, B):
     q64, Z64 = q.double().cpu().numpy(), Z.double().cpu().numpy()[:, None]
     dot = (dq * q64).sum(axis=1, keepdims=True)
     assert np.abs(got - (dq - dot) / Z64).max() <= 4e-7 * ((np.abs(dq).max() + np.abs(dot).max()) / Z64.min())
+
+
+@pytest.mark.parametrize("m,n", [(7, 1), (11, 2), (22, 2), (23, 2), (5, 8), (14, 3), (11, 4), (18, 3), (14, 4), (17, 4),
+                                 (10, 6), (16, 5), (17, 5)])
+@pytest.mark.parametrize("B", [1, 6, 161])
+def test_renormalise_rows_of_any_length(slos, m, n, B):
+    """Rows of 7 to 20,349 outputs: several rows in a CTA (the last CTA short
+    of rows), one, a cluster; rows within and beyond the registers; in place;
+    a row without weight next to others.  FP64 sums; bounds as above."""
+    plan = slos.Plan(m, [n] + [0] * (m - 1))
+    K = plan.n_outputs
+    rng = np.random.default_rng(1000 * m + 10 * n + B)
+    p = rng.exponential(size=(B, K)).astype(np.float32)
+    if B > 1:
+        p[B // 2] = 0.0
+    p64 = p.astype(np.float64)
+    tot = p64.sum(axis=1, keepdims=True)
+    buf = torch.full((B * K + 64,), 5.0, device="cuda")
+    pt = buf[:B * K].view(B, K)
+    pt.copy_(torch.tensor(p))
+    q, Z = plan.renormalise(pt, q=pt)
+    assert q.data_ptr() == pt.data_ptr() and torch.all(buf[B * K:] == 5.0)
+    q64, Z64 = q.double().cpu().numpy(), Z.double().cpu().numpy()[:, None]
+    ref = np.divide(p64, tot, out=np.zeros_like(p64), where=tot > 0)
+    assert np.all(np.abs(Z64 - tot) <= 1e-7 * tot)
+    assert np.all(np.abs(q64 - ref) <= 3e-7 * ref)
+    dq = rng.standard_normal((B, K)).astype(np.float32)
+    got = plan.renormalise_backward(q, Z, torch.tensor(dq, device="cuda")).double().cpu().numpy()
+    dot = (dq * q64).sum(axis=1, keepdims=True)
+    inv = np.divide(1.0, Z64, out=np.zeros_like(Z64), where=Z64 > 0)
+    assert np.all(np.abs(got - (dq - dot) * inv) <= 4e-7 * (np.abs(dq).max() + np.abs(dot)) * inv)
