@@ -9,7 +9,8 @@
 // the first t with C(t) > target.  Three kernels: sums of runs of 32 weights,
 // an in-place inclusive scan of the run sums per instance, and eight lanes per
 // shot that search the run prefix nine ways at a time and then resolve the
-// run's 32 weights, four per lane.
+// run's 32 weights, four per lane.  Rows of few outcomes take one kernel
+// instead (sample_small_kernel).
 //
 // What bounds it: the shots' dependent reads.  One thread per shot that
 // bisected sums of 256 weights and then walked its run took 127 us for 256 x
@@ -20,6 +21,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 
 #include "../../include/slos.h"
@@ -37,9 +39,18 @@ constexpr int kSumWeights = 8;                              // consecutive weigh
 constexpr int kSumLanes = kSampleRun / kSumWeights;         // threads per run
 constexpr int kScanThreads = 1024;
 constexpr int kShotThreads = 256;
+constexpr int kSmallWeights = 4;                            // weights per thread of the one-kernel form
+constexpr int64_t kSmallOutcomes = kShotThreads * kSmallWeights;
 
 __device__ __forceinline__ uint64_t fixed32(float x) {
     return x > 0.f ? __float2ull_rz(x * 4294967296.0f) : 0ull;  // NaN and negatives weigh nothing
+}
+
+// floor(floor(x 2^32) T / 2^32)
+__device__ __forceinline__ uint64_t shot_target(float x, uint64_t T) {
+    const uint64_t U32 = x > 0.f ? (uint64_t)__float2uint_rz(x * 4294967296.0f) : 0ull;  // saturates at 2^32 - 1
+    const uint64_t lo64 = T * U32, hi64 = __umul64hi(T, U32);
+    return (hi64 << 32) | (lo64 >> 32);
 }
 
 // sums[b][r] = weights of run r; clears the counts of the same outcomes.
@@ -124,10 +135,7 @@ __global__ void __launch_bounds__(kShotThreads) sample_kernel(const float *p, in
         if (g == 0) samples[idx] = -1;  // no outcome carries any weight
         return;
     }
-    const float x = u[idx];
-    const uint64_t U32 = x > 0.f ? (uint64_t)__float2uint_rz(x * 4294967296.0f) : 0ull;  // saturates at 2^32 - 1
-    const uint64_t lo64 = T * U32, hi64 = __umul64hi(T, U32);
-    const uint64_t target = (hi64 << 32) | (lo64 >> 32);  // floor(U32 T / 2^32)
+    const uint64_t target = shot_target(u[idx], T);
     // first run whose inclusive prefix exceeds the target: [l, h] is cut into
     // nine parts, the lanes read the last entry of the first eight
     int64_t l = 0, h = nruns - 1;
@@ -177,6 +185,75 @@ __global__ void __launch_bounds__(kShotThreads) sample_kernel(const float *p, in
     }
 }
 
+// Rows of up to kSmallOutcomes outcomes: each CTA scans its row into shared
+// memory and takes `per` shots, a thread each, by bisection; the counts are
+// gathered in shared memory.  One launch instead of three, and no lanes wasted
+// on short searches: what bounds it is the shots' reads and writes.  Measured,
+// us a call, eight lanes a shot over the prefix in memory / this form: 16 x
+// 1,000,000 shots of 10 outcomes 1022 / 54, with counts 5467 / 58; 256 x 1000
+// of 330 35 / 4.8; 4096 x 100 of 330 80 / 10.
+__global__ void __launch_bounds__(kShotThreads) sample_small_kernel(const float *p, int K, const float *u, int shots,
+                                                                    int per, int32_t *samples, int32_t *counts) {
+    __shared__ uint64_t C[kSmallOutcomes];
+    __shared__ int hist[kSmallOutcomes];
+    __shared__ uint64_t tot[kShotThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = blockIdx.y;
+    const float *pb = p + (size_t)b * K;
+    uint64_t w[kSmallWeights], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kSmallWeights; ++i) {
+        const int t = threadIdx.x * kSmallWeights + i;
+        w[i] = t < K ? fixed32(pb[t]) : 0ull;
+        sum += w[i];
+    }
+    uint64_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) tot[warp] = incl;
+    __syncthreads();
+    uint64_t acc = incl - sum;
+    for (int q = 0; q < warp; ++q) acc += tot[q];
+#pragma unroll
+    for (int i = 0; i < kSmallWeights; ++i) {
+        const int t = threadIdx.x * kSmallWeights + i;
+        acc += w[i];
+        if (t < K) {
+            C[t] = acc;
+            hist[t] = 0;
+        }
+    }
+    __syncthreads();
+    const uint64_t T = C[K - 1];
+    const int64_t s0 = (int64_t)blockIdx.x * per, s1 = min(s0 + per, (int64_t)shots);
+    const size_t row = (size_t)b * shots;
+    for (int64_t s = s0 + threadIdx.x; s < s1; s += kShotThreads) {
+        if (T == 0) {
+            samples[row + s] = -1;  // no outcome carries any weight
+            continue;
+        }
+        const uint64_t target = shot_target(u[row + s], T);
+        int l = 0, h = K - 1;
+        while (l < h) {
+            const int mid = (l + h) >> 1;
+            if (C[mid] > target) h = mid;
+            else l = mid + 1;
+        }
+        samples[row + s] = l;
+        if (counts) atomicAdd(hist + l, 1);
+    }
+    if (!counts) return;
+    __syncthreads();
+    for (int t = threadIdx.x; t < K; t += kShotThreads) {
+        int32_t *c = counts + (size_t)b * K + t;
+        if (gridDim.x == 1) *c = hist[t];
+        else if (hist[t] > 0) atomicAdd(c, hist[t]);
+    }
+}
+
 static int64_t runs_of(const slos_plan_s *p) { return (p->K + kSampleRun - 1) / kSampleRun; }
 
 }  // namespace slos
@@ -207,6 +284,21 @@ slos_status_t slos_sample(slos_plan_t p, const float *probs, int batch, int shot
     uint64_t *pre = reinterpret_cast<uint64_t *>(workspace);
     ProfScope ps("slos_sample", (double)batch * (4.0 * p->K) + (double)batch * shots * 8.0, s);
     cudaError_t e;
+    if (p->K <= kSmallOutcomes) {
+        // as many CTAs a row as fill the GPU, each with a block of shots at least
+        const int blocks = (int)std::min<int64_t>(((int64_t)shots + kShotThreads - 1) / kShotThreads,
+                                                  (int64_t)p->sm_count * (2048 / kShotThreads) / batch);
+        const int g = std::max(1, blocks);
+        if (counts && g > 1 &&
+            (e = cudaMemsetAsync(counts, 0, (size_t)batch * p->K * sizeof(int32_t), s)) != cudaSuccess)
+            return fail(SLOS_ERR_CUDA, std::string("slos_sample: ") + cudaGetErrorString(e));
+        if (shots > 0 || counts)
+            sample_small_kernel<<<dim3((unsigned)g, batch), kShotThreads, 0, s>>>(
+                probs, (int)p->K, uniforms, shots, (int)(((int64_t)shots + g - 1) / g), samples, counts);
+        if ((e = cudaGetLastError()) != cudaSuccess)
+            return fail(SLOS_ERR_CUDA, std::string("slos_sample: ") + cudaGetErrorString(e));
+        return SLOS_OK;
+    }
     // 16-byte accesses where every row starts on a 16-byte boundary
     const bool vec = p->K % 4 == 0 && reinterpret_cast<uintptr_t>(probs) % 16 == 0 &&
                      reinterpret_cast<uintptr_t>(counts) % 16 == 0;

@@ -85,3 +85,28 @@ def test_samples_off_a_16_byte_boundary_and_ragged_shots(slos, m, s, offset, B, 
         ref = oracle.sample_outcomes(p[b], u[b])
         assert np.array_equal(samples[b].cpu().numpy(), ref)
         assert np.array_equal(counts[b].cpu().numpy(), np.bincount(ref, minlength=K))
+
+
+@pytest.mark.parametrize("m,n", [(2, 1), (3, 2), (8, 2), (10, 4), (11, 4), (22, 2), (5, 10), (12, 4)])
+@pytest.mark.parametrize("B,shots", [(1, 0), (1, 1), (2, 257), (1, 60_000), (1300, 300)])
+def test_shots_of_few_and_of_many_outcomes(slos, m, n, B, shots):
+    """Rows of 2 to 1365 outcomes on both sides of the one-kernel form's 1024:
+    no shot, one, one past a block, many CTAs a row, a row a CTA; rows without
+    weight, weights far above 1; the oracle's outcomes and counts exactly."""
+    plan = slos.Plan(m, [n] + [0] * (m - 1))
+    K = plan.n_outputs
+    p = workloads.random_distributions(B, K, seed=80 + m, zero_fraction=0.3 if K > 10 else 0.0)
+    p[B - 1] *= 1e6
+    if B > 1:
+        p[0] = 0.0
+    u = workloads.uniforms(B, shots, seed=81 + m)
+    pt, ut = torch.tensor(p, device="cuda"), torch.tensor(u, device="cuda")
+    samples, counts = plan.sample(pt, ut, counts=True)
+    assert torch.equal(samples, plan.sample(pt, ut))
+    for b in {0, B // 2, B - 1}:
+        if B > 1 and b == 0:
+            assert torch.all(samples[0] == -1) and torch.all(counts[0] == 0)
+            continue
+        ref = oracle.sample_outcomes(p[b], u[b])
+        assert np.array_equal(samples[b].cpu().numpy(), ref)
+        assert np.array_equal(counts[b].cpu().numpy(), np.bincount(ref, minlength=K))
