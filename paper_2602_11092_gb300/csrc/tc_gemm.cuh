@@ -481,6 +481,31 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t x) {
     return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x));
 }
 
+// What the epilogue of 32 rows x 32 columns reads: Z (four lanes a row) or C
+// before the sum (eight lanes a row).  Read a block ahead, the first before
+// the wait for the sums, so that its latency is nobody's (us, read where it is
+// used / now: accumulating 8192 x 8192 x 2048 330 / 211, 4096 x 12376 x 512 238 / 123;
+// GELU' 4096 x 12376 x 512 175 / 116, 4096 x 2048 x 2048 43 / 41; over many
+// tiles of a long K GELU' is bound by its arithmetic, 243 at 8192 x 8192 x 2048).
+template <int EPI>
+constexpr int kPairAhead = EPI == TC_F32_ACCUM ? 8 : (EPI == TC_GELU_BWD ? 4 : 0);
+template <int EPI>
+__device__ __forceinline__ void pair_load32(const TcArgs &g, int row0, int col0, int lane,
+                                            uint4 (&in)[kPairAhead<EPI> + 1]) {
+    constexpr int N = kPairAhead<EPI>;  // 16-byte pieces of a row's 32 values, and lanes a row
+    if constexpr (N > 0) {
+        const size_t bytes = EPI == TC_GELU_BWD ? 2 : 4;
+        const char *src = reinterpret_cast<const char *>(EPI == TC_GELU_BWD ? (const void *)g.aux : g.C);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const int r = 32 / N * i + lane / N;
+            if (row0 + r < g.M)
+                in[i] = *(reinterpret_cast<const uint4 *>(src + ((int64_t)(row0 + r) * g.ldc + col0) * bytes) +
+                          lane % N);
+        }
+    }
+}
+
 // Epilogue of 32 rows x 32 columns by a warp, columns col0 .. col0 + 31 all
 // inside the matrix, rows and bias 16-byte aligned: v holds row row0 + lane.
 // The block is turned in `box` (32 rows of eight 16-byte slots, slot q of row r
@@ -488,7 +513,8 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t x) {
 // write a row's 128 bytes (64 of C and 64 of Z for the bf16 outputs); a thread
 // writing its own row sends 16 bytes to each of 32 rows an instruction.
 template <int EPI>
-__device__ __forceinline__ void pair_store32(const TcArgs &g, int row0, int col0, int lane, float (&v)[32], uint4 *box) {
+__device__ __forceinline__ void pair_store32(const TcArgs &g, int row0, int col0, int lane, float (&v)[32],
+                                             const uint4 (&in)[kPairAhead<EPI> + 1], uint4 *box) {
     constexpr bool kBf16 = EPI == TC_GELU || EPI == TC_GELU_BWD;
     if (EPI == TC_F32_BIAS || EPI == TC_GELU) {
         const float4 *b = reinterpret_cast<const float4 *>(g.bias + col0);
@@ -508,9 +534,7 @@ __device__ __forceinline__ void pair_store32(const TcArgs &g, int row0, int col0
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int r = 8 * i + (lane >> 2), q = lane & 3;
-            if (row0 + r < g.M)
-                box[r * 8 + (q ^ (r & 7))] =
-                    *(reinterpret_cast<const uint4 *>(g.aux + (int64_t)(row0 + r) * g.ldc + col0) + q);
+            if (row0 + r < g.M) box[r * 8 + (q ^ (r & 7))] = in[i];
         }
         __syncwarp();
     }
@@ -554,11 +578,10 @@ __device__ __forceinline__ void pair_store32(const TcArgs &g, int row0, int col0
         if (!kBf16) {
             uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<float *>(g.C) + o) + q;
             if (EPI == TC_F32_ACCUM) {
-                const uint4 old = *dst;
-                x.x = __float_as_uint(__uint_as_float(x.x) + __uint_as_float(old.x));
-                x.y = __float_as_uint(__uint_as_float(x.y) + __uint_as_float(old.y));
-                x.z = __float_as_uint(__uint_as_float(x.z) + __uint_as_float(old.z));
-                x.w = __float_as_uint(__uint_as_float(x.w) + __uint_as_float(old.w));
+                x.x = __float_as_uint(__uint_as_float(x.x) + __uint_as_float(in[i].x));
+                x.y = __float_as_uint(__uint_as_float(x.y) + __uint_as_float(in[i].y));
+                x.z = __float_as_uint(__uint_as_float(x.z) + __uint_as_float(in[i].z));
+                x.w = __float_as_uint(__uint_as_float(x.w) + __uint_as_float(in[i].w));
             }
             *dst = x;
         } else if (q >= 4) {
@@ -682,6 +705,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         int j = 0;
         for (int t = pair; t < ntiles; t += npairs, ++j) {
             const int acc = j & 1;
+            const int row0 = (t / ntn) * 2 * BM + rank * BM + q * 32, n0 = (t % ntn) * BN;
+            uint4 ahead[kPairAhead<EPI> + 1];
+            if (vec && n0 + c0 + 32 <= g.N) pair_load32<EPI>(g, row0, n0 + c0, lane, ahead);
             const bool ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(tfull + acc, (j >> 1) & 1));
             if (!ok) {
                 if (lane == 0) {
@@ -691,15 +717,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 break;
             }
             tc_fence_after();
-            const int row0 = (t / ntn) * 2 * BM + rank * BM + q * 32, n0 = (t % ntn) * BN;
             const uint32_t src = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
             for (int c = c0; c < c0 + kCols; c += 32) {
                 if (row0 >= g.M || n0 + c >= g.N) break;
                 if (vec && n0 + c + 32 <= g.N) {
+                    uint4 in[kPairAhead<EPI> + 1];
+#pragma unroll
+                    for (int i = 0; i < kPairAhead<EPI>; ++i) in[i] = ahead[i];
+                    if (c + 32 < c0 + kCols && n0 + c + 64 <= g.N) pair_load32<EPI>(g, row0, n0 + c + 32, lane, ahead);
                     float v[32];
                     tmem_ld32(src + (uint32_t)c, v);
-                    pair_store32<EPI>(g, row0, n0 + c, lane, v, box);
+                    pair_store32<EPI>(g, row0, n0 + c, lane, v, in, box);
                 } else {
 #pragma unroll 1
                     for (int h = 0; h < 32; h += 16) {
