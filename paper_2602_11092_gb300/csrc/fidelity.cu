@@ -62,7 +62,13 @@ struct FidArgs {
     bool sym;        // Ub is Ua: tiles on and above the diagonal, written twice
 };
 
-__device__ __forceinline__ void fid_tile(int Nb, bool sym, int64_t b, int &ti, int &tj);
+__device__ __forceinline__ void fid_tile(int Nb, bool sym, uint32_t b, int &ti, int &tj);
+// blockIdx.x, read anew at each use (the compiler keeps nothing derived from it)
+__device__ __forceinline__ uint32_t fid_block() {
+    uint32_t b;
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(b));
+    return b;
+}
 
 template <int N>
 __global__ void __launch_bounds__(kFidTile *kFidTile) fidelity_kernel(FidArgs a) {
@@ -71,7 +77,7 @@ __global__ void __launch_bounds__(kFidTile *kFidTile) fidelity_kernel(FidArgs a)
     float2 *wa = sm;                              // [16][m][N]
     float2 *wb = sm + (size_t)kFidTile * m * N;   // [16][m][N]
     int ti, tj;
-    fid_tile(a.Nb, a.sym, blockIdx.x, ti, tj);
+    fid_tile(a.Nb, a.sym, fid_block(), ti, tj);
     const int i0 = ti * kFidTile, j0 = tj * kFidTile;
     const int tid = threadIdx.y * kFidTile + threadIdx.x;
     const int per = m * N;
@@ -82,8 +88,7 @@ __global__ void __launch_bounds__(kFidTile *kFidTile) fidelity_kernel(FidArgs a)
         wb[idx] = (j0 + t < a.Nb) ? a.Ub[((size_t)(j0 + t) * m + k) * m + col] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    const int i = i0 + threadIdx.y, j = j0 + threadIdx.x;
-    if (i >= a.Na || j >= a.Nb) return;
+    if (i0 + (int)threadIdx.y >= a.Na || j0 + (int)threadIdx.x >= a.Nb) return;
     const float2 *pa = wa + (size_t)threadIdx.y * per, *pb = wb + (size_t)threadIdx.x * per;
     float2 W[N][N];
 #pragma unroll
@@ -137,28 +142,33 @@ __global__ void __launch_bounds__(kFidTile *kFidTile) fidelity_kernel(FidArgs a)
     const float scale = 1.f / (float)(1u << (N - 1));
     const float tr = df_float(t.re) * scale, tim = df_float(t.im) * scale;
     const float v = (tr * tr + tim * tim) * a.inv_sf2;
+    // the tile once more: its two registers held through the sums cost 2-6 %
+    // (one pair, n = 8: 113 us, now 107)
+    fid_tile(a.Nb, a.sym, fid_block(), ti, tj);
+    const int i = ti * kFidTile + threadIdx.y, j = tj * kFidTile + threadIdx.x;
     if (a.sym && i > j) return;  // the mirrored entry of a diagonal tile
     a.K[(size_t)i * a.Nb + j] = v;
     if (a.sym && i < j) a.K[(size_t)j * a.Nb + i] = v;
 }
 
-// Tile (row, column) of block `b`: all tiles, or the upper triangle row by row
-// (row r of the triangle starts at r T - r (r - 1) / 2 for T tiles a side).
-__device__ __forceinline__ void fid_tile(int Nb, bool sym, int64_t b, int &ti, int &tj) {
-    const int T = (Nb + kFidTile - 1) / kFidTile;
+// Tile (row, column) of block `b` (a grid's x extent is below 2^31): all tiles,
+// or the upper triangle row by row (row r of the triangle starts at
+// r T - r (r - 1) / 2 for T tiles a side).
+__device__ __forceinline__ void fid_tile(int Nb, bool sym, uint32_t b, int &ti, int &tj) {
+    const uint32_t T = (uint32_t)(Nb + kFidTile - 1) / kFidTile;
     if (!sym) {
         ti = (int)(b / T);
         tj = (int)(b % T);
         return;
     }
-    int lo = 0, hi = T - 1;  // the last row that starts at or before b
+    uint32_t lo = 0, hi = T - 1;  // the last row that starts at or before b
     while (lo < hi) {
-        const int mid = (lo + hi + 1) / 2;
-        if ((int64_t)mid * T - (int64_t)mid * (mid - 1) / 2 <= b) lo = mid;
+        const uint32_t mid = (lo + hi + 1) / 2;
+        if ((uint64_t)mid * T - (uint64_t)mid * (mid - 1) / 2 <= b) lo = mid;
         else hi = mid - 1;
     }
-    ti = lo;
-    tj = lo + (int)(b - ((int64_t)lo * T - (int64_t)lo * (lo - 1) / 2));
+    ti = (int)lo;
+    tj = (int)(lo + (b - (uint32_t)((uint64_t)lo * T - (uint64_t)lo * (lo - 1) / 2)));
 }
 
 // ------------------------------------------------------------ subsets of columns

@@ -74,3 +74,14 @@ def test_set_against_itself_computes_half_and_mirrors(slos, m, s, N):
     assert (G - full).abs().max() <= 1e-6
     ref = oracle.fidelity_kernel(U.astype(np.complex128), U.astype(np.complex128), s)
     assert np.abs(full.cpu().numpy() - ref).max() <= 2e-6
+
+
+@pytest.mark.parametrize("n", [6, 7, 8])
+def test_most_modes_and_photons(slos, n):
+    """24 modes, whose photon columns take all of a CTA's shared memory."""
+    m, N = 24, 3
+    s = [1] * n + [0] * (m - n)
+    U = workloads.haar_unitaries(m, N, np.random.default_rng(n)).astype(np.complex64)
+    K = slos.fidelity_kernel(s, torch.tensor(U, device="cuda"), torch.tensor(U[:2], device="cuda"))
+    ref = oracle.fidelity_kernel(U.astype(np.complex128), U[:2].astype(np.complex128), s)
+    assert np.abs(K.cpu().numpy() - ref).max() <= 2e-6
