@@ -1574,13 +1574,23 @@ static slos_status_t launch_prefix_fwd(const slos_plan_s *p, const Layout &Ly, c
 //   on chip, 1024-thread CTAs: m=12 n=6 1 17 / 32, 192 30 / 37, 384 46 / 37;
 //                  m=13 n=6 192 37 / 37; m=16 n=5 256 30 / 37, 384 45 / 37
 //   on chip, small: m=10 n=5 1 10.4 / 8.4, 4..256 10.5 / 12.5, 384 17 / 13; m=9 n=4 8.5 / 6.4
-// hence the lines: final states of the whole batch for the layered plans, a
-// little over one instance per SM for the on-chip ones.
+// hence the lines: final states of the whole batch for the layered plans (which
+// give up a few points: m=14 n=7 batch 512, m=20 n=6 threshold 48, m=16 n=4
+// threshold 2048), a little over one instance per SM for the on-chip ones.
+// The largest on-chip plans stop sooner: while every instance has an SM of its
+// own there, the on-chip time does not grow with the batch, and this one's
+// grows with the parents gathered (plan's parents x batch, us, this / on chip:
+// collision-free m=16 n=8, 262,000 x 64 32 / 38, x 150 57 / 39; m=7 n=12,
+// 223,000 x 100 41 / 45, x 150 51 / 46, x 190 63 / 87; m=13 n=6, 111,000 x 150 27 / 36).
 static int narrow_width(const slos_plan_s *p, int batch) {
     if (!p->tab.enabled) return kLanes;
     const int width = slos_narrow_width(batch);
     if (p->fused_ni > 0) {
         if (4 * (int64_t)batch > 5 * (int64_t)p->sm_count) return kLanes;
+        int64_t parents = 0;
+        for (int k = 1; k <= p->n; ++k)
+            parents += p->space == SLOS_SPACE_UNBUNCHED ? k * p->F[k] : p->m * p->F[k - 1];
+        if (batch <= p->sm_count && parents * batch > 25000000) return kLanes;
         if (p->fused_threads == 1024) return width;
         return p->F[p->n] >= 2000 && batch >= 4 ? width : kLanes;
     }

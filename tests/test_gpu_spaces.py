@@ -352,3 +352,19 @@ def test_renormalise_rows_of_any_length(slos, m, n, B):
     dot = (dq * q64).sum(axis=1, keepdims=True)
     inv = np.divide(1.0, Z64, out=np.zeros_like(Z64), where=Z64 > 0)
     assert np.all(np.abs(got - (dq - dot) * inv) <= 4e-7 * (np.abs(dq).max() + np.abs(dot)) * inv)
+
+
+@pytest.mark.parametrize("m,n,space,batches", [(16, 8, 1, (64, 95, 96, 150, 153)), (7, 12, 0, (111, 112, 150, 190)),
+                                               (13, 6, 0, (150, 190, 191))])
+def test_on_chip_plans_over_their_batches(slos, m, n, space, batches):
+    """Inference of plans that fit a CTA on both sides of the batches where
+    the kernel changes: every instance's outputs against the training
+    forward's (the same sums in FP32: a few ulps of a probability)."""
+    s = [1] * n + [0] * (m - n) if n <= m else [n - m + 1] + [1] * (m - 1)
+    plan = slos.Plan(m, s, slos.PNR, space=space)
+    U = torch.tensor(workloads.haar_unitaries(m, max(batches), np.random.default_rng(m)), dtype=torch.complex64,
+                     device="cuda")
+    ref = plan.forward(U, save_for_backward=True)
+    for b in batches:
+        got = plan.forward(U[:b].contiguous())
+        assert (got - ref[:b]).abs().max() <= 1e-6
