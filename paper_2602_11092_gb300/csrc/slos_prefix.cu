@@ -184,11 +184,10 @@ __device__ __forceinline__ void prefix_warp_sum(const float2 (&du)[MM], float *r
 // MM: a bound on m (16 or 24), the size of the per-thread dU accumulators.
 // One barrier per layer: the layer's G and its warps' dU sums are published
 // together, and the sums are added over the warps (in warp order) while the
-// next layer is walked, its sums going to the other half of `red`.
+// next layer is walked, its sums going to the other half of the rows.
 template <int MM>
 __global__ void __launch_bounds__(kPrefixThreads, 2) slos_bwd_prefix_kernel(PrefixArgs a) {
     extern __shared__ float2 pf_sm[];
-    __shared__ float red[2][kPrefixMaxNI][kPrefixThreads / 32][2 * MM];
     const int NI = a.NI, L = a.L, m = a.m;
     const int warp = threadIdx.x >> 5;
     float2 *us = pf_sm;                                  // [NI][L][kPfUsRow]
@@ -196,6 +195,10 @@ __global__ void __launch_bounds__(kPrefixThreads, 2) slos_bwd_prefix_kernel(Pref
     float2 *gbuf[2];                                     // G_k in gbuf[k & 1]: [NI][cap[k & 1]]
     gbuf[0] = as + (size_t)NI * a.asum;
     gbuf[1] = gbuf[0] + (size_t)NI * a.cap[0];
+    // [NI][2][warps of a full CTA][2 MM]: the warps' dU sums (no more of it than
+    // the CTA has instances: it decides whether two CTAs of m = 20 fit an SM)
+    using Rows = float[2][kPrefixThreads / 32][2 * MM];
+    Rows *red = reinterpret_cast<Rows *>(gbuf[1] + (size_t)NI * a.cap[1]);
     const int inst0 = blockIdx.x * NI;
     const int ni = min(NI, a.B - inst0);
     const int grp = inst0 / kLanes, l0 = inst0 % kLanes;
@@ -265,14 +268,14 @@ __global__ void __launch_bounds__(kPrefixThreads, 2) slos_bwd_prefix_kernel(Pref
                     }
                     if (k >= 2) gp[(size_t)i * capp + t] = gacc;
                 }
-                prefix_warp_sum<MM>(du, red[k & 1][i][warp]);
+                prefix_warp_sum<MM>(du, red[i][k & 1][warp]);
             }
         }
         __syncthreads();
         for (int x = threadIdx.x; x < ni * 2 * m; x += blockDim.x) {
             const int i = x / (2 * m), f = x % (2 * m);
             float s = 0.f;
-            for (int w = 0; w < nw; ++w) s += red[k & 1][i][w][f];
+            for (int w = 0; w < nw; ++w) s += red[i][k & 1][w][f];
             reinterpret_cast<float *>(a.dUpart[k] + ((size_t)grp * kLanes + l0 + i) * m)[f] = s;
         }
         aoff -= k >= 2 ? a.F[k - 2] : 0;
@@ -280,15 +283,22 @@ __global__ void __launch_bounds__(kPrefixThreads, 2) slos_bwd_prefix_kernel(Pref
 }
 
 // ------------------------------------------------------------------ launchers
+// Bytes of the warps' dU sums (slos_bwd_prefix_kernel), beside the
+// kPrefixSmemLimit bytes of the layers at most.
+static constexpr size_t prefix_sum_bytes(int NI, int m) {
+    return (size_t)NI * 2 * (kPrefixThreads / 32) * 2 * (m <= 16 ? 16 : kMaxModes) * sizeof(float);
+}
+constexpr size_t kPrefixSumBytes = prefix_sum_bytes(kPrefixMaxNI, kMaxModes);
+
 cudaError_t slos_prefix_init() {
     cudaError_t e = cudaFuncSetAttribute(slos_fwd_prefix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kPrefixSmemLimit);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(slos_bwd_prefix_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kPrefixSmemLimit);
+                             (int)(kPrefixSmemLimit + kPrefixSumBytes));
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(slos_bwd_prefix_kernel<kMaxModes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kPrefixSmemLimit);
+                                (int)(kPrefixSmemLimit + kPrefixSumBytes));
 }
 
 // Threads of a prefix CTA: the full 512 while the grid is too small to fill the
@@ -305,6 +315,24 @@ static size_t prefix_smem_args(const PrefixArgs &a, bool bwd) {
            (size_t)a.NI * ((bwd ? a.asum : 0) + a.cap[0] + a.cap[1]) * sizeof(float2);
 }
 
+// Shared memory a backward CTA asks for, `need` or more: enough that no more
+// CTAs fit an SM than the grid gives it (in waves of equal size), because the
+// SM's other memory is the L1 that holds the child tables and the split is
+// chosen for all that could fit.  At most twice `need`: a split far from the
+// neighbouring launches' costs more than it gives.  Measured, us: m=20 n=5,
+// batch 100 (one CTA an SM) 34 with room for one, 40 with room for two, batch
+// 304 (two) 67 and 61; m=17 n=6, batch 1000 (four) 40 with room for four, 44
+// for nine; m=24 n=5, batch 1000 (four) 59 in two waves of two, 71 with room
+// for three.
+static size_t prefix_request(size_t need, int grid, int sm_count) {
+    constexpr size_t kSm = 228 * 1024, kReserved = 1024;  // per SM; of it per CTA
+    const size_t fit = std::max<size_t>(1, kSm / (need + kReserved));
+    const size_t wanted = (size_t)(grid + sm_count - 1) / std::max(1, sm_count);
+    const size_t waves = (wanted + fit - 1) / fit;
+    const size_t ctas = (wanted + waves - 1) / waves;
+    return std::max(need, std::min({kSm / (ctas + 1), 2 * need, kPrefixSmemLimit}));
+}
+
 cudaError_t slos_launch_prefix_fwd(const PrefixArgs &a, cudaStream_t s) {
     const size_t sm = prefix_smem_args(a, false);
     if (sm > kPrefixSmemLimit || a.NI < 1 || a.lanes % a.NI != 0) return cudaErrorInvalidValue;
@@ -317,10 +345,11 @@ cudaError_t slos_launch_prefix_bwd(const PrefixArgs &a, cudaStream_t s) {
     if (sm > kPrefixSmemLimit || a.NI < 1 || kLanes % a.NI != 0) return cudaErrorInvalidValue;
     const int grid = (a.B + a.NI - 1) / a.NI;
     const int threads = prefix_threads(a, a.F[a.L - 1]);
+    const size_t total = prefix_request(sm + prefix_sum_bytes(a.NI, a.m), grid, a.sm_count);
     if (a.m <= 16)
-        slos_bwd_prefix_kernel<16><<<grid, threads, sm, s>>>(a);
+        slos_bwd_prefix_kernel<16><<<grid, threads, total, s>>>(a);
     else
-        slos_bwd_prefix_kernel<kMaxModes><<<grid, threads, sm, s>>>(a);
+        slos_bwd_prefix_kernel<kMaxModes><<<grid, threads, total, s>>>(a);
     return cudaGetLastError();
 }
 

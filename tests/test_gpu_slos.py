@@ -707,6 +707,42 @@ def test_on_chip_prefix_layers_forward_and_backward(slos, B):
         assert rel <= G_TOL, f"instance {b}: rel err {rel:.2e}"
 
 
+@pytest.mark.parametrize("m,n", [(12, 6), (13, 6), (17, 6), (20, 5)])
+@pytest.mark.parametrize("budget", [0, 1])
+def test_training_on_both_sides_of_the_prefix_depths(slos, m, n, budget):
+    """The on-chip prefix takes fewer layers past two instances per SM
+    (12, 6: five and four; 13, 6: four and three), and its backward one or two
+    CTAs per SM before that; with every layer kept and with as few as the
+    backward allows.  The same instances give the same probabilities and, in
+    sums cut elsewhere (rounding of FP32 sums of the layer's states), dU."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    batches = [2 * sms + 1, 2 * sms, sms + 1, 5]
+    s = workloads.even_mode_input(m, n)
+    rng = np.random.default_rng(m + n)
+    plan = slos.Plan(m, s, mem_budget_bytes=budget)
+    Us = workloads.haar_unitaries(m, 40, rng)
+    U = c64(Us)[torch.arange(batches[0]) % 40]
+    c = torch.tensor(rng.standard_normal((40, plan.n_outputs)), dtype=torch.float32,
+                     device=dev())[torch.arange(batches[0]) % 40]
+    ref = None
+    for b in batches:
+        ws = plan.workspace(b, training=True)
+        Ub = U[:b].contiguous()
+        p = plan.forward(Ub, save_for_backward=True, workspace=ws)
+        dU = plan.backward(Ub, c[:b].contiguous(), ws)
+        plan.sync_status()
+        if ref is None:
+            ref = p, dU
+            if m == 12:
+                outs = oracle.enumerate_fock(m, n)
+                g = _grad_U_ref(up(Ub)[3], s, c[3].double().cpu().numpy(), outs)
+                assert np.linalg.norm(dU[3].cpu().numpy() - g) / np.linalg.norm(g) <= G_TOL
+            continue
+        assert (p - ref[0][:b]).abs().max() <= 1e-6
+        err = torch.linalg.matrix_norm(dU - ref[1][:b]) / torch.linalg.matrix_norm(ref[1][:b])
+        assert err.max() <= 1e-5
+
+
 def test_autotune_picks_a_shape_caches_it_and_keeps_parity(slos, tmp_path):
     m, s, B = 8, [1, 0, 1, 0, 1, 0, 1, 1], 40
     rng = np.random.default_rng(77)
