@@ -1914,14 +1914,18 @@ slos_status_t slos_backward(slos_plan_t p, const void *U, int batch, slos_output
 }
 
 // ------------------------------------------------------------------ single-shape autotuner
-// Key of a single-shape plan's tuned launch shapes: device, shape and batch.
+// Key of a single-shape plan's tuned launch shapes: device, shape, batch and
+// the kernels they were timed with (kTuneKernels grows when those change, so
+// that a file of an older build is timed anew).
+constexpr int kTuneKernels = 2;
 static std::string tune_key(const slos_plan_s *p, int batch) {
     cudaDeviceProp prop;
     std::string dev = cudaGetDeviceProperties(&prop, p->device) == cudaSuccess ? prop.name : "unknown";
     std::ostringstream k;
     k << dev << "|single:m" << p->m << ",n" << p->n << ",s";
     for (int v : p->s) k << v << ".";
-    k << ",det" << (int)p->det << ",space" << p->space << ",stride" << p->stride << ",batch" << batch;
+    k << ",det" << (int)p->det << ",space" << p->space << ",stride" << p->stride << ",batch" << batch << ",kernels"
+      << kTuneKernels;
     return k.str();
 }
 
@@ -1934,7 +1938,17 @@ static bool json_int(const std::string &line, const char *name, int *v) {
     return true;
 }
 
-static bool tune_lookup(const char *path, const std::string &key, int out[4]) {
+// A shape the tuner can have written for this plan and batch: anything else in
+// a file (edited, cut short) would reach the launches.
+static bool tune_valid(const slos_plan_s *p, int batch, const int t[4]) {
+    const int L = t[0], ni = t[1], res = slos_pair_resident_blocks(p->m);
+    if (t[2] < 1 || t[2] > res || t[3] < 1 || t[3] > kSplitBwdMinBlocks) return false;
+    if (L == 0) return ni == 0;
+    return L >= 2 && L <= p->prefix_L && (ni == 1 || ni == 2 || ni == 4) && ni <= batch &&
+           slos_prefix_bwd_smem(ni, L, p->F.data()) <= kPrefixSmemLimit;
+}
+
+static bool tune_lookup(const slos_plan_s *p, int batch, const char *path, const std::string &key, int out[4]) {
     std::ifstream f(path);
     if (!f) return false;
     std::string line;
@@ -1944,7 +1958,8 @@ static bool tune_lookup(const char *path, const std::string &key, int out[4]) {
         if (line.find(kq) == std::string::npos) continue;
         int v[4];
         if (json_int(line, "prefix_layers", &v[0]) && json_int(line, "prefix_ni", &v[1]) &&
-            json_int(line, "fwd_blocks_per_sm", &v[2]) && json_int(line, "bwd_blocks_per_sm", &v[3])) {
+            json_int(line, "fwd_blocks_per_sm", &v[2]) && json_int(line, "bwd_blocks_per_sm", &v[3]) &&
+            tune_valid(p, batch, v)) {
             memcpy(out, v, sizeof(v));
             found = true;  // the last entry for the key wins
         }
@@ -1968,7 +1983,7 @@ slos_status_t slos_autotune(slos_plan_t p, const void *U, int batch, void *out, 
         return fail(SLOS_ERR_INVALID_ARG, "slos_autotune: empty batch or NULL pointer");
     const std::string key = tune_key(p, batch);
     int best_t[4] = {-1, 0, 0, 0};
-    if (cache_path && tune_lookup(cache_path, key, best_t)) {
+    if (cache_path && tune_lookup(p, batch, cache_path, key, best_t)) {
         tune_apply(p, best_t);
         return SLOS_OK;
     }

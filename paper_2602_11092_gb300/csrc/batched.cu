@@ -45,6 +45,7 @@
 #include <chrono>
 #include <cstdio>
 #include <fstream>
+#include <iterator>
 #include <map>
 #include <sstream>
 #include <string>
@@ -530,7 +531,7 @@ struct BatchedPlan {
     std::vector<BShape> shapes;
     std::vector<BLaneGroup> lgs;
     std::string signature;
-    // launch configuration (default_launch, or autotuned)
+    // launch configuration (default_chunk, or autotuned)
     int chunk = 256, threads = 256, blocks_per_sm = 3, minb = 3;
     // device copies (owned)
     BShape *d_shapes = nullptr;
@@ -633,14 +634,15 @@ static slos_status_t build_items(BatchedPlan *b, int chunk) {
 // 128 / 256 / 512 / 1024): 1024 instances of m 8..20 (46,000 states a warp)
 // - / 4.9 / 4.75 / 4.65; 500 of m 10..17 (2,700) - / 0.334 / 0.329 / -; 30 of
 // m 12..16 (270) 0.097 / 0.101 / 0.102 / -; 100 of m 8..14 (40) 0.047 / 0.05 / - / -.
-static void default_launch(BatchedPlan *b, int sm_count) {
+static int default_chunk(const BatchedPlan *b, int sm_count) {
+    const BatchedPlan shape;  // the default blocks and threads
     int64_t states = 0;
     for (const auto &g : b->lgs) {
         const BShape &sh = b->shapes[g.shape];
         for (int k = 1; k <= sh.n; ++k) states += sh.F[k];
     }
-    const int64_t per_warp = states / ((int64_t)sm_count * b->blocks_per_sm * (b->threads / 32));
-    b->chunk = per_warp < 512 ? 128 : (per_warp < 2048 ? 256 : (per_warp < 16384 ? 512 : 1024));
+    const int64_t per_warp = states / ((int64_t)sm_count * shape.blocks_per_sm * (shape.threads / 32));
+    return per_warp < 512 ? 128 : (per_warp < 2048 ? 256 : (per_warp < 16384 ? 512 : 1024));
 }
 
 static slos_status_t batched_launch(slos_plan_s *p, const void *U, float *out, void *ws, size_t ws_bytes,
@@ -703,11 +705,27 @@ static std::string device_name(int dev) {
     return prop.name;
 }
 
+// Launch shapes the tuner times.  kTuneKernels is part of the cache's key and
+// grows when the kernel or its options change, so that a file of an older
+// build is timed anew.
+constexpr int kTuneKernels = 2;
+constexpr int kTuneChunks[] = {128, 256, 512, 1024};
+constexpr int kTuneThreads[] = {128, 256};
+constexpr int kTuneMinBlocks[] = {3, 4};
+
+static int resident_blocks(int minb, int threads) {
+    int nb = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batched_kernel(minb), threads,
+                                                  (size_t)(threads / 32) * kBWarpF2 * sizeof(float2));
+    return nb;
+}
+
 static bool cache_lookup(const std::string &path, const std::string &key, int *chunk, int *threads, int *bps,
                          int *minb) {
     std::ifstream f(path);
     if (!f) return false;
     std::string line;
+    bool found = false;
     while (std::getline(f, line)) {
         // one JSON object per line:
         // {"key": "...", "chunk": C, "threads": T, "blocks_per_sm": B, "min_blocks": R, "ms": X}
@@ -720,9 +738,21 @@ static bool cache_lookup(const std::string &path, const std::string &key, int *c
             *dst = atoi(line.c_str() + pos + nq.size());
             return true;
         };
-        return num("chunk", chunk) && num("threads", threads) && num("blocks_per_sm", bps) && num("min_blocks", minb);
+        auto listed = [](const auto &list, int v) {
+            return std::find(std::begin(list), std::end(list), v) != std::end(list);
+        };
+        int c, t, b, r;
+        if (num("chunk", &c) && num("threads", &t) && num("blocks_per_sm", &b) && num("min_blocks", &r) &&
+            listed(kTuneChunks, c) && listed(kTuneThreads, t) && listed(kTuneMinBlocks, r) && b >= 1 &&
+            b <= resident_blocks(r, t)) {
+            *chunk = c;
+            *threads = t;
+            *bps = b;
+            *minb = r;
+            found = true;  // the last entry for the key wins
+        }
     }
-    return false;
+    return found;
 }
 
 }  // namespace slos
@@ -941,7 +971,7 @@ slos_status_t slos_batched_plan(int count, const int *m, const int *n, const int
     const bool built = cudaStreamSynchronize(0) == cudaSuccess && cudaGetLastError() == cudaSuccess;
     free_scratch();
     if (!built) return cleanup("slos_batched_plan: building the transition tables failed");
-    default_launch(b, p->sm_count);
+    b->chunk = default_chunk(b, p->sm_count);
     slos_status_t st = build_items(b, b->chunk);
     if (st != SLOS_OK) {
         batched_destroy(p);
@@ -987,7 +1017,8 @@ slos_status_t slos_batched_autotune(slos_plan_t p, const void *U_packed, float *
     if (!p || p->kind != 1 || !p->batched) return fail(SLOS_ERR_INVALID_ARG, "slos_batched_autotune: not a batched plan");
     BatchedPlan *b = p->batched;
     cudaStream_t s = (cudaStream_t)stream;
-    const std::string key = device_name(p->device) + "|" + std::to_string(std::hash<std::string>()(b->signature));
+    const std::string key = device_name(p->device) + "|" + std::to_string(std::hash<std::string>()(b->signature)) +
+                            "|kernels" + std::to_string(kTuneKernels);
     int c = 0, t = 0, bp = 0, mb = 0;
     if (cache_path && cache_lookup(cache_path, key, &c, &t, &bp, &mb)) {
         b->chunk = c;
@@ -996,22 +1027,21 @@ slos_status_t slos_batched_autotune(slos_plan_t p, const void *U_packed, float *
         b->minb = mb;
         return build_items(b, c);
     }
-    const int chunks[] = {128, 256, 512, 1024};
-    const int thread_opts[] = {128, 256};
-    const int minb_opts[] = {3, 4};
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
+    // chunks of up to twice the default: larger ones leave warps idle, and on a
+    // small batch only noise would choose them
+    const int most = 2 * default_chunk(b, p->sm_count);
     float best = 1e30f;
     int bc = b->chunk, bt = b->threads, bb = b->blocks_per_sm, bm = b->minb;
-    for (int mbv : minb_opts) {
-        for (int th : thread_opts) {
-            int nb = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batched_kernel(mbv), th,
-                                                          (size_t)(th / 32) * kBWarpF2 * sizeof(float2));
+    for (int mbv : kTuneMinBlocks) {
+        for (int th : kTuneThreads) {
+            const int nb = resident_blocks(mbv, th);
             // a persistent grid must be fully resident: all of it, or one block per SM less
             for (int bps = std::max(1, nb - 1); bps <= nb; ++bps) {
-                for (int ch : chunks) {
+                for (int ch : kTuneChunks) {
+                    if (ch > most) continue;
                     slos_status_t st =
                         batched_launch(p, U_packed, out_packed, workspace, workspace_bytes, s, ch, th, bps, mbv);
                     if (st != SLOS_OK) return st;  // warm-up (also builds the items)

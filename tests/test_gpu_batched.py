@@ -334,3 +334,34 @@ def test_uneven_workspace_on_any_address(slos, off):
     assert torch.equal(ref, got)
     with pytest.raises(slos.SlosError):
         bp.forward(U, got, buf[off:off + 64])
+
+
+@pytest.mark.parametrize("field,value", [("min_blocks", 6), ("chunk", 0), ("chunk", 192), ("threads", 512),
+                                         ("blocks_per_sm", 99), ("key", "older")])
+def test_uneven_tuning_of_another_build_is_timed_anew(slos, tmp_path, field, value):
+    """A cache line whose values this build does not time, or whose key names
+    no kernel generation, is not applied: the tuner runs and appends its own."""
+    rng = np.random.default_rng(3)
+    inst = small_uneven(rng, count=9)
+    bp = make_plan(slos, inst)
+    U = pack([workloads.haar_unitaries(it.m, 1, rng)[0] for it in inst])
+    ws = torch.empty(bp.workspace_bytes, dtype=torch.uint8, device="cuda")
+    out = torch.empty(bp.out_offsets[-1], device="cuda")
+    cache = tmp_path / "autotune.json"
+    bp.autotune(U, out, ws, cache_path=str(cache))
+    entry = json.loads(cache.read_text())
+    ref = out.clone()
+    if field == "key":
+        entry["key"] = entry["key"].rsplit("|", 1)[0]
+    else:
+        entry[field] = value
+    cache.write_text(json.dumps(entry) + "\n")
+    again = make_plan(slos, inst)
+    again.autotune(U, out, ws, cache_path=str(cache))
+    assert len(cache.read_text().splitlines()) == 2
+    again.forward(U, out, ws)
+    again.sync_status()
+    assert torch.equal(out, ref)
+    third = make_plan(slos, inst)
+    third.autotune(U, out, ws, cache_path=str(cache))  # the new line is taken
+    assert len(cache.read_text().splitlines()) == 2

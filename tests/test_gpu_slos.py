@@ -5,6 +5,7 @@ Tolerances (stated by the target): max |dp| <= 1e-5 and total variation
 indexing bit-exact.  The oracle evaluates the complex64-rounded unitary the
 GPU received (upcast to complex128), so the gap is the device arithmetic.
 """
+import json
 import math
 
 import numpy as np
@@ -769,3 +770,27 @@ def test_autotune_picks_a_shape_caches_it_and_keeps_parity(slos, tmp_path):
         check_dist(p[b], oracle.probabilities(Uh[b], s, outs))
         ref = _grad_U_ref(Uh[b], s, c.astype(np.float64), outs)
         assert np.linalg.norm(dU[b] - ref) / np.linalg.norm(ref) <= G_TOL
+
+
+@pytest.mark.parametrize("field,value", [("prefix_layers", 5), ("prefix_layers", 1), ("prefix_ni", 3), ("prefix_ni", 0),
+                                         ("fwd_blocks_per_sm", 0), ("bwd_blocks_per_sm", 99), ("key", "older")])
+def test_tuning_of_another_build_is_timed_anew(slos, tmp_path, field, value):
+    """A cache line this build's tuner cannot have written (m=8, n=5 runs at
+    most layers 1..4 on chip) is not applied: the tuner runs and appends."""
+    m, s, B = 8, [1, 0, 1, 0, 1, 0, 1, 1], 40
+    U = c64(workloads.haar_unitaries(m, B, np.random.default_rng(78)))
+    cache = tmp_path / "tune.json"
+    plan = slos.Plan(m, s)
+    plan.autotune(U, cache_path=str(cache))
+    entry = json.loads(cache.read_text())
+    entry["prefix_layers"], entry["prefix_ni"] = 4, 1
+    if field == "key":
+        entry["key"] = entry["key"].rsplit(",", 1)[0]
+    else:
+        entry[field] = value
+    cache.write_text(json.dumps(entry) + "\n")
+    t = slos.Plan(m, s).autotune(U, cache_path=str(cache))
+    lines = cache.read_text().splitlines()
+    assert len(lines) == 2 and t == {k: json.loads(lines[1])[k] for k in t}
+    assert slos.Plan(m, s).autotune(U, cache_path=str(cache)) == t
+    assert len(cache.read_text().splitlines()) == 2
