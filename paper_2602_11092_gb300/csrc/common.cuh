@@ -95,8 +95,11 @@ __device__ __forceinline__ float2 cfma_conj_a(float2 a, float2 b, float2 c) {
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-// |a|^2 with a fixed rounding, so that every kernel that forms a probability
-// gives the same bits.
+// |a|^2 with a fixed rounding: the kernels of single-shape plans with tables
+// (training forward, lane = state, on chip) sum a state's parents in the same
+// order too, so an instance's outputs are the same bits whichever of them its
+// batch and its need for a backward select.  (Plans without tables and the
+// uneven launcher's pattern sums round in their own order.)
 __device__ __forceinline__ float cabs2(float2 a) { return __fmaf_rn(a.x, a.x, __fmul_rn(a.y, a.y)); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 

@@ -81,8 +81,7 @@ __device__ __forceinline__ void fused_layer(const FusedArgs &a, int k, const flo
                 if (!final_layer) {
                     cur[(size_t)i * cap_cur + c] = acc;
                 } else if (EPI == EPI_PROBS) {
-                    reinterpret_cast<float *>(a.out)[(size_t)(inst0 + i) * a.K + c] =
-                        wc * (acc.x * acc.x + acc.y * acc.y);
+                    reinterpret_cast<float *>(a.out)[(size_t)(inst0 + i) * a.K + c] = wc * cabs2(acc);
                 } else {
                     reinterpret_cast<float2 *>(a.out)[(size_t)(inst0 + i) * a.K + c] = cscale(acc, sqrtf(wc));
                 }
@@ -202,8 +201,7 @@ __device__ __forceinline__ void fused_block(const FusedArgs &a, int k, const flo
     for (int i = 0; i < NI; ++i) {
         if (i < ni) {
             if (EPI == EPI_PROBS)
-                reinterpret_cast<float *>(a.out)[(size_t)(inst0 + i) * a.K + oc] =
-                    wc * (acc[i].x * acc[i].x + acc[i].y * acc[i].y);
+                reinterpret_cast<float *>(a.out)[(size_t)(inst0 + i) * a.K + oc] = wc * cabs2(acc[i]);
             else
                 reinterpret_cast<float2 *>(a.out)[(size_t)(inst0 + i) * a.K + oc] = cscale(acc[i], sqrtf(wc));
         }

@@ -794,3 +794,35 @@ def test_tuning_of_another_build_is_timed_anew(slos, tmp_path, field, value):
     assert len(lines) == 2 and t == {k: json.loads(lines[1])[k] for k in t}
     assert slos.Plan(m, s).autotune(U, cache_path=str(cache)) == t
     assert len(cache.read_text().splitlines()) == 2
+
+
+@pytest.mark.parametrize("m,n,det,space", [(6, 3, 0, 0), (10, 5, 0, 0), (12, 6, 0, 0), (14, 6, 0, 0), (16, 5, 1, 0),
+                                           (8, 6, 1, 0), (16, 6, 0, 1), (5, 10, 0, 0), (16, 7, 0, 0)])
+def test_inference_gives_the_training_forwards_bits(slos, m, n, det, space):
+    """Which kernel computes an instance's outputs depends on its batch and on
+    whether a backward follows; its outputs do not, bit for bit."""
+    s = workloads.even_mode_input(m, n) if 2 * n <= m + 1 else [n - min(n, m) + 1] + [1] * (min(n, m) - 1) + [0] * (m - min(n, m))
+    plan = slos.Plan(m, s, det, space=space)
+    U = c64(workloads.haar_unitaries(m, 33, np.random.default_rng(m * n)))[torch.arange(400) % 33]
+    kinds = [slos.PROBS] if det else [slos.PROBS, slos.AMPS]
+    for kind in kinds:
+        ref = plan.forward(U, kind, save_for_backward=True)
+        for B in (1, 2, 3, 64, 150, 191, 400):
+            if B * plan.n_outputs > 20_000_000:
+                continue
+            Ub = U[:B].contiguous()
+            assert torch.equal(plan.forward(Ub, kind), ref[:B]), B
+            assert torch.equal(plan.forward(Ub, kind, save_for_backward=True), ref[:B]), B
+
+
+@pytest.mark.parametrize("det,measure,B", [(0, "probs", 3), (0, "expectations", 200), (1, "probs", 40), (0, "amps", 1)])
+def test_layer_evaluation_gives_the_training_bits(slos, det, measure, B):
+    from paper_2602_11092_gb300 import functions as F
+    layer = F.QuantumLayer(12, workloads.even_mode_input(12, 6), det, measurement=measure)
+    x = torch.rand(B, 12, device=dev())
+    y = layer(x)
+    assert y.requires_grad
+    with torch.no_grad():
+        assert torch.equal(layer(x), y)
+    layer.theta.requires_grad_(False)
+    assert torch.equal(layer(x), y)
