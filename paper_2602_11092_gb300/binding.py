@@ -127,15 +127,22 @@ def _ptr(t: torch.Tensor | None):
     return None if t is None else t.data_ptr()
 
 
+# torch's internal handle reads, where this torch has them
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream=None):
     """The stream's handle; by default the current device's current stream
-    (read as a handle: building a torch.cuda.Stream object takes 3 us, more
-    than a launch)."""
+    (read as a handle where torch allows it: building a torch.cuda.Stream
+    object takes 3 us, more than a launch)."""
     if stream is not None:
         return stream.cuda_stream
+    if _raw_stream is None or _raw_device is None:
+        return torch.cuda.current_stream().cuda_stream
     if not torch.cuda.is_initialized():
         torch.cuda.init()
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_raw_device())
 
 
 def _need(t: torch.Tensor, dtype, name: str):

@@ -199,3 +199,15 @@ def test_host_table_validation_rejects_corrupted_tables(lib, m, k):
     assert check(slots, badc) == 6
     badc = ctab.copy(); badc[0, 0] = -1                                         # no holes in the Fock lattice
     assert check(slots, badc) == 6
+
+
+@pytest.mark.parametrize("missing", ["_raw_stream", "_raw_device"])
+def test_current_stream_without_torch_internals(monkeypatch, missing):
+    """A torch without its internal handle reads: the public call serves."""
+    from types import SimpleNamespace
+
+    from paper_2602_11092_gb300 import binding
+    monkeypatch.setattr(binding, missing, None)
+    monkeypatch.setattr(binding.torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=1234))
+    assert binding._stream() == 1234
+    assert binding._stream(SimpleNamespace(cuda_stream=7)) == 7
