@@ -191,6 +191,8 @@ slos_status_t slos_workspace_bytes(slos_plan_t plan, int batch, int training, si
  *      threshold (PROBS only) -> float32 [batch][n_outputs] q(b), each one sum
  *      over the pattern's states in a fixed order (outputs reproducible bit
  *      for bit; every output element is written, so out needs no clearing).
+ * Plans with transition tables give an instance the same bits whatever the
+ * batch and with or without save_for_backward.
  * save_for_backward = 1 keeps the activations slos_backward needs inside
  * `workspace` (sized with training = 1); the caller must hand the same
  * workspace, untouched, to slos_backward.  The workspace must start on a
@@ -265,10 +267,12 @@ slos_status_t slos_sample(slos_plan_t plan, const float *probs, int batch, int s
  * |<s|Ua[i]^dag Ub[j]|s>|^2 = |Per(W_ij)|^2 / (prod s_i!)^2, W_ij the n x n
  * block of Ua[i]^dag Ub[j] on the photon columns.  Ua: complex64 [Na][m][m],
  * Ub: complex64 [Nb][m][m] (e.g. from mesh_unitary); K: float32 [Na][Nb].
- * W in FP32; the permanent (Glynn, Gray-code order) in double-float
- * arithmetic on the FP32 pipe (pairs of floats, about 44 bits), no FP64
- * instruction.  1 <= n <= 8
- * photons, m <= 24; otherwise SLOS_ERR_UNSUPPORTED.
+ * W in FP32; the permanent (up to 6 photons Laplace's expansion over two
+ * halves of the rows, beyond that Glynn's formula in Gray-code order) in
+ * double-float arithmetic on the FP32 pipe (pairs of floats, about 44 bits),
+ * no FP64 instruction.  A set against itself (Ub = Ua, Nb = Na) gives an
+ * exactly symmetric K.  1 <= n <= 8 photons, m <= 24; otherwise
+ * SLOS_ERR_UNSUPPORTED.
  * ---------------------------------------------------------------------- */
 slos_status_t slos_fidelity_kernel(int m, const int *input_state, const void *Ua, int Na, const void *Ub, int Nb,
                                    float *K, void *stream);
@@ -308,16 +312,19 @@ slos_status_t slos_encoded_forward(slos_plan_t plan, const void *U, const void *
  * fastest is kept in the plan.  U, out (float32 [batch][n_outputs]), dU and
  * workspace (the training size for `batch`) are the caller's, as for
  * slos_forward / slos_backward, and are overwritten.  cache_path (may be
- * NULL): a JSON-lines file keyed by device name, plan shape and batch; a
- * cached entry is applied without timing, a new result is appended.  Call it
+ * NULL): a JSON-lines file keyed by device name, plan shape, batch and kernel
+ * generation; a cached entry of a shape this build can have chosen is applied
+ * without timing, a new result is appended.  Call it
  * before a forward / backward pair, not between the two.  Synchronises
  * `stream`; not for stream capture. */
 slos_status_t slos_autotune(slos_plan_t plan, const void *U, int batch, void *out, const float *dout_shared, void *dU,
                             void *workspace, size_t workspace_bytes, const char *cache_path, void *stream);
 
-/* The launch shapes a plan uses: prefix_layers = L (0: none), prefix_ni,
- * fwd_blocks_per_sm, bwd_blocks_per_sm (0: the defaults, before tuning).
- * Any pointer may be NULL. */
+/* The launch shapes a plan uses once slos_autotune has run: prefix_layers = L
+ * (0: none), prefix_ni, fwd_blocks_per_sm, bwd_blocks_per_sm.  Before that the
+ * last three are 0 (the defaults) and prefix_layers is the depth for batches of
+ * up to two instances per SM; larger ones run as many of those layers as fit
+ * 48 KB an instance.  Any pointer may be NULL. */
 slos_status_t slos_plan_tuning(slos_plan_t plan, int *prefix_layers, int *prefix_ni, int *fwd_blocks_per_sm,
                                int *bwd_blocks_per_sm);
 
@@ -357,7 +364,8 @@ slos_status_t slos_batched_inject_stall(slos_plan_t plan, int enable);
 
 /* Times the launch configurations of slos_batched_forward on this GPU and
  * keeps the fastest in the plan; results are cached in the JSON file
- * `cache_path` (NULL = no cache), keyed by device name and problem shape. */
+ * `cache_path` (NULL = no cache), keyed by device name, problem shape and
+ * kernel generation. */
 slos_status_t slos_batched_autotune(slos_plan_t plan, const void *U_packed, float *out_packed, void *workspace,
                                     size_t workspace_bytes, const char *cache_path, void *stream);
 

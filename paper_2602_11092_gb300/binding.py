@@ -421,6 +421,8 @@ class Plan:
         return self.tuning()
 
     def tuning(self) -> dict:
+        """slos_plan_tuning (before autotune: the depth for batches of up to
+        two instances per SM, and zeros for the defaults)."""
         v = [_int() for _ in range(4)]
         _check(load().slos_plan_tuning(self._h, *[ctypes.byref(x) for x in v]))
         return {"prefix_layers": v[0].value, "prefix_ni": v[1].value, "fwd_blocks_per_sm": v[2].value,

@@ -162,7 +162,11 @@ class QuantumLayer(torch.nn.Module):
     space: FOCK or UNBUNCHED (collision-free outputs only); renormalise:
     condition the distribution on the space (divide by its total);
     measurement: "probs" (the distribution), "expectations" (per-mode photon
-    numbers, or click probabilities under threshold detection) or "amps"."""
+    numbers, or click probabilities under threshold detection) or "amps".
+
+    Without gradients (torch.no_grad(), or nothing that requires one) the
+    plan's inference kernels run; with transition tables they give the
+    training forward's outputs bit for bit."""
 
     def __init__(self, m: int, input_state, detection: int = B.PNR, output: int = B.PROBS,
                  mem_budget_bytes: int = 0, theta: torch.Tensor | None = None, w: torch.Tensor | None = None,
