@@ -25,7 +25,7 @@
 // the row's largest magnitude to [2^50, 2^51), so that products of small
 // vectors and small outputs stay far above FP32's subnormals; the epilogue
 // undoes both.  The batch runs in chunks of kEncodeChunk rows, so the split
-// copy of X needs a fixed workspace.
+// copy of X needs a fixed workspace.  (Bases of a few states: encode_small_kernel.)
 //
 // One call, 4096 states of 2002 amplitudes: 818 us with TF32 pairs on single
 // CTAs (GEMM 645, splits and their clearing 110, transfer matrix 47), now
@@ -253,6 +253,39 @@ __global__ void __launch_bounds__(kSplitThreads) encode_split_a_kernel(const flo
     if (tid == 0) rowscale[r] = pow2f(tc::kSplitTarget - ex);
 }
 
+// Bases of up to kSmallStates states: the whole product in FP32 on the CUDA
+// cores, thread = one output of one vector, Phi (at most 32 KB) and a CTA's
+// vectors in shared memory.  Bound by launch latency up to a few thousand
+// vectors; what it saves is two launches and the tensor pipeline's start.
+// One call, us, split GEMM / this: 4096 states of 10 17.1 / 6.4, 16 of 56
+// 20.5 / 10.3, 8192 of 56 33.0 / 19.6.
+constexpr int kSmallStates = 64;
+constexpr int kSmallThreads = 256;
+__global__ void __launch_bounds__(kSmallThreads) encode_small_kernel(const float2 *A, const float *g, const float2 *X,
+                                                                     int K, int64_t batch, int amps, void *out) {
+    __shared__ float2 phi[kSmallStates * kSmallStates];  // A[s][t]
+    __shared__ float2 x[kSmallThreads];                  // the rows' vectors over g
+    for (int i = threadIdx.x; i < K * K; i += kSmallThreads) phi[i] = A[i];
+    const int rows = kSmallThreads / K, r = threadIdx.x / K, t = threadIdx.x % K;
+    const float gt = __ldg(g + t);
+    for (int64_t b0 = (int64_t)blockIdx.x * rows; b0 < batch; b0 += (int64_t)gridDim.x * rows) {
+        const bool own = r < rows && b0 + r < batch;
+        const int64_t o = b0 * K + threadIdx.x;
+        __syncthreads();
+        if (own) {
+            const float2 v = X[o];
+            x[threadIdx.x] = make_float2(v.x / gt, v.y / gt);
+        }
+        __syncthreads();
+        if (!own) continue;
+        float2 acc = make_float2(0.f, 0.f);
+        for (int s = 0; s < K; ++s) acc = cfma(x[r * K + s], phi[s * K + t], acc);
+        acc = cscale(acc, gt);
+        if (amps) reinterpret_cast<float2 *>(out)[o] = acc;
+        else reinterpret_cast<float *>(out)[o] = cabs2(acc);
+    }
+}
+
 // BF16 matrix [rows][cols] (row stride ld elements, a multiple of 8), box
 // 64 x box_rows, 128-byte swizzle: the operand layout of tc_gemm.cuh.
 static PFN_cuTensorMapEncodeTiled_v12000 encode_map_fn() {
@@ -355,7 +388,8 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
     unsigned int *colmax = reinterpret_cast<unsigned int *>(ws + L.colmax);
     const float2 *Ud = reinterpret_cast<const float2 *>(U);
     cudaError_t e;
-    if (n == 1 && (e = cudaMemsetAsync(colmax, 0, (size_t)p->K * sizeof(unsigned int), s)) != cudaSuccess)
+    const bool small = p->K <= kSmallStates;
+    if (!small && n == 1 && (e = cudaMemsetAsync(colmax, 0, (size_t)p->K * sizeof(unsigned int), s)) != cudaSuccess)
         return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
     {
         ProfScope ps("slos_transfer", 0.0, s);
@@ -365,7 +399,7 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
             const float2 *prev = k >= 2 ? buf[(n - k + 1) & 1] : nullptr;
             dim3 grid((unsigned)((Fk + kTransferThreads - 1) / kTransferThreads),
                       (unsigned)((Fk + kTransferRows - 1) / kTransferRows));
-            unsigned int *top = k == n ? colmax : nullptr, *clr = k == n - 1 ? colmax : nullptr;
+            unsigned int *top = !small && k == n ? colmax : nullptr, *clr = !small && k == n - 1 ? colmax : nullptr;
             const uint32_t *sl = p->tab.layer[k].slots, *ci = p->tab.layer[k].colinfo;
             switch (p->tab.layer[k].kw) {
                 case 4: transfer_kernel<4><<<grid, kTransferThreads, 0, s>>>(Ud, m, sl, ci, Fk, Fp, prev, cur, k == 1, top, clr, p->K); break;
@@ -378,6 +412,15 @@ slos_status_t slos_encoded_forward(slos_plan_t p, const void *U, const void *X, 
     }
     if (batch == 0) return SLOS_OK;
     const int64_t K = p->K, K2 = encode_k2(p);
+    if (small) {
+        const int64_t rows = kSmallThreads / K, ctas = (batch + rows - 1) / rows;
+        ProfScope ps("slos_encode_gemm", 8.0 * batch * (double)K * K, s);  // flops
+        encode_small_kernel<<<(unsigned)std::min<int64_t>(ctas, (int64_t)p->sm_count * 4), kSmallThreads, 0, s>>>(
+            buf[0], p->tab.gfact, reinterpret_cast<const float2 *>(X), (int)K, batch, output == SLOS_OUT_AMPS, out);
+        if ((e = cudaGetLastError()) != cudaSuccess)
+            return fail(SLOS_ERR_CUDA, std::string("slos_encoded_forward: ") + cudaGetErrorString(e));
+        return SLOS_OK;
+    }
     __nv_bfloat16 *bsplit = reinterpret_cast<__nv_bfloat16 *>(ws + L.bsplit);
     __nv_bfloat16 *asplit = reinterpret_cast<__nv_bfloat16 *>(ws + L.asplit);
     float *colscale = reinterpret_cast<float *>(ws + L.colscale), *rowscale = reinterpret_cast<float *>(ws + L.rowscale);

@@ -195,3 +195,25 @@ def test_encoded_components_of_very_different_size(slos, u, m, n, B):
     got = plan.encoded_forward(torch.tensor(U, device="cuda"), torch.tensor(X, device="cuda"), slos.AMPS).cpu().numpy()
     ref = X.astype(np.complex128) @ transfer_by_recursion(U.astype(np.complex128), m, n).T
     assert np.all(np.abs(got - ref) <= 4e-6 * np.abs(ref) + 1e-37)
+
+
+@pytest.mark.parametrize("m,n,B", [(2, 1, 1), (3, 1, 130), (4, 2, 5000), (2, 11, 20), (4, 4, 77), (10, 2, 12), (6, 3, 3001),
+                                   (16, 1, 17), (3, 9, 9), (11, 2, 40), (22, 1, 700)])
+@pytest.mark.parametrize("kind", ["amps", "probs"])
+def test_encoded_small_bases(slos, m, n, B, kind):
+    """Bases of 2 to 66 states (both sides of the FP32 product's 64): vectors
+    that do not fill the last CTA, more of them than the grid takes at once.
+    FP32 recursion, products and sums of at most 66 terms."""
+    rng = np.random.default_rng(31 * m + B)
+    plan = slos.Plan(m, [n] + [0] * (m - 1))
+    U = workloads.haar_unitaries(m, 1, rng)[0].astype(np.complex64)
+    X = rand_states(rng, B, plan.n_outputs).astype(np.complex64)
+    out = slos.AMPS if kind == "amps" else slos.PROBS
+    got = plan.encoded_forward(torch.tensor(U, device="cuda"), torch.tensor(X, device="cuda"), out)
+    assert torch.equal(got, plan.encoded_forward(torch.tensor(U, device="cuda"), torch.tensor(X, device="cuda"), out))
+    got = got.cpu().numpy()
+    ref = X.astype(np.complex128) @ transfer_by_recursion(U.astype(np.complex128), m, n).T
+    if kind == "amps":
+        assert np.abs(got - ref).max() <= 4e-6
+    else:
+        assert np.abs(got - np.abs(ref) ** 2).max() <= 8e-6
