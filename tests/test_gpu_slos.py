@@ -826,3 +826,31 @@ def test_layer_evaluation_gives_the_training_bits(slos, det, measure, B):
         assert torch.equal(layer(x), y)
     layer.theta.requires_grad_(False)
     assert torch.equal(layer(x), y)
+
+
+@pytest.mark.parametrize("m,n,kind,B", [(10, 5, "probs", 520), (10, 5, "amps", 545), (16, 4, "threshold", 300),
+                                        (12, 6, "probs", 100)])
+def test_output_gradient_rows_of_few_and_many_values(slos, m, n, kind, B):
+    """Per-instance output gradients on both sides of the size where their
+    transposition goes through shared memory (32,768 states x groups; ragged
+    groups and tiles): the same instances' dU, sums of the layers' states in
+    FP32 cut elsewhere."""
+    det = slos.THRESHOLD if kind == "threshold" else slos.PNR
+    out = slos.AMPS if kind == "amps" else slos.PROBS
+    plan = slos.Plan(m, workloads.even_mode_input(m, n), det)
+    rng = np.random.default_rng(m * B)
+    U = c64(workloads.haar_unitaries(m, 37, rng))[torch.arange(B) % 37]
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    d = torch.randn(B, plan.n_outputs, dtype=torch.complex64 if kind == "amps" else torch.float32, device=dev(),
+                    generator=gen)
+    few = 33
+    dim = workloads.fock_dim(m, n)
+    assert dim * ((B + 31) // 32) > 32768 >= dim * 2
+    grads = []
+    for b in (B, few):
+        ws = plan.workspace(b, training=True)
+        plan.forward(U[:b].contiguous(), out, save_for_backward=True, workspace=ws)
+        grads.append(plan.backward(U[:b].contiguous(), d[:b].contiguous(), ws, out))
+        plan.sync_status()
+    err = torch.linalg.matrix_norm(grads[0][:few] - grads[1]) / torch.linalg.matrix_norm(grads[1])
+    assert err.max() <= 1e-5
